@@ -220,7 +220,9 @@ typedef struct start_stats {
                                    round (own state), 2 s per slot that advanced
                                    (first successor read, write), s per further
                                    successor read, s per slot copied once when its
-                                   chain closed; s = 8 (16 in the counting form) */
+                                   chain closed; s = 8 (16 in the counting form);
+                                   plus the chain states the Gamma sum read of the
+                                   chains that the last round left open */
     long long first_hop_scanned;  /* memoised march, every 64th target: candidates
                                      the first hops of its pairs scanned */
     long long first_hop_full;     /* the same targets: neighbours x pairs (what a

@@ -1187,7 +1187,7 @@ int start_get_stats(start_ctx *c, start_stats *out)
     out->links = (long long)(c->p.march_mode == 1 ? v[C_SLOTS] : 0);
     out->chunks = c->chunks;
     out->jump_rounds = c->jump_rounds;
-    out->jump_bytes = (long long)c->jump_bytes;
+    out->jump_bytes = (long long)(c->jump_bytes + 8ull * v[C_JUMP_TAIL]);
     out->first_hop_scanned = (long long)v[C_ROW_CAND];
     out->first_hop_full = (long long)v[C_ROW_NB];
     return START_OK;

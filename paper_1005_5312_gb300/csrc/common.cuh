@@ -218,12 +218,12 @@ enum Counter {
     C_SLOTS,      // memoised chain links (virtual source, particle)
     C_MEMO_OVF,   // memo slot capacity exceeded (the host retries larger)
     C_MISS,       // first-level links not found in their upstream row
-    C_JUMP_ADV,   // pointer jumping: slot updates that read a successor
-    C_JUMP_COPY,  // pointer jumping: closed chains copied to the other buffer
+    C_JUMP_MOVED, // pointer jumping: states read and written beyond the slots' own
+    C_JUMP_LEFT,  // pointer jumping: slots whose chains the last round left open
     C_TAIL_CAP,   // memo tail kernel: a chain exceeded the iteration cap
     C_HARD,       // first hops listed for the FP64 kernel
     C_NB_OVER,    // targets with more neighbours than the counting walk keeps
-    C_JUMP_EXTRA, // pointer jumping: successor reads beyond the first in a round
+    C_JUMP_TAIL,  // chain states the Gamma sum read beyond the pairs' own
     C_WALK_OVER,  // one-walk lists: targets whose row exceeds the scratch row
     C_LEVEL,      // memoised march: device frontier {fbase, nf, total} (3 words)
     C_WALK_FB_GROUP = C_LEVEL + 3,   // opening tests re-decided by the walks of a group

@@ -25,7 +25,9 @@
 //      (each round reads three successors, so log4 of the longest chain
 //      rounds; double-buffered, so the sum order depends only on the chain):
 //      FP32 sums over the march's 8-byte (next, d_tau) states, or compensated
-//      double-float sums with link counts in the 16-byte counting form;
+//      double-float sums with link counts in the 16-byte counting form.  The
+//      8-byte form stops while chains are still open (kJumpOpen) and the Gamma
+//      sum follows them block by block, in the order the rounds would add;
 //   4. each pair contributes L e^-tau / (4 pi r^2).
 // Count-1 source cells and their single member are the same source and
 // share one chain forest.
@@ -926,6 +928,16 @@ constexpr u32 kDone = 0xfffffffeu;     // 8-byte form: next of a resolved, copie
 constexpr int kJumpR = 6;    // counting form: slots per thread (independent loads in flight)
 constexpr int kJumpG = 3;    // successor reads per slot and round
 constexpr int kJumpR8 = 12;  // 8-byte form: slots per thread
+// Rounds of the 8-byte form: another one runs while more than this share of
+// the slots is open.  The Gamma sum follows the open chains block by block; of
+// chain lengths spread evenly, a share p left open means 1 / (2 (1 - p))
+// blocks to follow per pair, and a round costs about as much as 16 of them
+// (GB300, jumping + Gamma: 2.6 against 2.9 ms with a second round on 64^3 x
+// 1024 sources, p = 0.91; 9.4 against 10.2 ms with three rounds on 1.7 M x 500
+// sources, p = 0.96; 7.2 against 5.4 ms with three on 128^3 x 64 sources,
+// p = 0.98; 147 against 165 ms at half open on the 128^3 diffuse step).
+constexpr double kJumpOpen = 0.97;
+constexpr int kGammaU = 2;   // pairs per lane in flight in the rows of a group
 
 // The march's states widened for the counting form: one link, no
 // compensation term.
@@ -938,12 +950,13 @@ __global__ void k_memo_widen(long long n, const uint2 *__restrict__ st, uint4 *_
     }
 }
 
-// One round of the 8-byte form.  part[3 (8 b + w) ..] accumulate warp w of
-// block b's advancing updates, extra successor reads and copies over the
-// rounds (plain stores: stream-ordered launches of the same grid).
+// One round of the 8-byte form.  part[2 (8 b + w) ..] of warp w of block b:
+// the states it read and wrote beyond every slot's own (accumulated over the
+// rounds: plain stores, stream-ordered launches of the same grid), and its
+// slots whose chains are still open after this round.
 template <int G, int R>
 __global__ void __launch_bounds__(256) k_memo_jump8(long long n, const uint2 *__restrict__ st,
-                                                    uint2 *__restrict__ st2, unsigned *active,
+                                                    uint2 *__restrict__ st2,
                                                     unsigned long long *ctr,
                                                     unsigned long long *part)
 {
@@ -961,7 +974,7 @@ __global__ void __launch_bounds__(256) k_memo_jump8(long long n, const uint2 *__
         }
         if (me[r].x < n32) go |= 1u << r;
     }
-    unsigned adv = __popc(go), extra = 0, cpy = 0;
+    unsigned moved = 2 * __popc(go), left = 0;
 #pragma unroll
     for (int g = 0; g < G; ++g) {
         uint2 nx[R];
@@ -971,12 +984,11 @@ __global__ void __launch_bounds__(256) k_memo_jump8(long long n, const uint2 *__
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             if (me[r].x >= n32) continue;
-            if (g > 0) ++extra;
+            if (g > 0) ++moved;
             me[r] = make_uint2(nx[r].x,
                                __float_as_uint(__uint_as_float(me[r].y) + __uint_as_float(nx[r].y)));
         }
     }
-    bool act = false;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const long long s = s0 + 256 * r;
@@ -984,35 +996,28 @@ __global__ void __launch_bounds__(256) k_memo_jump8(long long n, const uint2 *__
         if ((go >> r) & 1u) {
             if (me[r].x >= n32) me[r].x = kNone;
             st2[s] = me[r];
-            act |= me[r].x != kNone;
+            left += me[r].x != kNone;
         } else if (me[r].x == kNone) {
             me[r].x = kDone;
             st2[s] = me[r];
-            ++cpy;
+            ++moved;
         }
     }
     for (int o = 16; o; o >>= 1) {
-        adv += __shfl_xor_sync(0xffffffffu, adv, o);
-        extra += __shfl_xor_sync(0xffffffffu, extra, o);
-        cpy += __shfl_xor_sync(0xffffffffu, cpy, o);
+        moved += __shfl_xor_sync(0xffffffffu, moved, o);
+        left += __shfl_xor_sync(0xffffffffu, left, o);
     }
-    const int lane = threadIdx.x & 31;
-    if (__any_sync(0xffffffffu, act) && lane == 0) *active = 1u;
-    if (lane == 0) {
-        unsigned long long *q = part + 3 * ((long long)blockIdx.x * 8 + (threadIdx.x >> 5));
-        q[0] += adv;
-        q[1] += extra;
-        q[2] += cpy;
+    if ((threadIdx.x & 31) == 0) {
+        unsigned long long *q = part + 2 * ((long long)blockIdx.x * 8 + (threadIdx.x >> 5));
+        q[0] += moved;
+        q[1] = left;
     }
 }
 
-// part[3 b .. 3 b + 2] accumulate block b's advancing updates, extra
-// successor reads and copies over the rounds (plain stores: a block index is
-// unique within a launch and the rounds are stream-ordered), summed once
-// after the last round.
+// One round of the counting form; part[2 b ..] of block b as above.
 template <int G>
 __global__ void __launch_bounds__(256, 2) k_memo_jump(long long n, const uint4 *__restrict__ st,
-                                                    uint4 *__restrict__ st2, unsigned *active,
+                                                    uint4 *__restrict__ st2,
                                                     unsigned long long *ctr,
                                                     unsigned long long *part)
 {
@@ -1029,7 +1034,7 @@ __global__ void __launch_bounds__(256, 2) k_memo_jump(long long n, const uint4 *
         }
         if (me[r].x != kNone) go |= 1u << r;
     }
-    unsigned adv = __popc(go), extra = 0, cpy = 0;
+    unsigned moved = 2 * __popc(go), left = 0;
     // successors are read only below n (kNone is above it); an index out of
     // range ends the chain here and is counted when its own slot is loaded.
     // A slot that does not advance has next = kNone throughout.
@@ -1043,14 +1048,13 @@ __global__ void __launch_bounds__(256, 2) k_memo_jump(long long n, const uint4 *
 #pragma unroll
         for (int r = 0; r < kJumpR; ++r) {
             if (me[r].x >= n32) continue;
-            if (g > 0) ++extra;
+            if (g > 0) ++moved;
             float2 t = cadd(make_float2(__uint_as_float(me[r].z), __uint_as_float(me[r].w)),
                             make_float2(__uint_as_float(nx[r].z), __uint_as_float(nx[r].w)));
             me[r] = make_uint4(nx[r].x, (me[r].y & ~kStable) + (nx[r].y & ~kStable),
                                __float_as_uint(t.x), __float_as_uint(t.y));
         }
     }
-    bool act = false;
 #pragma unroll
     for (int r = 0; r < kJumpR; ++r) {
         long long s = s0 + 256 * r;
@@ -1058,63 +1062,114 @@ __global__ void __launch_bounds__(256, 2) k_memo_jump(long long n, const uint4 *
         if ((go >> r) & 1u) {
             if (me[r].x >= n32) me[r].x = kNone;
             st2[s] = me[r];
-            act |= me[r].x != kNone;
+            left += me[r].x != kNone;
         } else if (!(me[r].y & kStable)) {
             me[r].y |= kStable;
             st2[s] = me[r];
-            ++cpy;
+            ++moved;
         }
     }
     for (int o = 16; o; o >>= 1) {
-        adv += __shfl_xor_sync(0xffffffffu, adv, o);
-        extra += __shfl_xor_sync(0xffffffffu, extra, o);
-        cpy += __shfl_xor_sync(0xffffffffu, cpy, o);
+        moved += __shfl_xor_sync(0xffffffffu, moved, o);
+        left += __shfl_xor_sync(0xffffffffu, left, o);
     }
-    __shared__ unsigned wadv[8], wext[8], wcpy[8];
+    __shared__ unsigned wmoved[8], wleft[8];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (lane == 0) {
-        wadv[wid] = adv;
-        wext[wid] = extra;
-        wcpy[wid] = cpy;
+        wmoved[wid] = moved;
+        wleft[wid] = left;
     }
-    if (__any_sync(0xffffffffu, act) && lane == 0) *active = 1u;
     __syncthreads();
     if (threadIdx.x == 0) {
-        unsigned long long ba = 0, be = 0, bc = 0;
+        unsigned long long bm = 0, bl = 0;
         for (int k = 0; k < 8; ++k) {
-            ba += wadv[k];
-            be += wext[k];
-            bc += wcpy[k];
+            bm += wmoved[k];
+            bl += wleft[k];
         }
-        part[3 * blockIdx.x] += ba;
-        part[3 * blockIdx.x + 1] += be;
-        part[3 * blockIdx.x + 2] += bc;
+        part[2 * (long long)blockIdx.x] += bm;
+        part[2 * (long long)blockIdx.x + 1] = bl;
     }
 }
 
-// Sums the per-block pointer-jumping counts into their counters.
-// (grid-strided over the entries; each block adds its sums to the counters,
-// which the caller cleared)
-__global__ void k_sum_jump_counts(const unsigned long long *part, long long nblocks,
-                                  unsigned long long *ctr)
+// Sums the states moved so far and the open slots of the last round into
+// out[0] and out[1], which the caller cleared (grid-strided over the parts).
+__global__ void k_sum_jump_counts(const unsigned long long *part, long long nparts,
+                                  unsigned long long *out)
 {
-    unsigned long long v[3] = {0, 0, 0};
-    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < nblocks;
+    unsigned long long v[2] = {0, 0};
+    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < nparts;
          k += (long long)gridDim.x * blockDim.x)
-        for (int q = 0; q < 3; ++q) v[q] += part[3 * k + q];
-    __shared__ unsigned long long sv[3][32];
-    for (int q = 0; q < 3; ++q) {
+        for (int q = 0; q < 2; ++q) v[q] += part[2 * k + q];
+    __shared__ unsigned long long sv[2][32];
+    for (int q = 0; q < 2; ++q) {
         for (int o = 16; o; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
         if ((threadIdx.x & 31) == 0) sv[q][threadIdx.x >> 5] = v[q];
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long t[3] = {0, 0, 0};
-        for (unsigned k = 0; k < blockDim.x / 32; ++k)
-            for (int q = 0; q < 3; ++q) t[q] += sv[q][k];
-        if (t[0]) atomicAdd(&ctr[C_JUMP_ADV], t[0]);
-        if (t[1]) atomicAdd(&ctr[C_JUMP_EXTRA], t[1]);
-        if (t[2]) atomicAdd(&ctr[C_JUMP_COPY], t[2]);
+    if (threadIdx.x < 2) {
+        unsigned long long t = 0;
+        for (unsigned k = 0; k < blockDim.x / 32; ++k) t += sv[threadIdx.x][k];
+        if (t) atomicAdd(&out[threadIdx.x], t);
+    }
+}
+
+// The chain sums of U slots whose states st cover a block of links each (all
+// blocks of one launch the same power of four, the last of a chain shorter):
+// the remaining blocks are read one after the other and added as further
+// rounds of three successor reads would add them -- four blocks left to right
+// make one of the next size -- so the sum is bit for bit the one the rounds
+// give, however many of them ran.  s[u][k] holds the finished blocks of size
+// 4^k of the block of size 4^(k+1) being filled.
+template <int U>
+__device__ __forceinline__ void chain_tails(const uint2 *__restrict__ all, uint2 (&st)[U], u32 n32,
+                                            float (&tau)[U], unsigned &reads)
+{
+    constexpr int K = 6;   // blocks of up to 4^5, then a running sum
+    float s[U][K];
+    bool open = false;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+#pragma unroll
+        for (int k = 1; k < K; ++k) s[u][k] = 0.f;
+        s[u][0] = __uint_as_float(st[u].y);
+        open |= st[u].x < n32;
+    }
+    for (u32 m = 1; open; ++m) {
+        uint2 nx[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            nx[u] = st[u].x < n32 ? all[st[u].x] : make_uint2(kDone, 0u);
+        if ((m & 3u) == 0u) {
+            bool full = true;
+#pragma unroll
+            for (int k = 0; k + 1 < K; ++k) {
+                full = full && ((m >> (2 * k)) & 3u) == 0u;
+                if (full) {
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        if (st[u].x >= n32) continue;
+                        s[u][k + 1] += s[u][k];
+                        s[u][k] = 0.f;
+                    }
+                }
+            }
+        }
+        open = false;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (st[u].x >= n32) continue;
+            ++reads;
+            s[u][0] += __uint_as_float(nx[u].y);
+            st[u].x = nx[u].x;
+            open |= st[u].x < n32;
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        float v = s[u][0];
+#pragma unroll
+        for (int k = 1; k < K; ++k) v = s[u][k] + v;
+        tau[u] = v;
     }
 }
 
@@ -1167,6 +1222,7 @@ __global__ void __launch_bounds__(256) k_memo_gamma(MemoArgs a, const u64 *off, 
     long long i = t0 + ((long long)blockIdx.x * blockDim.x + threadIdx.x) / LANES;
     unsigned long long hops = 0, ovf = 0, rays = 0;
     u32 maxh = 0;
+    unsigned reads = 0;   // chain states read beyond the pairs' own
     if (i < t1) {
         u64 e0 = off[i] - base, e1 = off[i + 1] - base;
         float4 pt = a.m.pq[i];
@@ -1179,53 +1235,75 @@ __global__ void __launch_bounds__(256) k_memo_gamma(MemoArgs a, const u64 *off, 
             hsum = q.z;
             hcmp = q.w;
         }
-        for (u64 e = e0; e < e1; e += LANES) {   // uniform within the lane group
-            u64 p = e + gl;
-            float v = 0.f, hv = 0.f;
-            if (p < e1) {
-                float tau;
-                u32 l = 0;   // links of the chain (counting form)
+        // pairs per lane in flight: two in the short rows of a group (82 against
+        // 97 ms on the 128^3 diffuse step), one where a warp has the whole row
+        // (1.63 against 1.83 ms on 64^3 x 1024 sources)
+        constexpr int U = WIDE || LANES == 32 ? 1 : kGammaU;
+        for (u64 e = e0; e < e1; e += LANES * U) {   // uniform within the lane group
+            float v[U], hv[U], tau[U];
+            u32 links[U];   // of the chain (counting form)
+            uint2 st[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const u64 p = e + u * LANES + gl;
+                tau[u] = 0.f;
+                links[u] = 0;
+                st[u] = make_uint2(kDone, 0u);
+                if (p >= e1) continue;
                 if (WIDE) {
-                    const uint4 st = a.wstate[p];
-                    tau = __uint_as_float(st.z) + __uint_as_float(st.w);
-                    l = st.y & ~kStable;
+                    const uint4 w = a.wstate[p];
+                    tau[u] = __uint_as_float(w.z) + __uint_as_float(w.w);
+                    links[u] = w.y & ~kStable;
                 } else {
-                    tau = __uint_as_float(a.state[p].y);
+                    st[u] = a.state[p];
                 }
-                u32 vid = a.svid[p];
-                float4 src = vsource(a, vid);
+            }
+            if (!WIDE) chain_tails<U>(a.state, st, a.cap, tau, reads);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const u64 p = e + u * LANES + gl;
+                v[u] = hv[u] = 0.f;
+                if (p >= e1) continue;
+                const u32 vid = a.svid[p];
+                const float4 src = vsource(a, vid);
                 float rx = pt.x - src.x, ry = pt.y - src.y, rz = pt.z - src.z;
                 float r2 = fmaxf(rx * rx + ry * ry + rz * rz, rf2);
                 float dil = src.w / (12.566370614359172f * r2);
                 if (MODE == 1) {
-                    float xs = tau * 1e-14f;
-                    v = dil * (xs <= 1.f ? 1.f : powf(xs, -0.75f));
+                    float xs = tau[u] * 1e-14f;
+                    v[u] = dil * (xs <= 1.f ? 1.f : powf(xs, -0.75f));
                 } else if (MODE == 2 && (vid < x.point_end ? x.point_bb : x.emit_band)) {
                     const float *tb = x.tab + (vid < x.point_end ? 0 : 2 * kSpecN);
-                    float sidx = log1pf(tau * x.inv_tau0) * x.inv_ds;
-                    v = dil * spec_lookup(tb, sidx);
-                    hv = dil * spec_lookup(tb + kSpecN, sidx);
+                    float sidx = log1pf(tau[u] * x.inv_tau0) * x.inv_ds;
+                    v[u] = dil * spec_lookup(tb, sidx);
+                    hv[u] = dil * spec_lookup(tb + kSpecN, sidx);
                 } else {
-                    v = dil * expf(-tau);
+                    v[u] = dil * expf(-tau[u]);
                 }
                 if (WIDE) {
-                    hops += l;
-                    maxh = max(maxh, l);
-                    if ((long long)l > a.m.hop_cap) ovf += 1;
+                    hops += links[u];
+                    maxh = max(maxh, links[u]);
+                    if ((long long)links[u] > a.m.hop_cap) ovf += 1;
                 }
                 rays += 1;
             }
-            for (int o = LANES / 2; o; o >>= 1) v += __shfl_xor_sync(gmask, v, o);
-            float yk = v - cmp;
-            float tk = sum + yk;
-            cmp = (tk - sum) - yk;
-            sum = tk;
-            if (MODE == 2) {
-                for (int o = LANES / 2; o; o >>= 1) hv += __shfl_xor_sync(gmask, hv, o);
-                float hy = hv - hcmp;
-                float ht = hsum + hy;
-                hcmp = (ht - hsum) - hy;
-                hsum = ht;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (e + u * LANES >= e1) continue;   // uniform within the lane group
+                for (int o = LANES / 2; o; o >>= 1)
+                    v[u] += __shfl_xor_sync(gmask, v[u], o);
+                float yk = v[u] - cmp;
+                float tk = sum + yk;
+                cmp = (tk - sum) - yk;
+                sum = tk;
+                if (MODE == 2) {
+                    for (int o = LANES / 2; o; o >>= 1)
+                        hv[u] += __shfl_xor_sync(gmask, hv[u], o);
+                    float hy = hv[u] - hcmp;
+                    float ht = hsum + hy;
+                    hcmp = (ht - hsum) - hy;
+                    hsum = ht;
+                }
             }
         }
         if (gl == 0 && !last) {
@@ -1238,6 +1316,7 @@ __global__ void __launch_bounds__(256) k_memo_gamma(MemoArgs a, const u64 *off, 
         }
     }
     block_add(&a.m.counters[C_RAYS], rays);
+    if (!WIDE) block_add(&a.m.counters[C_JUMP_TAIL], reads);
     if (WIDE) {
         block_add(&a.m.counters[C_HOPS], hops);
         block_add(&a.m.counters[C_CHAIN_OVF], ovf);
@@ -1547,51 +1626,53 @@ static int memo_attempt(start_ctx *c, const MarchArgs &m, float theta, size_t ca
     }
     c->memo_evals += (unsigned long long)nslots;
     c->memo_links += (unsigned long long)nslots;
-    // pointer jumping; its flag lives in the context's small scratch (allocated
-    // here too: a batch context never runs the builds that allocate it)
+    // pointer jumping
     const bool wide = memo_counts_links(c);
     if (wide && (ensure(c->m_w[0], cap * 16) || ensure(c->m_w[1], cap * 16)))
         return set_err(c, START_ENOMEM, "out of device memory (memoised march)");
     int b = 0;
-    if (ensure(c->flags, 64 + 2 * (kLevels + 1) * sizeof(unsigned long long)))
-        return set_err(c, START_ENOMEM, "out of device memory (memoised march)");
-    unsigned *active = c->flags.as<unsigned>() + 12;
     const long long jblocks = (long long)grid_for(nslots, 256 * (wide ? kJumpR : kJumpR8));
     const long long nparts = wide ? jblocks : jblocks * 8;   // per block / per warp
-    if (ensure(c->m_part, (size_t)nparts * 24))
+    if (ensure(c->m_part, (size_t)nparts * 16))
         return set_err(c, START_ENOMEM, "out of device memory (memoised march)");
-    ST_CUDA(c, cudaMemsetAsync(c->m_part.p, 0, (size_t)nparts * 24, s));
+    ST_CUDA(c, cudaMemsetAsync(c->m_part.p, 0, (size_t)nparts * 16, s));
     if (wide) {
         k_memo_widen<<<grid_for(nslots, 256), 256, 0, s>>>(nslots, c->m_st[0].as<uint2>(),
                                                            c->m_w[0].as<uint4>());
         ++c->launches;
     }
+    static_assert(C_JUMP_LEFT == C_JUMP_MOVED + 1, "adjacent counters");
+    // the counting form runs until every chain is closed; the 8-byte form
+    // until few slots are open, whose chains the Gamma sum follows itself
+    const unsigned long long few = wide ? 0ull : (unsigned long long)(kJumpOpen * (double)nslots);
     long long rounds = 0;
+    unsigned long long jc[2] = {0, 0};
     for (int round = 0; round < 40; ++round) {
-        ST_CUDA(c, cudaMemsetAsync(active, 0, sizeof(unsigned), s));
+        ST_CUDA(c, cudaMemsetAsync(ctr + C_JUMP_MOVED, 0, sizeof(jc), s));
         if (timing) cudaEventRecord(c->hev[0], s);
         if (wide)
             k_memo_jump<kJumpG><<<(unsigned)jblocks, 256, 0, s>>>(
-                nslots, c->m_w[b].as<uint4>(), c->m_w[b ^ 1].as<uint4>(), active, ctr,
+                nslots, c->m_w[b].as<uint4>(), c->m_w[b ^ 1].as<uint4>(), ctr,
                 c->m_part.as<unsigned long long>());
         else
             k_memo_jump8<kJumpG, kJumpR8><<<(unsigned)jblocks, 256, 0, s>>>(
-                nslots, c->m_st[b].as<uint2>(), c->m_st[b ^ 1].as<uint2>(), active, ctr,
+                nslots, c->m_st[b].as<uint2>(), c->m_st[b ^ 1].as<uint2>(), ctr,
                 c->m_part.as<unsigned long long>());
         if (timing) cudaEventRecord(c->hev[1], s);
-        ++c->launches;
+        k_sum_jump_counts<<<grid_for(nparts, 1024, 4 * (long long)nsm), 1024, 0, s>>>(
+            c->m_part.as<unsigned long long>(), nparts, ctr + C_JUMP_MOVED);
+        c->launches += 2;
         ++rounds;
         ST_CUDA(c, cudaGetLastError());
         b ^= 1;
-        unsigned act = 0;
-        ST_CUDA(c, cudaMemcpyAsync(&act, active, sizeof(act), cudaMemcpyDeviceToHost, s));
+        ST_CUDA(c, cudaMemcpyAsync(jc, ctr + C_JUMP_MOVED, sizeof(jc), cudaMemcpyDeviceToHost, s));
         ST_CUDA(c, cudaStreamSynchronize(s));
         if (timing) {
             float ms = 0.f;
             if (cudaEventElapsedTime(&ms, c->hev[0], c->hev[1]) == cudaSuccess) jump_ms += ms;
             else cudaGetLastError();
         }
-        if (!act) break;
+        if (jc[1] <= few) break;
     }
     if (timing && pending) {   // the tail's events (the rounds above waited on them)
         float ms = 0.f;
@@ -1600,23 +1681,14 @@ static int memo_attempt(start_ctx *c, const MarchArgs &m, float theta, size_t ca
         if (cudaEventElapsedTime(&ms, c->lev_ev[2], c->lev_ev[3]) == cudaSuccess) c->link_ms += ms;
         else cudaGetLastError();
     }
-    for (int q : {(int)C_JUMP_ADV, (int)C_JUMP_EXTRA, (int)C_JUMP_COPY})
-        ST_CUDA(c, cudaMemsetAsync(ctr + q, 0, sizeof(unsigned long long), s));
-    k_sum_jump_counts<<<grid_for(nparts, 1024, 4 * (long long)nsm), 1024, 0, s>>>(
-        c->m_part.as<unsigned long long>(), nparts, ctr);
-    ++c->launches;
-    unsigned long long jc[3] = {0, 0, 0};
-    ST_CUDA(c, cudaMemcpyAsync(&jc[0], ctr + C_JUMP_ADV, 8, cudaMemcpyDeviceToHost, s));
-    ST_CUDA(c, cudaMemcpyAsync(&jc[1], ctr + C_JUMP_EXTRA, 8, cudaMemcpyDeviceToHost, s));
-    ST_CUDA(c, cudaMemcpyAsync(&jc[2], ctr + C_JUMP_COPY, 8, cudaMemcpyDeviceToHost, s));
-    ST_CUDA(c, cudaStreamSynchronize(s));
     c->jump_rounds += rounds;
-    // own state read per slot and round; per advancing slot one successor read
-    // and the write, plus the extra successor reads; closed chains copied once
-    // (16-byte states in the counting form, 8-byte ones otherwise)
+    // own state read per slot and round, and what the rounds moved beyond
+    // that: per advancing slot one successor read and the write, the extra
+    // successor reads, closed chains copied once (16-byte states in the
+    // counting form, 8-byte ones otherwise); the Gamma sum counts its own
+    // chain reads (C_JUMP_TAIL)
     const unsigned long long sb = wide ? 16ull : 8ull;
-    c->jump_bytes += sb * (unsigned long long)nslots * (unsigned long long)rounds +
-                     2 * sb * jc[0] + sb * jc[1] + sb * jc[2];
+    c->jump_bytes += sb * ((unsigned long long)nslots * (unsigned long long)rounds + jc[0]);
     if (timing) c->jump_ms += jump_ms;
     c->memo_final = b;
     c->memo_wide = wide;
@@ -1644,6 +1716,7 @@ int memo_gamma(start_ctx *c, const MarchArgs &m, long long t0, long long t1, u64
     a.EN = (u32)(c->walk_emit ? c->et.n : 0);
     a.svid = c->m_vid.as<u32>();
     a.state = c->m_st[c->memo_final].as<uint2>();
+    a.cap = (u32)c->memo_slots;   // chain links of the march
     a.wstate = c->memo_wide ? c->m_w[c->memo_final].as<uint4>() : nullptr;
     // a whole row per warp; the short rows of one group of a split solve eight
     // lanes each
