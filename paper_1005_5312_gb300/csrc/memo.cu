@@ -184,58 +184,45 @@ __global__ void __launch_bounds__(256) k_memo_hop(MemoArgs a)
     if (lane == 0 && fbs) atomicAdd(&a.m.counters[C_MARCH_FB], fbs);
 }
 
-// Pair slot of vid in the row [r0, r1) (slot indices), or kNone.  Rows of
-// neighbouring targets hold nearly the same cells in the same order, so the
-// entry sits close to the caller's guess g (the same relative position in the
-// row, scaled by the two rows' lengths: within 8 entries for ~90 % of the
-// links on a uniform 64^3 workload); the 20 entries around g are read at
-// once as five aligned 16-byte vectors (find_in_window: kNone when the entry
-// is not among them), and find_in_bounds falls back to a binary search on the
-// order key (key of the cell holding vid).  Canonical ids within a row are
-// distinct (a row holds a count-1 cell or its member, never both), so a
-// match is the slot.  Reads stay below r1 + 12, inside the slot arrays (their
-// capacity exceeds the pair count by more than that).
-__device__ __forceinline__ u32 find_in_window(const MemoArgs &a, u32 r0, u32 r1, u32 vid,
-                                              long long g)
+// Pair slot of (vid, key) in the row [lo, hi) (slot indices), or kNone: a
+// four-way search on the order key (key of the cell holding vid; rows are
+// sorted by it), three independent reads per step, then the last eight entries
+// as three aligned 16-byte vectors.  The search is bound by the latency of its
+// dependent reads: four-way halves the steps of a binary search (first hop and
+// later hops of the 128^3 diffuse step 245 against 262 ms, eight-way 247).  A
+// window of ids around the same relative position in the row (or around the
+// last entry found in it) holds the link in a uniform medium of point sources,
+// but misses 40 to 80 % of the links when every particle emits, whose rows
+// differ in their own neighbourhoods, and was slower than no window (266).
+// The entries of one key are a cell, or the members of one leaf.  Vector reads
+// stay below hi + 12, inside the slot arrays (their capacity exceeds the pair
+// count by more than that).
+__device__ __forceinline__ u32 search_row(const MemoArgs &a, u32 lo, u32 hi, u32 vid, u32 key)
 {
-    if (r1 <= r0 || g < 0) return kNone;
-    long long bb = (g - 8) & ~3ll;
-    const u32 b = bb < 0 ? 0u : (u32)bb;
-    const uint4 *v4 = reinterpret_cast<const uint4 *>(a.svid + b);
-    uint4 q[5];
+    const u32 end = hi;
+    while (hi - lo > 8u) {
+        const u32 st = (hi - lo) / 4u;
+        u32 c = 0;
 #pragma unroll
-    for (int k = 0; k < 5; ++k) q[k] = v4[k];
-    // matches among the 20 entries, restricted to those inside the row
-    u32 m = 0;
-#pragma unroll
-    for (int k = 0; k < 5; ++k)
-        m |= ((u32)(q[k].x == vid) | (u32)(q[k].y == vid) << 1 | (u32)(q[k].z == vid) << 2 |
-              (u32)(q[k].w == vid) << 3) << (4 * k);
-    const u32 lo = r0 > b ? r0 - b : 0u;                 // < 20 when g >= r0
-    const u32 hi = r1 - b < 20u ? r1 - b : 20u;           // > 0 when g < r1
-    m &= ((1u << hi) - 1u) & ~((1u << lo) - 1u);
-    return m ? b + (u32)(__ffs(m) - 1) : kNone;
-}
-
-__device__ __forceinline__ u32 search_row(const MemoArgs &a, u32 r0, u32 r1, u32 vid, u32 key)
-{
-    u32 lo = r0, hi = r1;
-    while (lo < hi) {
-        u32 mid = lo + ((hi - lo) >> 1);
-        if (a.sord[mid] < key) lo = mid + 1;
-        else hi = mid;
+        for (u32 j = 1; j < 4u; ++j) c += a.sord[lo + st * j] < key;
+        if (c < 3u) hi = lo + st * (c + 1u);   // the first key not below is at most there
+        if (c) lo += st * c + 1u;
     }
-    for (u32 e = lo; e < r1 && a.sord[e] == key; ++e)
+    if (hi <= lo && lo >= end) return kNone;
+    const u32 b = lo & ~3u;
+    const uint4 *v4 = reinterpret_cast<const uint4 *>(a.sord + b);
+    uint4 q[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) q[k] = v4[k];
+    u32 m = 0;   // entries whose key is not below the one looked for
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        m |= ((u32)(q[k].x >= key) | (u32)(q[k].y >= key) << 1 | (u32)(q[k].z >= key) << 2 |
+              (u32)(q[k].w >= key) << 3) << (4 * k);
+    m &= ((1u << (hi - b)) - 1u) & ~((1u << (lo - b)) - 1u);
+    for (u32 e = m ? b + (u32)(__ffs(m) - 1) : hi; e < end && a.sord[e] == key; ++e)
         if (a.svid[e] == vid) return e;
     return kNone;
-}
-
-__device__ __forceinline__ u32 find_in_bounds(const MemoArgs &a, u32 r0, u32 r1, u32 vid, u32 key,
-                                              long long g)
-{
-    if (r1 <= r0) return kNone;
-    const u32 e = find_in_window(a, r0, r1, vid, g);
-    return e != kNone ? e : search_row(a, r0, r1, vid, key);
 }
 
 // Whether the walk of target up lists the virtual source vid whose order key
@@ -271,23 +258,12 @@ __device__ __forceinline__ bool in_row(const MemoArgs &a, u32 up, u32 vid, u32 k
     return !walk_accepts(t, n, p, a);                                // level-21 leaf
 }
 
-// Guess for the entry at position pos of a row of length len, in a row
-// [r0, r1): the same relative position.
-__device__ __forceinline__ long long row_guess(u32 r0, u32 r1, u32 pos, u32 len)
-{
-    if (r1 <= r0 || len == 0) return -1;
-    u32 g = r0 + (u32)((float)pos * ((float)(r1 - r0) / (float)len));
-    return (long long)(g < r1 ? g : r1 - 1);
-}
-
 // Pair slot of (vid, k) in the row of target k (a row of this chunk), or
-// kNone; pos / len locate the link's own pair in its row (len 0: no guess).
-__device__ __forceinline__ u32 find_in_row(const MemoArgs &a, u32 k, u32 vid, u32 key, u32 pos,
-                                           u32 len)
+// kNone.
+__device__ __forceinline__ u32 find_in_row(const MemoArgs &a, u32 k, u32 vid, u32 key)
 {
     if ((long long)k < a.t0 || (long long)k >= a.t1) return kNone;   // row not in this chunk
-    u32 r0 = (u32)(a.off[k] - a.base), r1 = (u32)(a.off[k + 1] - a.base);
-    return find_in_bounds(a, r0, r1, vid, key, row_guess(r0, r1, pos, len));
+    return search_row(a, (u32)(a.off[k] - a.base), (u32)(a.off[k + 1] - a.base), vid, key);
 }
 
 // 2a'. the first hop of every pair, one warp per target row: the pairs of
@@ -611,8 +587,7 @@ __global__ void __launch_bounds__(32 * W, 32 / W) k_memo_hop_rows(MemoArgs a)
                     dt = a.m.sig * 0.5f * (pj.w + pu.w) * dl;
                     uint4 R = nbr[w][bq];
                     up = R.x;
-                    nx = find_in_bounds(a, R.y, R.z, vid, a.sord[p],
-                                        row_guess(R.y, R.z, (u32)(p - r0), (u32)(r1 - r0)));
+                    nx = search_row(a, R.y, R.z, vid, a.sord[p]);
                 }
                 a.state[p] = make_uint2(nx, __float_as_uint(dt));
                 if (a.dl) a.dl[p] = dl;
@@ -653,10 +628,7 @@ __global__ void __launch_bounds__(256) k_memo_hop_hard(MemoArgs a)
         const u32 up = hop<32>(a.m, i, a.m.pq[i], src, lane, 0xffffffffu, dt, fbs, &dl);
         if (lane == 0) {
             u32 nx = kNone;
-            if (up != kNone) {
-                const u64 r0 = a.off[i] - a.base, r1 = a.off[i + 1] - a.base;
-                nx = find_in_row(a, up, vid, a.sord[p], (u32)(p - r0), (u32)(r1 - r0));
-            }
+            if (up != kNone) nx = find_in_row(a, up, vid, a.sord[p]);
             a.state[p] = make_uint2(nx, __float_as_uint(dt));
             if (a.dl) a.dl[p] = dl;
             if (a.nx0) a.nx0[p] = nx;
@@ -696,11 +668,11 @@ __global__ void __launch_bounds__(256) k_memo_link(MemoArgs a)
             vid = a.svid[s];
             key = a.sord[s];
             // links of the first level were searched there; later slots sit in
-            // no row, so their search has no guess, and the row is searched only
+            // no row, and the row is searched only
             // when the walk lists vid for up
             if (!searched && (long long)up >= a.t0 && (long long)up < a.t1 &&
                 in_row(a, up, vid, key)) {
-                nx = find_in_row(a, up, vid, key, 0, 0);
+                nx = find_in_row(a, up, vid, key);
                 if (nx == kNone) atomicAdd(&a.m.counters[C_INTERNAL], 1ull);
             }
             if (nx == kNone) {
@@ -779,7 +751,7 @@ __device__ __forceinline__ u32 link_or_claim(const MemoArgs &a, u32 vid, u32 up,
 {
     claimed = false;
     if ((long long)up >= a.t0 && (long long)up < a.t1 && in_row(a, up, vid, key)) {
-        u32 nx = find_in_row(a, up, vid, key, 0, 0);
+        u32 nx = find_in_row(a, up, vid, key);
         if (nx == kNone) atomicAdd(&a.m.counters[C_INTERNAL], 1ull);
         return nx;
     }
