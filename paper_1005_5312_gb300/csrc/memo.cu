@@ -296,26 +296,26 @@ __device__ __forceinline__ void warp_append(bool flag, u32 slot, u32 tgt, uint2 
 }
 
 // Stages the neighbour list of target i (record pj) for one warp, entry q at
-// list offset q: the source-independent terms of neighbour k -- nba (r_k -
-// r_j, rsqrt |r_k - r_j|^2), nbb (|r_k - r_j|^2, e1, e0, -) with e1 |b| + e0
-// the error bound of the closer-than test, nbp the record of k, nbr (k, its
-// row bounds when its row belongs to [t0, t1)).  An entry at j's own
-// position is staged as one that never passes the test (A = 0, B = (1, 0,
-// 0)).  Returns the number staged (the list length); odd is set
-// (warp-uniform) when a distinct neighbour's FP32 offset underflowed, amax2
-// is the largest |r_k - r_j|^2.
+// list offset q: the source-independent terms of neighbour k -- nba the unit
+// vector e along r_k - r_j and |r_k - r_j| / 2, nbp the record of k, nbr (k,
+// its row bounds when its row belongs to [t0, t1)).  An entry at j's own
+// position is staged as one that never passes the closer-than test (e = 0, half
+// distance kFar).  Returns the number staged (the list length); odd is set
+// (warp-uniform) when a distinct neighbour's FP32 offset underflowed or comes
+// near it, amax2 is the largest |r_k - r_j|^2.
+constexpr float kFar = 1e30f;
+
 __device__ __forceinline__ int stage_row(const MarchArgs &m, u32 s0, u32 s1, float4 pj,
                                          long long t0, long long t1, const u64 *off, u64 base,
-                                         float4 *nba, float4 *nbb, float4 *nbp, uint4 *nbr,
-                                         bool &odd, float &amax2)
+                                         float4 *nba, float4 *nbp, uint4 *nbr, bool &odd,
+                                         float &amax2)
 {
-    const float eps_q = 16.f * kU32;
     const int lane = threadIdx.x & 31;
     bool od = false;
     float mx = 0.f;
     for (u32 b = s0; b < s1; b += 32) {
         u32 s = b + lane;
-        float4 A = make_float4(0.f, 0.f, 0.f, 0.f), B = make_float4(1.f, 0.f, 0.f, 0.f), P = A;
+        float4 A = make_float4(0.f, 0.f, 0.f, kFar), P = make_float4(0.f, 0.f, 0.f, 0.f);
         uint4 R = make_uint4(0u, 0u, 0u, 0u);
         if (s < s1) {
             u32 k = m.nb_idx[s];
@@ -323,13 +323,11 @@ __device__ __forceinline__ int stage_row(const MarchArgs &m, u32 s0, u32 s1, flo
                 P = m.pq[k];
                 float ax = P.x - pj.x, ay = P.y - pj.y, az = P.z - pj.z;
                 float a2 = ax * ax + ay * ay + az * az;
-                if (a2 == 0.f) {
+                if (a2 < 1e-34f) {
                     if (P.x != pj.x || P.y != pj.y || P.z != pj.z) od = true;
                 } else {
                     float ra = rsqrtf(a2);
-                    float an = a2 * ra;
-                    A = make_float4(ax, ay, az, ra);
-                    B = make_float4(a2, eps_q * 2.f * an, eps_q * a2 + 1e-37f, 0.f);
+                    A = make_float4(ax * ra, ay * ra, az * ra, 0.5f * a2 * ra);
                     R.x = k;
                     if ((long long)k >= t0 && (long long)k < t1) {
                         R.y = (u32)(off[k] - base);
@@ -340,7 +338,6 @@ __device__ __forceinline__ int stage_row(const MarchArgs &m, u32 s0, u32 s1, flo
             }
             const u32 q = s - s0;
             nba[q] = A;
-            nbb[q] = B;
             nbp[q] = P;
             nbr[q] = R;
         }
@@ -376,7 +373,7 @@ template <int W>
 __global__ void __launch_bounds__(32 * W) k_row_bins(MarchArgs m, const float4 *geo, int N,
                                                      unsigned long long *out, float *ramax)
 {
-    __shared__ float4 nba[W][kRowNB], nbb[W][kRowNB], nbp[W][kRowNB];
+    __shared__ float4 nba[W][kRowNB], nbp[W][kRowNB];
     __shared__ uint4 nbr[W][kRowNB];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / 32;
@@ -388,8 +385,8 @@ __global__ void __launch_bounds__(32 * W) k_row_bins(MarchArgs m, const float4 *
     bool odd = false;
     float amax2 = 0.f;
     if (s1 - s0 <= (u32)kRowNB)
-        nst = stage_row(m, s0, s1, m.pq[i], 0, 0, nullptr, 0, nba[w], nbb[w], nbp[w], nbr[w],
-                        odd, amax2);
+        nst = stage_row(m, s0, s1, m.pq[i], 0, 0, nullptr, 0, nba[w], nbp[w], nbr[w], odd,
+                        amax2);
     if (odd || nst == 0 || s1 - s0 > (u32)kRowNB || !(amax2 > 0.f)) {
         for (int b = lane; b < nbins; b += 32) row[b] = 0ull;
         if (lane == 0) ramax[i] = __int_as_float(0x7f800000);
@@ -398,20 +395,16 @@ __global__ void __launch_bounds__(32 * W) k_row_bins(MarchArgs m, const float4 *
     if (lane == 0) ramax[i] = sqrtf(amax2);
     // per neighbour: unit offset e_k and t_k = |r_k - r_j| / (2 amax) + eta
     // (over the staged record; 2 marks an entry at the target's own position)
-    // and sqrt(1 - t_k^2) (over the bound coefficients); with a_k = acos t_k,
+    // and sqrt(1 - t_k^2) (over the half distance); with a_k = acos t_k,
     // k passes the closer-than test for the whole bin iff theta_k < a_k - rho
     // (a_k > rho), i.e. cos theta_k > cos(a_k - rho) = t_k cos rho + sqrt(1 -
     // t_k^2) sin rho; the qualifying neighbour of largest cos theta_k sets L
     const float inv = 0.5f * rsqrtf(amax2);
     for (int q = lane; q < nst; q += 32) {
-        const float4 A = nba[w][q];
-        if (A.w > 0.f) {
-            const float t = nbb[w][q].x * A.w * inv + kBinEta;
-            nbp[w][q] = make_float4(A.x * A.w, A.y * A.w, A.z * A.w, t);
-            nbb[w][q].w = sqrtf(fmaxf(0.f, 1.f - t * t));
-        } else {
-            nbp[w][q] = make_float4(0.f, 0.f, 0.f, 2.f);
-        }
+        const float an = 2.f * nba[w][q].w;
+        const float t = an < kFar ? an * inv + kBinEta : 2.f;
+        nbp[w][q].x = t;
+        nba[w][q].w = sqrtf(fmaxf(0.f, 1.f - t * t));
     }
     __syncwarp();
     for (int b = lane; b < nbins; b += 32) {
@@ -419,10 +412,11 @@ __global__ void __launch_bounds__(32 * W) k_row_bins(MarchArgs m, const float4 *
         const float cr = g.w, sr = geo[2 * b + 1].x, rho = geo[2 * b + 1].y;
         float best = -2.f;   // cos theta of the qualifying neighbour nearest the axis
         for (int q = 0; q < nst; ++q) {
-            const float4 u = nbp[w][q];
+            const float4 u = nba[w][q];
+            const float t = nbp[w][q].x;
             const float ct = u.x * g.x + u.y * g.y + u.z * g.z;
-            const float thr = u.w * cr + nbb[w][q].w * sr;
-            if (u.w < cr && ct > thr + 1e-5f) best = fmaxf(best, ct);
+            const float thr = t * cr + u.w * sr;
+            if (t < cr && ct > thr + 1e-5f) best = fmaxf(best, ct);
         }
         unsigned long long mk = 0ull;
         if (best > -2.f) {
@@ -434,33 +428,49 @@ __global__ void __launch_bounds__(32 * W) k_row_bins(MarchArgs m, const float4 *
             const float ang = Lp <= -1.f ? 4.f : acosf(Lp) + rho;
             const float cmin = ang >= 3.14159f ? -2.f : cosf(ang) - 1e-5f;
             for (int q = 0; q < nst; ++q) {
-                const float4 u = nbp[w][q];
+                const float4 u = nba[w][q];
                 const float ct = u.x * g.x + u.y * g.y + u.z * g.z;
-                if (u.w < 1.5f && ct >= cmin) mk |= 1ull << q;
+                if (nbp[w][q].x < 1.5f && ct >= cmin) mk |= 1ull << q;
             }
         }
         row[b] = mk;
     }
 }
 
-// One staged candidate q of the first hop for a source at b = r_s - r_j
-// (|b| = bn): hop<G>'s closer-than test and score with their error bounds;
-// keeps the best and second-best scores, the best candidate and the
-// smallest margin of the tests.
-__device__ __forceinline__ void score_staged(const float4 A, const float4 B, float bx, float by,
-                                             float bz, float bn, int q, float &bc, float &sc,
-                                             int &bq, float &margin)
+// Four staged candidates q of the first hop for a source at b = r_s - r_j:
+// neighbour k is closer to the source than j iff its score b.e (e the unit
+// vector towards it) exceeds |r_k - r_j| / 2, hop<G>'s test divided by
+// 2 |r_k - r_j|.  Keeps the best and second-best scores of those that pass, the
+// best candidate and the smallest distance of a score from its threshold.  One
+// 16-byte read per candidate: with the unnormalised offsets, their bound
+// coefficients and a list of single candidates the scan took a second read
+// and about a quarter more instructions, and the kernel is bound by their
+// issue.
+__device__ __forceinline__ void score_staged4(const float4 *nba, uchar4 q, float bx, float by,
+                                              float bz, float &bc, float &sc, int &bq,
+                                              float &margin)
 {
-    const float dot = bx * A.x + by * A.y + bz * A.z;
-    const float qv = 2.f * dot - B.x;
-    const float eq = B.y * bn + B.z;
-    const bool pass = qv > eq;
-    margin = fminf(margin, fabsf(qv) - eq);
-    const float cv = pass ? dot * A.w : -2.f;
-    const bool better = cv > bc;
-    sc = better ? bc : fmaxf(sc, cv);
-    bc = better ? cv : bc;
-    bq = better ? q : bq;
+    float c[4];
+    const int id[4] = {q.x, q.y, q.z, q.w};
+    float mg = margin;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float4 A = nba[id[k]];
+        const float cv = bx * A.x + by * A.y + bz * A.z;
+        const float d = cv - A.w;
+        mg = fminf(mg, fabsf(d));
+        c[k] = d > 0.f ? cv : -1.f;
+    }
+    margin = mg;
+    const float h0 = fmaxf(c[0], c[1]), l0 = fminf(c[0], c[1]);
+    const float h1 = fmaxf(c[2], c[3]), l1 = fminf(c[2], c[3]);
+    const int i0 = c[1] > c[0] ? id[1] : id[0], i1 = c[3] > c[2] ? id[3] : id[2];
+    const float h = fmaxf(h0, h1);
+    const int ih = h1 > h0 ? i1 : i0;
+    const float second = fmaxf(fmaxf(l0, l1), fminf(h0, h1));
+    sc = fmaxf(fmaxf(sc, second), fminf(bc, h));
+    bq = h > bc ? ih : bq;
+    bc = fmaxf(bc, h);
 }
 
 // Appends the flagged lanes' (slot, upstream) to the first level's list of
@@ -489,11 +499,12 @@ __device__ __forceinline__ void append_miss(const MemoArgs &a, bool flag, u32 sl
 template <int W>
 __global__ void __launch_bounds__(32 * W, 32 / W) k_memo_hop_rows(MemoArgs a)
 {
-    __shared__ float4 nba[W][kRowNB];   // (r_k - r_j, rsqrt |r_k - r_j|^2)
-    __shared__ float4 nbb[W][kRowNB];   // (|r_k - r_j|^2, e1, e0, -): bound e1 |b| + e0
+    __shared__ float4 nba[W][kRowNB + 1];   // (unit vector to k, |r_k - r_j| / 2); one
+                                            // entry that never passes
     __shared__ float4 nbp[W][kRowNB];   // record of k
     __shared__ uint4 nbr[W][kRowNB];    // (k, row start, row end, -), slot indices
-    __shared__ unsigned char qsel[W][kRowNB];   // the candidates a warp iteration scans
+    // the candidates a warp iteration scans, padded to fours
+    __shared__ uchar4 qsel4[W][kRowNB / 4 + 1];
     const float two_eps = 32.f * kU32;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned me = 1u << lane;
@@ -510,8 +521,10 @@ __global__ void __launch_bounds__(32 * W, 32 / W) k_memo_hop_rows(MemoArgs a)
     }
     bool odd = false;   // a distinct neighbour whose FP32 offset underflowed
     float amax2 = 0.f;
-    const int nst = stage_row(a.m, s0, s1, pj, a.t0, a.t1, a.off, a.base, nba[w], nbb[w],
-                              nbp[w], nbr[w], odd, amax2);
+    if (lane == 0) nba[w][kRowNB] = make_float4(0.f, 0.f, 0.f, kFar);
+    const int nst = stage_row(a.m, s0, s1, pj, a.t0, a.t1, a.off, a.base, nba[w], nbp[w],
+                              nbr[w], odd, amax2);
+    unsigned char *qsel = reinterpret_cast<unsigned char *>(qsel4[w]);
     const unsigned long long all = nst >= 64 ? ~0ull : (1ull << nst) - 1ull;   // every candidate
     const float amax = sqrtf(amax2);
     const int nbins = 6 * a.m.rbn * a.m.rbn;
@@ -540,37 +553,28 @@ __global__ void __launch_bounds__(32 * W, 32 / W) k_memo_hop_rows(MemoArgs a)
                 if (bm) um = bm;
             }
         }
-        int nsel = nst;   // the union of the lanes' sets, listed in qsel when smaller
-        if (nbins) {
-            const unsigned lo = __reduce_or_sync(0xffffffffu, (unsigned)um);
-            const unsigned hi = __reduce_or_sync(0xffffffffu, (unsigned)(um >> 32));
-            const int n0 = __popc(lo);
-            nsel = n0 + __popc(hi);
-            if (nsel < nst) {
-                const unsigned below = me - 1u;
-                __syncwarp();   // the previous iteration's reads of qsel are done
-                if ((lo >> lane) & 1u) qsel[w][__popc(lo & below)] = (unsigned char)lane;
-                if ((hi >> lane) & 1u) qsel[w][n0 + __popc(hi & below)] = (unsigned char)(32 + lane);
-                __syncwarp();
-            }
+        // the union of the lanes' sets, listed
+        const unsigned lo = __reduce_or_sync(0xffffffffu, (unsigned)um);
+        const unsigned hi = __reduce_or_sync(0xffffffffu, (unsigned)(um >> 32));
+        const int n0 = __popc(lo), nsel = n0 + __popc(hi);
+        {
+            const unsigned below = me - 1u;
+            __syncwarp();   // the previous iteration's reads of qsel are done
+            if ((lo >> lane) & 1u) qsel[__popc(lo & below)] = (unsigned char)lane;
+            if ((hi >> lane) & 1u) qsel[n0 + __popc(hi & below)] = (unsigned char)(32 + lane);
+            if (lane < 3) qsel[nsel + lane] = (unsigned char)kRowNB;
+            __syncwarp();
         }
         if (valid) {
             float bc = -1.f, sc = -1.f;
             int bq = -1;
-            float margin = 1.f;   // min |q| - bound: <= 0 when a test is unsure
+            float margin = kFar;   // smallest distance of a score from its threshold
             if (count) cand += (unsigned)nsel;
-            if (nsel == nst) {
-#pragma unroll 4
-                for (int q = 0; q < nst; ++q)
-                    score_staged(nba[w][q], nbb[w][q], bx, by, bz, bn, q, bc, sc, bq, margin);
-            } else {
-#pragma unroll 4
-                for (int k = 0; k < nsel; ++k) {
-                    const int q = qsel[w][k];
-                    score_staged(nba[w][q], nbb[w][q], bx, by, bz, bn, q, bc, sc, bq, margin);
-                }
-            }
-            if (odd || !(margin > 0.f) || (sc > 0.f && sc > bc - two_eps * bn)) {
+            for (int k = 0; k < nsel; k += 4)
+                score_staged4(nba[w], qsel4[w][k >> 2], bx, by, bz, bc, sc, bq, margin);
+            // |score error| <= 16u |b| (as hop<G>'s), the threshold's <= 16u of it
+            if (odd || !(margin > 16.f * kU32 * (bn + 0.5f * amax)) ||
+                (sc > 0.f && sc > bc - two_eps * bn)) {
                 hard = true;   // decided in FP64 by k_memo_hop_hard
             } else {
                 float dt, dl;
