@@ -224,16 +224,11 @@ __global__ void k_scatter_d(const double *in, const u32 *inv, long long n, doubl
     if (i < n) out[inv[i]] = in[i];
 }
 
-__global__ void k_invert(const u32 *perm, long long n, u32 *inv)
-{
-    long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r < n) inv[perm[r]] = (u32)r;
-}
-
 // Morton-ordered particle records from the staged SoA inputs.
 __global__ void k_gather_particles(const float *pos, const float *h, const double *V,
                                    const u32 *perm, long long n, float4 *pq, float *ph,
-                                   double *Vm, float *nH, double *y, float *gam)
+                                   double *Vm, float *nH, double *y, float *gam, u32 *inv,
+                                   double *eL, float *eLs, double *Tg)
 {
     long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
@@ -245,6 +240,10 @@ __global__ void k_gather_particles(const float *pos, const float *h, const doubl
     nH[r] = 0.f;
     y[r] = 1.0;
     gam[r] = 0.f;
+    inv[i] = (u32)r;
+    eL[r] = 0.0;
+    eLs[r] = 0.f;
+    Tg[r] = 1e4;
 }
 
 __global__ void k_gather_sources(const float *pos, const double *L, const u32 *perm, long long n,
@@ -412,6 +411,14 @@ using namespace st;
 
 // ---------------------------------------------------------------- staging buffers
 namespace {
+// What a build leaves on the device for the host to read.
+struct BuildNotes {
+    FrameRec frame;
+    unsigned long long hist[3][kLevels + 1];   // cells per level: particles, sources, emitters
+    u32 cursor[3][kLevels + 1];
+    int bounds[8];
+};
+
 struct Staged {
     DBuf pos, h, spos, L, V;
     ~Staged()
@@ -563,19 +570,23 @@ int start_build_trees(start_ctx *c, const float *pos, const float *h, long long 
     ST_TRY(stage_in(c, in.spos, src_pos, 3 * n_s * sizeof(float)));
     ST_TRY(stage_in(c, in.L, src_L, n_s * sizeof(double)));
     if (diffuse) ST_TRY(stage_in(c, in.V, V, n_p * sizeof(double)));
-    ST_CUDA(c, cudaMemsetAsync(ctr + C_INTERNAL, 0, sizeof(unsigned long long), s));
     if (n_p) { k_check_pos_h<<<grid_for(n_p, 256), 256, 0, s>>>(in.h.as<float>(), n_p, ctr + C_BAD_INPUT); ++c->launches; }
     if (n_s) { k_check_nonneg_d<<<grid_for(n_s, 256), 256, 0, s>>>(in.L.as<double>(), n_s, ctr + C_BAD_INPUT, 0); ++c->launches; }
-    if (diffuse && n_p)
-        k_check_nonneg_d<<<grid_for(n_p, 256), 256, 0, s>>>(in.V.as<double>(), n_p, ctr + C_BAD_INPUT, 1); ++c->launches;
-    ST_TRY(check_bad(c, "h, src_L or V"));
+    if (diffuse && n_p) { k_check_nonneg_d<<<grid_for(n_p, 256), 256, 0, s>>>(in.V.as<double>(), n_p, ctr + C_BAD_INPUT, 1); ++c->launches; }
     if (n_p + n_s == 0) {
         c->pt.n = c->stree.n = c->et.n = 0;
         c->nb_total = 0;
         c->built = true;
         return START_OK;
     }
-    ST_TRY(compute_frame(c, in.pos.as<float>(), n_p, in.spos.as<float>(), n_s, &c->fr));
+    // the device's notes of a build: frame, cells per level of the three trees,
+    // and scratch; the host reads them once, when the sizes are needed
+    if (ensure(c->flags, sizeof(BuildNotes)))
+        return set_err(c, START_ENOMEM, "out of device memory (inputs)");
+    BuildNotes *notes = c->flags.as<BuildNotes>();
+    ST_CUDA(c, cudaMemsetAsync(notes, 0, sizeof(BuildNotes), s));
+    ST_TRY(compute_frame(c, in.pos.as<float>(), n_p, in.spos.as<float>(), n_s, notes->bounds,
+                         &notes->frame));
 
     // particles: keys, stable sort, Morton-ordered records
     size_t P = (size_t)(n_p ? n_p : 1), S = (size_t)(n_s ? n_s : 1);
@@ -586,24 +597,23 @@ int start_build_trees(start_ctx *c, const float *pos, const float *h, long long 
         ensure(c->skey, S * 8) || ensure(c->tv[1], S * 8) || ensure(c->sorig, S * 4) ||
         ensure(c->sq, S * 16) || ensure(c->sL, S * 8))
         return set_err(c, START_ENOMEM, "out of device memory (inputs)");
+    const FrameRec *frame = &notes->frame;   // device address
+    const Segs one;
     u64 *pks = c->tk[1].as<u64>();
     if (n_p) {
-        ST_TRY(morton_keys(c, in.pos.as<float>(), n_p, c->fr, pks, c->porig.as<u32>()));
+        ST_TRY(morton_keys(c, in.pos.as<float>(), n_p, frame, pks, c->porig.as<u32>()));
         ST_CUDA(c, cudaMemcpyAsync(c->pkey.p, pks, n_p * 8, cudaMemcpyDeviceToDevice, s));
         ST_TRY(radix_sort_pairs(c, pks, c->porig.as<u32>(), n_p));
-        k_invert<<<grid_for(n_p, 256), 256, 0, s>>>(c->porig.as<u32>(), n_p, c->pinv.as<u32>()); ++c->launches;
         k_gather_particles<<<grid_for(n_p, 256), 256, 0, s>>>(
             in.pos.as<float>(), in.h.as<float>(), diffuse ? in.V.as<double>() : nullptr,
             c->porig.as<u32>(), n_p, c->pq.as<float4>(), c->ph.as<float>(), c->V.as<double>(),
-            c->nH.as<float>(), c->y.as<double>(), c->gam.as<float>()); ++c->launches;
-        ST_CUDA(c, cudaMemsetAsync(c->eL.p, 0, n_p * 8, s));
-        ST_CUDA(c, cudaMemsetAsync(c->eLs.p, 0, n_p * 4, s));
-        k_fill_d<<<grid_for(n_p, 256), 256, 0, s>>>(c->Tg.as<double>(), n_p, 1e4); ++c->launches;
+            c->nH.as<float>(), c->y.as<double>(), c->gam.as<float>(), c->pinv.as<u32>(),
+            c->eL.as<double>(), c->eLs.as<float>(), c->Tg.as<double>()); ++c->launches;
         ST_CUDA(c, cudaGetLastError());
     }
     u64 *sks = c->tv[1].as<u64>();
     if (n_s) {
-        ST_TRY(morton_keys(c, in.spos.as<float>(), n_s, c->fr, sks, c->sorig.as<u32>()));
+        ST_TRY(morton_keys(c, in.spos.as<float>(), n_s, frame, sks, c->sorig.as<u32>()));
         ST_CUDA(c, cudaMemcpyAsync(c->skey.p, sks, n_s * 8, cudaMemcpyDeviceToDevice, s));
         ST_TRY(radix_sort_pairs(c, sks, c->sorig.as<u32>(), n_s));
         k_gather_sources<<<grid_for(n_s, 256), 256, 0, s>>>(in.spos.as<float>(), in.L.as<double>(),
@@ -611,14 +621,33 @@ int start_build_trees(start_ctx *c, const float *pos, const float *h, long long 
                                                             c->sq.as<float4>(), c->sL.as<double>()); ++c->launches;
         ST_CUDA(c, cudaGetLastError());
     }
-    ST_TRY(build_octree(c, c->pt, pks, n_p, c->p.ptree_leaf, c->fr));
-    ST_TRY(build_octree(c, c->stree, sks, n_s, c->p.src_leaf, c->fr));
+    ST_TRY(tree_census(c, c->pt, pks, n_p, c->p.ptree_leaf, one, notes->hist[0]));
+    ST_TRY(tree_census(c, c->stree, sks, n_s, c->p.src_leaf, one, notes->hist[1]));
+    c->et.n = 0;
+    if (diffuse) ST_TRY(tree_census(c, c->et, pks, n_p, c->p.src_leaf, one, notes->hist[2]));
+    BuildNotes bn;
+    unsigned long long bad[C_COUNT];
+    ST_CUDA(c, cudaMemcpyAsync(&bn, notes, sizeof(bn), cudaMemcpyDeviceToHost, s));
+    ST_CUDA(c, cudaMemcpyAsync(bad, ctr, sizeof(bad), cudaMemcpyDeviceToHost, s));
+    ST_CUDA(c, cudaStreamSynchronize(s));
+    if (bad[C_BAD_INPUT] || bad[C_BAD_POS]) {
+        ST_CUDA(c, cudaMemsetAsync(ctr, 0, C_COUNT * sizeof(unsigned long long), s));
+        return set_err(c, START_EINVAL, bad[C_BAD_INPUT] ? "invalid values in h, src_L or V"
+                                                         : "non-finite particle or source position");
+    }
+    for (int a = 0; a < 3; ++a) c->fr.lo[a] = bn.frame.lo[a];
+    c->fr.side = bn.frame.side;
+    c->fr.cmag = bn.frame.cmag;
+    ST_TRY(tree_emit(c, c->pt, pks, n_p, one, frame, bn.hist[0], notes->hist[0],
+                     notes->cursor[0], false));
+    ST_TRY(tree_emit(c, c->stree, sks, n_s, one, frame, bn.hist[1], notes->hist[1],
+                     notes->cursor[1], true));
     ST_TRY(tree_moments(c, c->stree, c->sq.as<float4>(), c->sL.as<double>(), c->p.L_unit));
-    if (diffuse) ST_TRY(build_octree(c, c->et, pks, n_p, c->p.src_leaf, c->fr));
-    else c->et.n = 0;
+    if (diffuse)
+        ST_TRY(tree_emit(c, c->et, pks, n_p, one, frame, bn.hist[2], notes->hist[2],
+                         notes->cursor[2], true));
     ST_TRY(build_neighbours(c));
     phase_mark(c, START_PHASE_BUILD, true);
-    ST_CUDA(c, cudaStreamSynchronize(s));
     ST_CUDA(c, cudaGetLastError());
     if (read_counter(c, C_INTERNAL)) return set_err(c, START_ECUDA, "internal inconsistency (trees or neighbour lists)");
     c->built = true;

@@ -49,7 +49,6 @@ long long bytes_in_use();
 // Octree in depth-first pre-order (children in octant order).
 struct Tree {
     long long n = 0;           // nodes
-    int depth = 0;             // deepest level present
     DBuf box;                  // float4: cube lower corner (rounded to float), edge
     DBuf meta;                 // uint4: skip, first, count, leaf
     DBuf cube;                 // double4-like: lower corner x,y,z, edge (exact frame values)
@@ -59,13 +58,39 @@ struct Tree {
     DBuf vsrc;                 // float4: luminosity centre, L / L_unit
     DBuf L;                    // double summed luminosity (photons/s)
     DBuf M;                    // double[3] summed L * r
-    // breadth-first bookkeeping used by the bottom-up moments
-    std::vector<long long> lvl_off;   // BFS index of the first node of each level
-    DBuf bfs2dfs;              // u32
-    DBuf bfs_first, bfs_count; // u32
-    DBuf bfs_cb, bfs_nc;       // u32 first child (BFS index), child count
-    bool small = false;        // built by one block (k_octree_small)
-    DBuf lvl_dev;              // u32 [depth + 2] level offsets (small trees)
+    // construction: per key the index of the first cell that starts there (u32,
+    // n + 1) and that cell's level (u8); the cells grouped by level (u32), with
+    // the first place of each level
+    DBuf pos, lst, lnode;
+    std::vector<long long> lvl_off;
+};
+
+// The root cube of one problem of a build, on the device.
+struct FrameRec {
+    double lo[3], side, scale;
+    float cmag, pad;
+};
+
+// Members of a batch of problems, one problem after the other: those of
+// problem b are [start[b], start[b + 1]).  n = 1: one problem (start unused).
+struct Segs {
+    const u32 *start = nullptr;
+    int n = 1;
+    int trees = 1;   // problems that hold members
+    // the problem of member i and its members [lo, hi) (left alone when n = 1)
+    __device__ __forceinline__ u32 range(u32 i, u32 &lo, u32 &hi) const
+    {
+        if (n == 1) return 0u;
+        u32 a = 0, b = (u32)n;   // the last b with start[b] <= i
+        while (b - a > 1) {
+            const u32 mid = (a + b) >> 1;
+            if (start[mid] <= i) a = mid;
+            else b = mid;
+        }
+        lo = start[a];
+        hi = start[a + 1];
+        return a;
+    }
 };
 
 struct Frame {
@@ -230,6 +255,7 @@ enum Counter {
     C_KLUM_BIG,   // kernel-weighted cell luminosities: cells left to a block each
     C_ROW_CAND,   // staged first hop, every 64th target: candidates scanned over its pairs
     C_ROW_NB,     // the same targets: staged neighbours x pairs (a full scan)
+    C_BAD_POS,    // non-finite positions of a build
     C_COUNT = 32
 };
 
@@ -274,13 +300,16 @@ int exclusive_scan_u32(start_ctx *c, const u32 *in, u32 *out, long long n, u32 *
 int exclusive_scan_u32_to_u64(start_ctx *c, const u32 *in, u64 *out, long long n);
 int radix_sort_pairs(start_ctx *c, u64 *keys, u32 *vals, long long n);
 int compute_frame(start_ctx *c, const float *ppos, long long np, const float *spos, long long ns,
-                  Frame *fr);
-int morton_keys(start_ctx *c, const float *pos_soa, long long n, const Frame &fr, u64 *keys,
+                  int *mm, FrameRec *fr);
+int morton_keys(start_ctx *c, const float *pos_soa, long long n, const FrameRec *fr, u64 *keys,
                 u32 *idx);
 
 // tree.cu
-int build_octree(start_ctx *c, Tree &t, const u64 *sorted_keys, long long n, int leaf,
-                 const Frame &fr);
+int tree_census(start_ctx *c, Tree &t, const u64 *keys, long long n, int leaf, const Segs &segs,
+                unsigned long long *hist);
+int tree_emit(start_ctx *c, Tree &t, const u64 *keys, long long n, const Segs &segs,
+              const FrameRec *frames, const unsigned long long *hist,
+              const unsigned long long *hist_dev, u32 *cursor, bool by_level);
 int tree_moments(start_ctx *c, Tree &t, const float4 *mem_pos, const double *mem_L,
                  double L_unit);
 void tree_release(Tree &t);

@@ -328,13 +328,6 @@ int radix_sort_pairs(start_ctx *c, u64 *keys, u32 *vals, long long n)
 }
 
 // ---------------------------------------------------------------- frame
-static float host_int_as_float(int i)
-{
-    float f;
-    memcpy(&f, &i, sizeof(f));
-    return f;
-}
-
 __device__ __forceinline__ int f2ord(float f)
 {
     int i = __float_as_int(f);
@@ -380,43 +373,41 @@ __global__ void k_bbox(const float *pos, long long n, int *mm, unsigned long lon
     }
 }
 
-int compute_frame(start_ctx *c, const float *ppos, long long np, const float *spos, long long ns,
-                  Frame *fr)
+// The root cube from the bounds mm: lower corner, largest extent (1 when it
+// is 0), keys per length, and a bound on every coordinate of a point or a cube
+// corner (FP64, never contracted).
+__global__ void k_frame(const int *mm, FrameRec *fr)
 {
-    ST_TRY(ensure(c->flags, 64));
-    int *mm = c->flags.as<int>();
-    unsigned long long *bad = c->counters.as<unsigned long long>() + C_BAD_INPUT;
-    k_bbox_init<<<1, 32, 0, c->stream>>>(mm); ++c->launches;
-    if (np) { k_bbox<<<grid_for(np, 256, 1024), 256, 0, c->stream>>>(ppos, np, mm, bad); ++c->launches; }
-    if (ns) { k_bbox<<<grid_for(ns, 256, 1024), 256, 0, c->stream>>>(spos, ns, mm, bad); ++c->launches; }
-    ST_CUDA(c, cudaGetLastError());
-    int h[6];
-    unsigned long long nbad = 0;
-    ST_CUDA(c, cudaMemcpyAsync(h, mm, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
-    ST_CUDA(c, cudaMemcpyAsync(&nbad, bad, sizeof(nbad), cudaMemcpyDeviceToHost, c->stream));
-    ST_CUDA(c, cudaStreamSynchronize(c->stream));
-    if (nbad) return set_err(c, START_EINVAL, "non-finite particle or source position");
-    double lo[3], hi[3];
+    double side = 0.0, mag;
+    double lo[3];
     for (int a = 0; a < 3; ++a) {
-        int i = h[a], j = h[3 + a];
-        lo[a] = (double)host_int_as_float(i >= 0 ? i : i ^ 0x7fffffff);
-        hi[a] = (double)host_int_as_float(j >= 0 ? j : j ^ 0x7fffffff);
-    }
-    double side = 0.0;
-    for (int a = 0; a < 3; ++a) {
-        double e = hi[a] - lo[a];
+        lo[a] = (double)ord2f(mm[a]);
+        const double e = __dsub_rn((double)ord2f(mm[3 + a]), lo[a]);
         if (e > side) side = e;
     }
     if (!(side > 0.0)) side = 1.0;
-    double mag = side;
+    mag = side;
     for (int a = 0; a < 3; ++a) {
         fr->lo[a] = lo[a];
-        mag = fmax(mag, fmax(fabs(lo[a]), fabs(lo[a] + side)));
+        mag = fmax(mag, fmax(fabs(lo[a]), fabs(__dadd_rn(lo[a], side))));
     }
     fr->side = side;
-    fr->scale = 2097152.0 / side;
-    fr->cmag = (float)(mag * (1.0 + 1e-6));
-    return START_OK;
+    fr->scale = __ddiv_rn(2097152.0, side);
+    fr->cmag = (float)__dmul_rn(mag, 1.0 + 1e-6);
+    fr->pad = 0.f;
+}
+
+// Issues the frame of np particles and ns sources (mm: six ints of scratch);
+// non-finite positions are counted in C_BAD_POS.
+int compute_frame(start_ctx *c, const float *ppos, long long np, const float *spos, long long ns,
+                  int *mm, FrameRec *fr)
+{
+    unsigned long long *bad = c->counters.as<unsigned long long>() + C_BAD_POS;
+    k_bbox_init<<<1, 32, 0, c->stream>>>(mm); ++c->launches;
+    if (np) { k_bbox<<<grid_for(np, 256, 1024), 256, 0, c->stream>>>(ppos, np, mm, bad); ++c->launches; }
+    if (ns) { k_bbox<<<grid_for(ns, 256, 1024), 256, 0, c->stream>>>(spos, ns, mm, bad); ++c->launches; }
+    k_frame<<<1, 1, 0, c->stream>>>(mm, fr); ++c->launches;
+    return cuda_check(c, cudaGetLastError(), "k_frame");
 }
 
 // ---------------------------------------------------------------- Morton keys
@@ -431,16 +422,15 @@ __device__ __forceinline__ u64 spread3(u64 v)
     return v;
 }
 
-__global__ void k_morton(const float *pos, long long n, double lox, double loy, double loz,
-                         double scale, u64 *keys, u32 *idx)
+__global__ void k_morton(const float *pos, long long n, const FrameRec *fr, u64 *keys, u32 *idx)
 {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    double lo[3] = {lox, loy, loz};
     u64 q[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        double t = floor(__dmul_rn(__dsub_rn((double)pos[(long long)a * n + i], lo[a]), scale));
+        double t = floor(__dmul_rn(__dsub_rn((double)pos[(long long)a * n + i], fr->lo[a]),
+                                   fr->scale));
         t = fmin(fmax(t, 0.0), 2097151.0);
         q[a] = (u64)t;
     }
@@ -448,11 +438,11 @@ __global__ void k_morton(const float *pos, long long n, double lox, double loy, 
     if (idx) idx[i] = (u32)i;
 }
 
-int morton_keys(start_ctx *c, const float *pos_soa, long long n, const Frame &fr, u64 *keys, u32 *idx)
+int morton_keys(start_ctx *c, const float *pos_soa, long long n, const FrameRec *fr, u64 *keys,
+                u32 *idx)
 {
     if (n <= 0) return START_OK;
-    k_morton<<<grid_for(n, 256), 256, 0, c->stream>>>(pos_soa, n, fr.lo[0], fr.lo[1], fr.lo[2],
-                                                     fr.scale, keys, idx); ++c->launches;
+    k_morton<<<grid_for(n, 256), 256, 0, c->stream>>>(pos_soa, n, fr, keys, idx); ++c->launches;
     return cuda_check(c, cudaGetLastError(), "k_morton");
 }
 

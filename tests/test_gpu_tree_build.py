@@ -1,0 +1,55 @@
+"""Octrees and orders at the sizes and clusterings where their passes change:
+one key, one block more or less, duplicates (a level-21 leaf of several
+members), leaves of several members, tight clumps (long runs of equal leading
+key bits).  Bit for bit against the oracle.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from start_inputs import ALPHA_A, ALPHA_B, KPC_CM, SIGMA_CM2
+
+pytestmark = pytest.mark.gpu
+
+
+def points(n, clump, seed):
+    """n points in a box, the first `clump` of them within 1e-5 of each
+    other, every seventh a duplicate of its predecessor when there are ten."""
+    rng = np.random.default_rng(seed)
+    pos = rng.uniform(0.0, 2.0, (3, n)).astype(np.float32)
+    if clump:
+        pos[:, :clump] = (pos[:, :1] + np.float32(1e-5) * rng.uniform(0, 1, (3, clump))
+                          ).astype(np.float32)
+    if n >= 10:
+        pos[:, 7::7] = pos[:, 6:-1:7]
+    return pos
+
+
+@pytest.mark.parametrize("n,clump", [(1, 0), (2, 0), (9, 0), (255, 0), (257, 40), (4096, 0),
+                                     (4097, 500), (16384, 0), (16385, 0), (20011, 33),
+                                     (20011, 3000), (70001, 20), (300007, 0)])
+@pytest.mark.parametrize("leaf", [1, 3])
+def test_orders_and_trees_are_the_oracles(n, clump, leaf):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1005_5312_gb300 as S
+    S.build()
+    src = points(n, clump, n + clump)
+    rng = np.random.default_rng(n)
+    L = rng.lognormal(0.0, 1.0, n) * 1e48
+    pos = rng.uniform(0.0, 2.0, (3, 3)).astype(np.float32)
+    h = np.full(3, 1e-3, np.float32)
+    ctx = S.Context(src_leaf=leaf)
+    orc = oracle.Oracle(pos, h, src, L, sigma_cm2=SIGMA_CM2, len_unit_cm=KPC_CM, alpha_A=ALPHA_A,
+                        alpha_B=ALPHA_B, src_leaf=leaf)
+    for _ in range(2):   # a second build of the same points uses what the first left
+        ctx.build_trees(pos, h, src, L)
+        assert np.array_equal(ctx.keys(1), orc.keys(1))
+        assert np.array_equal(ctx.perm(1).astype(np.int64), orc.perm(1))
+        tg, to = ctx.tree(1), orc.tree(1)
+        assert len(tg["level"]) == len(to["level"])
+        for k in ("level", "first", "count", "skip", "leaf"):
+            assert np.array_equal(tg[k].astype(np.int64), to[k].astype(np.int64)), k
+        for k in ("cube", "L", "cen"):
+            assert np.array_equal(tg[k], to[k]), k
