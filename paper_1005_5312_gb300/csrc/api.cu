@@ -416,6 +416,7 @@ struct BuildNotes {
     FrameRec frame;
     unsigned long long hist[3][kLevels + 1];   // cells per level: particles, sources, emitters
     u32 cursor[3][kLevels + 1];
+    u32 long_runs;   // runs of equal leading key bits that the sort left
     int bounds[8];
 };
 
@@ -599,42 +600,51 @@ int start_build_trees(start_ctx *c, const float *pos, const float *h, long long 
         return set_err(c, START_ENOMEM, "out of device memory (inputs)");
     const FrameRec *frame = &notes->frame;   // device address
     const Segs one;
-    u64 *pks = c->tk[1].as<u64>();
+    u64 *pks = c->tk[1].as<u64>(), *sks = c->tv[1].as<u64>();
+    if (n_p) ST_TRY(morton_keys(c, in.pos.as<float>(), n_p, frame, c->pkey.as<u64>()));
+    if (n_s) ST_TRY(morton_keys(c, in.spos.as<float>(), n_s, frame, c->skey.as<u64>()));
+    BuildNotes bn;
+    for (int attempt = 0;; ++attempt) {
+        ST_TRY(sort_keys(c, c->pkey.as<u64>(), n_p, pks, c->porig.as<u32>(), c->sort_all_bits,
+                         &notes->long_runs));
+        ST_TRY(sort_keys(c, c->skey.as<u64>(), n_s, sks, c->sorig.as<u32>(), c->sort_all_bits,
+                         &notes->long_runs));
+        ST_TRY(tree_census(c, c->pt, pks, n_p, c->p.ptree_leaf, one, notes->hist[0]));
+        ST_TRY(tree_census(c, c->stree, sks, n_s, c->p.src_leaf, one, notes->hist[1]));
+        c->et.n = 0;
+        if (diffuse)
+            ST_TRY(tree_census(c, c->et, pks, n_p, c->p.src_leaf, one, notes->hist[2]));
+        unsigned long long bad[C_COUNT];
+        ST_CUDA(c, cudaMemcpyAsync(&bn, notes, sizeof(bn), cudaMemcpyDeviceToHost, s));
+        ST_CUDA(c, cudaMemcpyAsync(bad, ctr, sizeof(bad), cudaMemcpyDeviceToHost, s));
+        ST_CUDA(c, cudaStreamSynchronize(s));
+        if (bad[C_BAD_INPUT] || bad[C_BAD_POS]) {
+            ST_CUDA(c, cudaMemsetAsync(ctr, 0, C_COUNT * sizeof(unsigned long long), s));
+            return set_err(c, START_EINVAL, bad[C_BAD_INPUT]
+                                                ? "invalid values in h, src_L or V"
+                                                : "non-finite particle or source position");
+        }
+        if (!bn.long_runs) break;
+        if (attempt) return set_err(c, START_ECUDA, "internal inconsistency (sort)");
+        c->sort_all_bits = true;   // tight clumps: all bits, also in the next builds
+        ST_CUDA(c, cudaMemsetAsync(notes->hist, 0, sizeof(bn.hist), s));
+        ST_CUDA(c, cudaMemsetAsync(&notes->long_runs, 0, sizeof(bn.long_runs), s));
+    }
     if (n_p) {
-        ST_TRY(morton_keys(c, in.pos.as<float>(), n_p, frame, pks, c->porig.as<u32>()));
-        ST_CUDA(c, cudaMemcpyAsync(c->pkey.p, pks, n_p * 8, cudaMemcpyDeviceToDevice, s));
-        ST_TRY(radix_sort_pairs(c, pks, c->porig.as<u32>(), n_p));
         k_gather_particles<<<grid_for(n_p, 256), 256, 0, s>>>(
             in.pos.as<float>(), in.h.as<float>(), diffuse ? in.V.as<double>() : nullptr,
             c->porig.as<u32>(), n_p, c->pq.as<float4>(), c->ph.as<float>(), c->V.as<double>(),
             c->nH.as<float>(), c->y.as<double>(), c->gam.as<float>(), c->pinv.as<u32>(),
-            c->eL.as<double>(), c->eLs.as<float>(), c->Tg.as<double>()); ++c->launches;
-        ST_CUDA(c, cudaGetLastError());
+            c->eL.as<double>(), c->eLs.as<float>(), c->Tg.as<double>());
+        ++c->launches;
     }
-    u64 *sks = c->tv[1].as<u64>();
     if (n_s) {
-        ST_TRY(morton_keys(c, in.spos.as<float>(), n_s, frame, sks, c->sorig.as<u32>()));
-        ST_CUDA(c, cudaMemcpyAsync(c->skey.p, sks, n_s * 8, cudaMemcpyDeviceToDevice, s));
-        ST_TRY(radix_sort_pairs(c, sks, c->sorig.as<u32>(), n_s));
         k_gather_sources<<<grid_for(n_s, 256), 256, 0, s>>>(in.spos.as<float>(), in.L.as<double>(),
                                                             c->sorig.as<u32>(), n_s, c->p.L_unit,
-                                                            c->sq.as<float4>(), c->sL.as<double>()); ++c->launches;
-        ST_CUDA(c, cudaGetLastError());
+                                                            c->sq.as<float4>(), c->sL.as<double>());
+        ++c->launches;
     }
-    ST_TRY(tree_census(c, c->pt, pks, n_p, c->p.ptree_leaf, one, notes->hist[0]));
-    ST_TRY(tree_census(c, c->stree, sks, n_s, c->p.src_leaf, one, notes->hist[1]));
-    c->et.n = 0;
-    if (diffuse) ST_TRY(tree_census(c, c->et, pks, n_p, c->p.src_leaf, one, notes->hist[2]));
-    BuildNotes bn;
-    unsigned long long bad[C_COUNT];
-    ST_CUDA(c, cudaMemcpyAsync(&bn, notes, sizeof(bn), cudaMemcpyDeviceToHost, s));
-    ST_CUDA(c, cudaMemcpyAsync(bad, ctr, sizeof(bad), cudaMemcpyDeviceToHost, s));
-    ST_CUDA(c, cudaStreamSynchronize(s));
-    if (bad[C_BAD_INPUT] || bad[C_BAD_POS]) {
-        ST_CUDA(c, cudaMemsetAsync(ctr, 0, C_COUNT * sizeof(unsigned long long), s));
-        return set_err(c, START_EINVAL, bad[C_BAD_INPUT] ? "invalid values in h, src_L or V"
-                                                         : "non-finite particle or source position");
-    }
+    ST_CUDA(c, cudaGetLastError());
     for (int a = 0; a < 3; ++a) c->fr.lo[a] = bn.frame.lo[a];
     c->fr.side = bn.frame.side;
     c->fr.cmag = bn.frame.cmag;

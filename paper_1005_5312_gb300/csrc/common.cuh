@@ -212,6 +212,7 @@ struct start_ctx {
     cudaStream_t r_cap = nullptr;      // private stream the graph is captured on
 
     // generic scratch
+    bool sort_all_bits = false;   // the last build's keys had long runs of equal leading bits
     st::DBuf tk[2], tv[2], hist, scan_tmp, stage, flags;
     st::DBuf counters; // u64[C_COUNT]
 
@@ -298,11 +299,11 @@ void phase_mark(start_ctx *c, int phase, bool end);
 // scan_sort.cu
 int exclusive_scan_u32(start_ctx *c, const u32 *in, u32 *out, long long n, u32 *total_dev);
 int exclusive_scan_u32_to_u64(start_ctx *c, const u32 *in, u64 *out, long long n);
-int radix_sort_pairs(start_ctx *c, u64 *keys, u32 *vals, long long n);
+int sort_keys(start_ctx *c, const u64 *keys, long long n, u64 *sorted, u32 *perm, bool all_bits,
+              u32 *longer);
 int compute_frame(start_ctx *c, const float *ppos, long long np, const float *spos, long long ns,
                   int *mm, FrameRec *fr);
-int morton_keys(start_ctx *c, const float *pos_soa, long long n, const FrameRec *fr, u64 *keys,
-                u32 *idx);
+int morton_keys(start_ctx *c, const float *pos_soa, long long n, const FrameRec *fr, u64 *keys);
 
 // tree.cu
 int tree_census(start_ctx *c, Tree &t, const u64 *keys, long long n, int leaf, const Segs &segs,

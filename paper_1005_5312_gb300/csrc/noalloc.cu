@@ -27,11 +27,10 @@ namespace st {
 // pointers into the fixed scratch.
 __global__ void k_bbox_init(int *mm);
 __global__ void k_bbox(const float *pos, long long n, int *mm, unsigned long long *bad);
-__global__ void __launch_bounds__(256) k_rs_hist(const u64 *keys, long long n, int shift,
-                                                 u32 *hist, int nblocks);
-__global__ void __launch_bounds__(256) k_rs_scatter(const u64 *kin, const u32 *vin, u64 *kout,
-                                                    u32 *vout, long long n, int shift,
-                                                    const u32 *offs, int nblocks);
+void rs_tile_hist(const u64 *keys, long long n, int shift, u32 *hist, int nblocks,
+                  cudaStream_t s);
+void rs_tile_scatter(const u64 *kin, const u32 *vin, u64 *kout, u32 *vout, long long n, int shift,
+                     const u32 *offs, int nblocks, cudaStream_t s);
 
 namespace {
 
@@ -211,9 +210,9 @@ extern "C" int start_morton_order_noalloc(const float *pos, long long n, unsigne
     u64 *k0 = ka, *k1 = kb;
     u32 *v0 = perm_out, *v1 = vb;
     for (int pass = 0; pass < 8; ++pass) {
-        k_rs_hist<<<nblocks, 256, 0, s>>>(k0, n, 8 * pass, hist, nblocks);
+        rs_tile_hist(k0, n, 8 * pass, hist, nblocks, s);
         k_scan_hist<<<1, 1024, 0, s>>>(hist, offs, 256 * nblocks);
-        k_rs_scatter<<<nblocks, 256, 0, s>>>(k0, v0, k1, v1, n, 8 * pass, offs, nblocks);
+        rs_tile_scatter(k0, v0, k1, v1, n, 8 * pass, offs, nblocks, s);
         u64 *tk = k0; k0 = k1; k1 = tk;
         u32 *tv = v0; v0 = v1; v1 = tv;
     }

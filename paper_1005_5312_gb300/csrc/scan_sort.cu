@@ -96,6 +96,34 @@ __global__ void k_tile_scan(const Tin *in, Tout *out, long long n, const Tout *t
     }
 }
 
+// Exclusive scan of up to kScanOne values by one block, each thread a
+// contiguous piece: one launch instead of the three of the tiled form, whose
+// latency the small scans of a sort pass consist of.
+constexpr long long kScanOne = 16384;
+
+template <class Tin, class Tout>
+__global__ void __launch_bounds__(1024) k_scan_one(const Tin *in, Tout *out, int n, Tout *total)
+{
+    __shared__ Tout wt[32];
+    const int per = (n + 1023) / 1024;
+    const int b0 = min(n, (int)threadIdx.x * per), b1 = min(n, b0 + per);
+    Tout v[(kScanOne + 1023) / 1024];
+    Tout s = 0;
+#pragma unroll
+    for (int i = 0; i < (int)((kScanOne + 1023) / 1024); ++i) {
+        v[i] = b0 + i < b1 ? (Tout)in[b0 + i] : Tout(0);
+        s += v[i];
+    }
+    Tout tot;
+    Tout run = block_exclusive_scan<Tout>(s, wt, &tot);
+#pragma unroll
+    for (int i = 0; i < (int)((kScanOne + 1023) / 1024); ++i) {
+        if (b0 + i < b1) out[b0 + i] = run;
+        run += v[i];
+    }
+    if (total && threadIdx.x == 0) *total = tot;
+}
+
 // Exclusive scan of n values; scratch holds the per-tile partial sums of
 // every recursion level.
 template <class Tin, class Tout>
@@ -107,9 +135,9 @@ static int scan_impl(start_ctx *c, const Tin *in, Tout *out, long long n, Tout *
         return START_OK;
     }
     long long tiles = (n + kScanTile - 1) / kScanTile;
-    if (tiles == 1) {
-        k_tile_scan<Tin, Tout><<<1, kScanThreads, 0, c->stream>>>(in, out, n, nullptr, total); ++c->launches;
-        return cuda_check(c, cudaGetLastError(), "k_tile_scan");
+    if (n <= kScanOne) {
+        k_scan_one<Tin, Tout><<<1, 1024, 0, c->stream>>>(in, out, (int)n, total); ++c->launches;
+        return cuda_check(c, cudaGetLastError(), "k_scan_one");
     }
     Tout *sums = scratch;
     Tout *sums_scan = scratch + tiles;
@@ -148,18 +176,20 @@ int exclusive_scan_u32_to_u64(start_ctx *c, const u32 *in, u64 *out, long long n
 
 // ---------------------------------------------------------------- radix sort
 constexpr int kRsThreads = 256;
-constexpr int kRsIpt = 16;
-constexpr int kRsTile = kRsThreads * kRsIpt;   // 4096 items per block
+// items per thread: tiles of 4096 items, or of 1024 below kRsSmallTiles items,
+// where the long tiles leave most SMs idle (18 against 6 us per pass at 23 k)
+constexpr long long kRsSmallTiles = 1LL << 18;
 constexpr int kRsWarps = kRsThreads / 32;
 
+template <int IPT>
 __global__ void __launch_bounds__(kRsThreads) k_rs_hist(const u64 *keys, long long n, int shift,
                                                         u32 *hist, int nblocks)
 {
     __shared__ u32 h[256];
     for (int d = threadIdx.x; d < 256; d += kRsThreads) h[d] = 0;
     __syncthreads();
-    long long t0 = (long long)blockIdx.x * kRsTile;
-    for (int i = 0; i < kRsIpt; ++i) {
+    long long t0 = (long long)blockIdx.x * (kRsThreads * IPT);
+    for (int i = 0; i < IPT; ++i) {
         long long idx = t0 + (long long)i * kRsThreads + threadIdx.x;
         if (idx < n) atomicAdd(&h[(keys[idx] >> shift) & 255u], 1u);
     }
@@ -168,7 +198,9 @@ __global__ void __launch_bounds__(kRsThreads) k_rs_hist(const u64 *keys, long lo
 }
 
 // Stable scatter: within a tile the items are ranked in index order
-// (warp-major, then round, then lane) with warp match/popc.
+// (warp-major, then round, then lane) with warp match/popc.  vin NULL: the
+// values are the items' indices.
+template <int IPT>
 __global__ void __launch_bounds__(kRsThreads) k_rs_scatter(const u64 *kin, const u32 *vin,
                                                            u64 *kout, u32 *vout, long long n,
                                                            int shift, const u32 *offs,
@@ -180,16 +212,16 @@ __global__ void __launch_bounds__(kRsThreads) k_rs_scatter(const u64 *kin, const
     for (int i = threadIdx.x; i < kRsWarps * 256; i += kRsThreads) (&wcnt[0][0])[i] = 0;
     __syncthreads();
     unsigned lt = (1u << lane) - 1u;
-    long long wbase = (long long)blockIdx.x * kRsTile + (long long)warp * 32 * kRsIpt;
-    u64 k[kRsIpt];
-    u32 v[kRsIpt], rank[kRsIpt];
-    int dg[kRsIpt];
+    long long wbase = (long long)blockIdx.x * (kRsThreads * IPT) + (long long)warp * 32 * IPT;
+    u64 k[IPT];
+    u32 v[IPT], rank[IPT];
+    int dg[IPT];
 #pragma unroll
-    for (int r = 0; r < kRsIpt; ++r) {
+    for (int r = 0; r < IPT; ++r) {
         long long idx = wbase + r * 32 + lane;
         bool valid = idx < n;
         k[r] = valid ? kin[idx] : 0ull;
-        v[r] = valid ? vin[idx] : 0u;
+        v[r] = !valid ? 0u : vin ? vin[idx] : (u32)idx;
         int d = valid ? (int)((k[r] >> shift) & 255u) : 256;
         dg[r] = d;
         unsigned peers = __match_any_sync(0xffffffffu, d);
@@ -212,7 +244,7 @@ __global__ void __launch_bounds__(kRsThreads) k_rs_scatter(const u64 *kin, const
     }
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < kRsIpt; ++r) {
+    for (int r = 0; r < IPT; ++r) {
         if (dg[r] < 256) {
             u32 pos = base[dg[r]] + wcnt[warp][dg[r]] + rank[r];
             kout[pos] = k[r];
@@ -221,110 +253,143 @@ __global__ void __launch_bounds__(kRsThreads) k_rs_scatter(const u64 *kin, const
     }
 }
 
-// One tile (n <= kRsTile): all eight passes in one block, the ranks as in
-// k_rs_scatter and the digit offsets from the block's own histogram; the
-// passes alternate between the caller's buffers and (tk, tv), global writes
-// made visible to the block by the barrier between passes.
-__global__ void __launch_bounds__(kRsThreads) k_rs_small(u64 *keys, u32 *vals, u64 *tk, u32 *tv,
-                                                         int n)
+// One pass over tiles of 4096 items for the allocation-free ordering, which
+// brings its own scratch.
+void rs_tile_hist(const u64 *keys, long long n, int shift, u32 *hist, int nblocks, cudaStream_t s)
 {
-    __shared__ u32 wcnt[kRsWarps][256];
-    __shared__ u32 base[256];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
-    const int wbase = warp * 32 * kRsIpt;
-    u64 *ka = keys, *kb = tk;
-    u32 *va = vals, *vb = tv;
-    for (int pass = 0; pass < 8; ++pass) {
-        const int shift = 8 * pass;
-        for (int i = threadIdx.x; i < kRsWarps * 256; i += kRsThreads) (&wcnt[0][0])[i] = 0;
-        __syncthreads();
-        u64 k[kRsIpt];
-        u32 v[kRsIpt], rank[kRsIpt];
-        int dg[kRsIpt];
-#pragma unroll
-        for (int r = 0; r < kRsIpt; ++r) {
-            const int idx = wbase + r * 32 + lane;
-            const bool valid = idx < n;
-            k[r] = valid ? ka[idx] : 0ull;
-            v[r] = valid ? va[idx] : 0u;
-            const int d = valid ? (int)((k[r] >> shift) & 255u) : 256;
-            dg[r] = d;
-            const unsigned peers = __match_any_sync(0xffffffffu, d);
-            const int leader = __ffs(peers) - 1;
-            const u32 before = valid ? wcnt[warp][d] : 0u;
-            __syncwarp();
-            if (valid && lane == leader) wcnt[warp][d] = before + __popc(peers);
-            __syncwarp();
-            rank[r] = before + __popc(peers & lt);
-        }
-        __syncthreads();
-        for (int d = threadIdx.x; d < 256; d += kRsThreads) {   // per digit: warps in order
-            u32 run = 0;
-            for (int w = 0; w < kRsWarps; ++w) {
-                const u32 t = wcnt[w][d];
-                wcnt[w][d] = run;
-                run += t;
-            }
-            base[d] = run;   // digit total, scanned below
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {   // exclusive scan of the 256 digit totals
-            u32 run = 0;
-            for (int d = 0; d < 256; ++d) {
-                const u32 t = base[d];
-                base[d] = run;
-                run += t;
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int r = 0; r < kRsIpt; ++r) {
-            if (dg[r] < 256) {
-                const u32 pos = base[dg[r]] + wcnt[warp][dg[r]] + rank[r];
-                kb[pos] = k[r];
-                vb[pos] = v[r];
-            }
-        }
-        __syncthreads();
-        u64 *t1 = ka; ka = kb; kb = t1;
-        u32 *t2 = va; va = vb; vb = t2;
-    }
-    // eight passes: the result is back in (keys, vals)
+    k_rs_hist<16><<<nblocks, kRsThreads, 0, s>>>(keys, n, shift, hist, nblocks);
 }
 
-// Sorts (keys, vals) in place by key, stably (equal keys keep their order).
-int radix_sort_pairs(start_ctx *c, u64 *keys, u32 *vals, long long n)
+void rs_tile_scatter(const u64 *kin, const u32 *vin, u64 *kout, u32 *vout, long long n, int shift,
+                     const u32 *offs, int nblocks, cudaStream_t s)
 {
-    if (n <= 1) return START_OK;
-    if (n <= kRsTile) {
-        ST_TRY(ensure(c->tk[0], n * sizeof(u64)));
-        ST_TRY(ensure(c->tv[0], n * sizeof(u32)));
-        k_rs_small<<<1, kRsThreads, 0, c->stream>>>(keys, vals, c->tk[0].as<u64>(),
-                                                    c->tv[0].as<u32>(), (int)n);
-        ++c->launches;
-        return cuda_check(c, cudaGetLastError(), "k_rs_small");
+    k_rs_scatter<16><<<nblocks, kRsThreads, 0, s>>>(kin, vin, kout, vout, n, shift, offs, nblocks);
+}
+
+// Sorting up to kRankSort keys by counting: the place of an item is the
+// number of keys below its own, and of equal keys before it.  A block places
+// 32 items, its eight warps counting an eighth of each staged tile of keys
+// (every lane reads the same key: a broadcast).  The count is n^2 comparisons,
+// but in one launch over the whole chip: 8 us at 2 k keys, where eight radix
+// passes by one block took 55 us; the four passes of a larger sort take 90 us
+// at 23 k keys.
+constexpr long long kRankSort = 16384;
+constexpr int kRankTile = 2048;
+
+__global__ void __launch_bounds__(256) k_rank_sort(const u64 *kin, int n, u64 *kout, u32 *perm)
+{
+    __shared__ __align__(16) u64 tile[kRankTile];
+    __shared__ u32 part[8][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + lane;
+    const u64 key = i < n ? kin[i] : 0ull;
+    u32 below = 0;
+    for (int t0 = 0; t0 < n; t0 += kRankTile) {
+        __syncthreads();
+        for (int j = threadIdx.x; j < kRankTile; j += 256)
+            tile[j] = t0 + j < n ? kin[t0 + j] : ~0ull;   // above every key
+        __syncthreads();
+        const int j0 = w * (kRankTile / 8);
+#pragma unroll 4
+        for (int j = 0; j < kRankTile / 8; j += 2) {
+            const ulonglong2 q = *reinterpret_cast<const ulonglong2 *>(&tile[j0 + j]);
+            const int g = t0 + j0 + j;
+            below += q.x < key || (q.x == key && g < i);
+            below += q.y < key || (q.y == key && g + 1 < i);
+        }
     }
-    int nblocks = (int)((n + kRsTile - 1) / kRsTile);
-    ST_TRY(ensure(c->tk[0], n * sizeof(u64)));
-    ST_TRY(ensure(c->tv[0], n * sizeof(u32)));
+    part[w][lane] = below;
+    __syncthreads();
+    if (w == 0 && i < n) {
+        u32 r = 0;
+        for (int k = 0; k < 8; ++k) r += part[k][lane];
+        kout[r] = key;
+        perm[r] = (u32)i;
+    }
+}
+
+// Completes an order by the leading kKeyHigh bits: each run of equal leading
+// bits is sorted by insertion (stable) by the thread at its first item; a run
+// of more than kRunMax items is counted in `longer` and left.
+constexpr int kKeyHigh = 32, kKeyLow = 3 * kLevels - kKeyHigh;
+constexpr int kRunMax = 32;
+
+__global__ void k_sort_runs(u64 *keys, u32 *vals, long long n, u32 *longer)
+{
+    const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k + 1 >= n) return;
+    const u64 p = keys[k] >> kKeyLow;
+    if ((keys[k + 1] >> kKeyLow) != p || (k > 0 && (keys[k - 1] >> kKeyLow) == p)) return;
+    int m = 2;
+    while (m <= kRunMax && k + m < n && (keys[k + m] >> kKeyLow) == p) ++m;
+    if (m > kRunMax) {
+        atomicAdd(longer, 1u);
+        return;
+    }
+    for (int a = 1; a < m; ++a) {
+        const u64 key = keys[k + a];
+        const u32 v = vals[k + a];
+        int b = a;
+        for (; b > 0 && keys[k + b - 1] > key; --b) {
+            keys[k + b] = keys[k + b - 1];
+            vals[k + b] = vals[k + b - 1];
+        }
+        keys[k + b] = key;
+        vals[k + b] = v;
+    }
+}
+
+template <int IPT>
+static int rs_pass(start_ctx *c, const u64 *ka, const u32 *va, u64 *kb, u32 *vb, long long n,
+                   int shift)
+{
+    const int nblocks = (int)((n + kRsThreads * IPT - 1) / (kRsThreads * IPT));
     ST_TRY(ensure(c->hist, (size_t)2 * 256 * nblocks * sizeof(u32)));
     u32 *hist = c->hist.as<u32>();
     u32 *offs = hist + (size_t)256 * nblocks;
-    u64 *ka = keys, *kb = c->tk[0].as<u64>();
-    u32 *va = vals, *vb = c->tv[0].as<u32>();
-    for (int pass = 0; pass < 8; ++pass) {
-        int shift = 8 * pass;
-        k_rs_hist<<<nblocks, kRsThreads, 0, c->stream>>>(ka, n, shift, hist, nblocks); ++c->launches;
-        ST_CUDA(c, cudaGetLastError());
-        ST_TRY(exclusive_scan_u32(c, hist, offs, (long long)256 * nblocks, nullptr));
-        k_rs_scatter<<<nblocks, kRsThreads, 0, c->stream>>>(ka, va, kb, vb, n, shift, offs, nblocks); ++c->launches;
-        ST_CUDA(c, cudaGetLastError());
-        u64 *tk = ka; ka = kb; kb = tk;
-        u32 *tv = va; va = vb; vb = tv;
+    k_rs_hist<IPT><<<nblocks, kRsThreads, 0, c->stream>>>(ka, n, shift, hist, nblocks);
+    ST_CUDA(c, cudaGetLastError());
+    ST_TRY(exclusive_scan_u32(c, hist, offs, (long long)256 * nblocks, nullptr));
+    k_rs_scatter<IPT><<<nblocks, kRsThreads, 0, c->stream>>>(ka, va, kb, vb, n, shift, offs,
+                                                             nblocks);
+    c->launches += 2;
+    return cuda_check(c, cudaGetLastError(), "k_rs_scatter");
+}
+
+// Sorted keys and the input index of every rank (stable: equal keys in input
+// order) of n keys in input order.  More than kRankSort keys: four radix passes
+// over the leading 32 bits, after which only particles within 2^-10.67 of the
+// box of each other share a run (sorted by insertion); runs that are too long
+// are counted in `longer`, which the caller cleared, and the caller sorts
+// again with all_bits: eight passes.
+int sort_keys(start_ctx *c, const u64 *keys, long long n, u64 *sorted, u32 *perm, bool all_bits,
+              u32 *longer)
+{
+    if (n <= 0) return START_OK;
+    if (n <= kRankSort) {
+        k_rank_sort<<<grid_for(n, 32), 256, 0, c->stream>>>(keys, (int)n, sorted, perm);
+        ++c->launches;
+        return cuda_check(c, cudaGetLastError(), "k_rank_sort");
     }
-    // 8 passes: the result is back in the caller's buffers
-    return START_OK;
+    ST_TRY(ensure(c->tk[0], n * sizeof(u64)));
+    ST_TRY(ensure(c->tv[0], n * sizeof(u32)));
+    u64 *tk = c->tk[0].as<u64>();
+    u32 *tv = c->tv[0].as<u32>();
+    const int first = all_bits ? 0 : kKeyLow;
+    for (int pass = 0, shift = first; shift < 3 * kLevels; ++pass, shift += 8) {
+        const u64 *ka = pass == 0 ? keys : (pass & 1 ? tk : sorted);
+        const u32 *va = pass == 0 ? nullptr : (pass & 1 ? tv : perm);
+        u64 *kb = pass & 1 ? sorted : tk;
+        u32 *vb = pass & 1 ? perm : tv;
+        ST_TRY(n < kRsSmallTiles ? rs_pass<4>(c, ka, va, kb, vb, n, shift)
+                                 : rs_pass<16>(c, ka, va, kb, vb, n, shift));
+    }
+    // four or eight passes: the result is in (sorted, perm)
+    if (!all_bits) {
+        k_sort_runs<<<grid_for(n, 256), 256, 0, c->stream>>>(sorted, perm, n, longer);
+        ++c->launches;
+    }
+    return cuda_check(c, cudaGetLastError(), "k_sort_runs");
 }
 
 // ---------------------------------------------------------------- frame
@@ -363,14 +428,21 @@ __global__ void k_bbox(const float *pos, long long n, int *mm, unsigned long lon
         }
     }
     for (int o = 16; o; o >>= 1) nbad += __shfl_xor_sync(0xffffffffu, nbad, o);
+    // one set of atomics per block
+    __shared__ int bound[6];
+    if (threadIdx.x < 6) bound[threadIdx.x] = threadIdx.x < 3 ? 0x7fffffff : (int)0x80000000;
+    __syncthreads();
     if ((threadIdx.x & 31) == 0) {
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            atomicMin(&mm[a], f2ord(lo[a]));
-            atomicMax(&mm[3 + a], f2ord(hi[a]));
+            atomicMin(&bound[a], f2ord(lo[a]));
+            atomicMax(&bound[3 + a], f2ord(hi[a]));
         }
         if (nbad) atomicAdd(bad, nbad);
     }
+    __syncthreads();
+    if (threadIdx.x < 3) atomicMin(&mm[threadIdx.x], bound[threadIdx.x]);
+    else if (threadIdx.x < 6) atomicMax(&mm[threadIdx.x], bound[threadIdx.x]);
 }
 
 // The root cube from the bounds mm: lower corner, largest extent (1 when it
@@ -422,7 +494,7 @@ __device__ __forceinline__ u64 spread3(u64 v)
     return v;
 }
 
-__global__ void k_morton(const float *pos, long long n, const FrameRec *fr, u64 *keys, u32 *idx)
+__global__ void k_morton(const float *pos, long long n, const FrameRec *fr, u64 *keys)
 {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -435,14 +507,12 @@ __global__ void k_morton(const float *pos, long long n, const FrameRec *fr, u64 
         q[a] = (u64)t;
     }
     keys[i] = (spread3(q[0]) << 2) | (spread3(q[1]) << 1) | spread3(q[2]);
-    if (idx) idx[i] = (u32)i;
 }
 
-int morton_keys(start_ctx *c, const float *pos_soa, long long n, const FrameRec *fr, u64 *keys,
-                u32 *idx)
+int morton_keys(start_ctx *c, const float *pos_soa, long long n, const FrameRec *fr, u64 *keys)
 {
     if (n <= 0) return START_OK;
-    k_morton<<<grid_for(n, 256), 256, 0, c->stream>>>(pos_soa, n, fr, keys, idx); ++c->launches;
+    k_morton<<<grid_for(n, 256), 256, 0, c->stream>>>(pos_soa, n, fr, keys); ++c->launches;
     return cuda_check(c, cudaGetLastError(), "k_morton");
 }
 
