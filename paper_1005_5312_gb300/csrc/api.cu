@@ -656,7 +656,7 @@ int start_build_trees(start_ctx *c, const float *pos, const float *h, long long 
     if (diffuse)
         ST_TRY(tree_emit(c, c->et, pks, n_p, one, frame, bn.hist[2], notes->hist[2],
                          notes->cursor[2], true));
-    ST_TRY(build_neighbours(c));
+    ST_TRY(build_neighbours(c, one, frame));
     phase_mark(c, START_PHASE_BUILD, true);
     ST_CUDA(c, cudaGetLastError());
     if (read_counter(c, C_INTERNAL)) return set_err(c, START_ECUDA, "internal inconsistency (trees or neighbour lists)");

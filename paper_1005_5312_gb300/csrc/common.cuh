@@ -316,7 +316,7 @@ int tree_moments(start_ctx *c, Tree &t, const float4 *mem_pos, const double *mem
 void tree_release(Tree &t);
 
 // neighbors.cu
-int build_neighbours(start_ctx *c);
+int build_neighbours(start_ctx *c, const Segs &segs, const FrameRec *frames);
 
 // density.cu
 int run_sph_density(start_ctx *c, const float *mass_dev, float *rho_dev);

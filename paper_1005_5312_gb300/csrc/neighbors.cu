@@ -2,14 +2,21 @@
 // RSPH upstream search of Section 2.2.1 chooses from), found through the
 // particle octree that Section 2.2.2 reuses from the gravity solver.
 //
-// One thread per target in Morton order walks the particle tree stacklessly
-// (pre-order index + skip pointer), so the 32 targets of a warp are spatial
-// neighbours and read the same cells.  Cells are visited by a conservative
-// FP32 distance test; members are accepted by the FP32-filtered exact test
-// with an FP64 fallback.  One walk counts the neighbours and keeps the first
-// kNbCap of them in a padded scratch; after the scan of the counts the rows
-// are copied into the CSR, and only targets with more neighbours than that
-// walk again to fill their rows.
+// A warp takes 32 targets in Morton order, spatial neighbours, and walks the
+// particle tree once for all of them: 32 consecutive cells of the pre-order at
+// a time, one per lane, are tested against the boxes around the spheres of the
+// targets' four octets, and the skip pointers of those outside tell which of
+// the 32 the walk reaches and where it goes on.  The members of the leaves it
+// reaches are read one per lane, those inside a box are staged, and every lane
+// tests its own target against each staged member (a broadcast read), first
+// without branches into a bit mask, then its few candidates by the FP32-filtered
+// exact test with an FP64 fallback.  The walk keeps the first kNbCap neighbours
+// per target; after the scan of the counts the rows are copied into the CSR,
+// and only targets with more neighbours than that walk again, a thread each, to
+// fill their rows.  (One walk per thread for every target, a chain of dependent
+// cell and member reads: 1570 us at 2^20 particles, 157 us at 2 k, where it
+// left most of the chip idle, against 1266 and 54 us; staging each octet's
+// members apart makes the tests fewer but the staging dearer: 1617 us.)
 #include "common.cuh"
 
 namespace st {
@@ -33,91 +40,293 @@ __device__ __forceinline__ bool member_in(float4 pk, float4 pi, float two_h, dou
 }
 
 constexpr u32 kNbCap = 48;   // neighbours kept per target by the counting walk
+constexpr int kNbWarps = 4;
+// an octet of targets whose box is wider than this many times their largest
+// reach straddles a jump of the Morton curve (eight lattice neighbours span
+// three): its group tests the cells against each target's own sphere
+constexpr float kNbWide = 6.f;
 
-// FILL = false: count into cnt[i] and keep the first kNbCap in scratch[i *
-// kNbCap ..], counting the targets that have more into n_over.  FILL = true:
-// write the rows of the targets listed in only[0, n) (all when NULL) at off.
-template <bool FILL>
-__global__ void __launch_bounds__(128) k_neighbours(const float4 *pq, const float *h, long long np,
-                                                    const float4 *box, const uint4 *meta,
-                                                    long long nn, float cmag, u32 *cnt,
-                                                    const u32 *off, u32 *idx,
-                                                    unsigned long long *fb_total, u32 *scratch,
-                                                    unsigned long long *n_over, const u32 *only)
+// Squared distance from p to a cell's cube (FP32, rounded to nearest).
+__device__ __forceinline__ float cell_d2(float4 b, float px, float py, float pz)
 {
-    long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    float dx = fmaxf(fmaxf(__fsub_rn(b.x, px), __fsub_rn(px, __fadd_rn(b.x, b.w))), 0.f);
+    float dy = fmaxf(fmaxf(__fsub_rn(b.y, py), __fsub_rn(py, __fadd_rn(b.y, b.w))), 0.f);
+    float dz = fmaxf(fmaxf(__fsub_rn(b.z, pz), __fsub_rn(pz, __fadd_rn(b.z, b.w))), 0.f);
+    return __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
+}
+
+// Reach of a target's sphere in FP32 tests of cells: 2 h and the rounding of
+// the cubes' corners.
+__device__ __forceinline__ float nb_reach(float two_h, float cmag)
+{
+    return __fadd_rn(__fmul_rn(two_h, 1.f + 1e-5f), __fmul_rn(16.f * kU32, cmag));
+}
+
+// The staged members [0, 32) against the lane's target: its neighbours among
+// them, in order, to its list.  thr: a little above (2 h)^2.
+__device__ __forceinline__ void nb_take(const float4 *buf, float4 pi, float two_h, double two_h64,
+                                        float thr, u32 self, u32 (*list)[33], int lane, u32 &c,
+                                        unsigned &fb)
+{
+    u32 m = 0;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+        const float4 p = buf[k];
+        const float ax = p.x - pi.x, ay = p.y - pi.y, az = p.z - pi.z;
+        if (ax * ax + ay * ay + az * az < thr) m |= 1u << k;
+    }
+    while (m) {
+        const float4 p = buf[__ffs(m) - 1];
+        m &= m - 1u;
+        const u32 r = __float_as_uint(p.w);
+        if (r != self && member_in(p, pi, two_h, two_h64, fb)) {
+            if (c < kNbCap) list[c][lane] = r;
+            ++c;
+        }
+    }
+}
+
+// Counts every target's neighbours into cnt[i] and keeps the first kNbCap in
+// scratch[i kNbCap ..], in Morton order; n_over counts the targets with more.
+// cells: the first cell of every key (the cells of problem b of a batch are
+// [cells[start b], cells[start b + 1])).
+__global__ void __launch_bounds__(32 * kNbWarps)
+k_neighbours(const float4 *pq, const float *h, long long np, const float4 *box, const uint4 *meta,
+             Segs segs, const u32 *cells, const FrameRec *frames, u32 *cnt,
+             unsigned long long *fb_total, u32 *scratch, unsigned long long *n_over)
+{
+    __shared__ float4 buf[kNbWarps][64];      // staged members: position, index
+    __shared__ float4 sphere[kNbWarps][32];   // the targets' positions and squared reaches
+    __shared__ float4 oct[kNbWarps][4][2];    // the octets' boxes: lower, upper corner
+    __shared__ u32 list[kNbWarps][kNbCap][33];
+    const float4 far = make_float4(1e30f, 1e30f, 1e30f, 0.f);   // no target's neighbour
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const long long i0 = ((long long)blockIdx.x * kNbWarps + w) * 32;
+    if (i0 >= np) return;   // warp-uniform
+    const long long i = i0 + lane;
+    const bool live = i < np;
+    float4 pi = make_float4(0.f, 0.f, 0.f, 0.f);
+    float two_h = 0.f;
+    double two_h64 = 0.0;
+    u32 s0 = 0u, s1 = (u32)np, prob = 0xffffffffu;
+    if (live) {
+        pi = pq[i];
+        two_h = __fmul_rn(2.f, h[i]);
+        two_h64 = 2.0 * (double)h[i];
+        prob = segs.range((u32)i, s0, s1);
+    }
+    u32 c = 0;
     unsigned fb = 0;
-    if (t < np) {
-        const long long i = only ? (long long)only[t] : t;
-        float4 pi = pq[i];
-        float two_h = __fmul_rn(2.f, h[i]);
-        double two_h64 = 2.0 * (double)h[i];
-        float reach = __fadd_rn(__fmul_rn(two_h, 1.f + 1e-5f), __fmul_rn(16.f * kU32, cmag));
-        float reach2 = __fmul_rn(reach, reach);
-        u32 c = 0, w = FILL ? off[i] : 0u;
-        const u32 wend = FILL ? off[i + 1] : 0u;
-        u32 n = 0;
-        while (n < (u32)nn) {
-            float4 b = box[n];
-            uint4 mt = meta[n];
-            float l = b.w;
-            float dx = fmaxf(fmaxf(__fsub_rn(b.x, pi.x), __fsub_rn(pi.x, __fadd_rn(b.x, l))), 0.f);
-            float dy = fmaxf(fmaxf(__fsub_rn(b.y, pi.y), __fsub_rn(pi.y, __fadd_rn(b.y, l))), 0.f);
-            float dz = fmaxf(fmaxf(__fsub_rn(b.z, pi.z), __fsub_rn(pi.z, __fadd_rn(b.z, l))), 0.f);
-            float bd2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
-            if (bd2 > reach2) {
-                n = mt.x;
-                continue;
+    unsigned todo = __ballot_sync(0xffffffffu, live);
+    while (todo) {   // the problems of the group's targets (nearly always one)
+        const int lead = __ffs(todo) - 1;
+        const u32 pb = __shfl_sync(0xffffffffu, prob, lead);
+        const bool mine = live && prob == pb;
+        todo &= ~__ballot_sync(0xffffffffu, mine);
+        const u32 n1 = cells[__shfl_sync(0xffffffffu, s1, lead)];
+        const float reach = nb_reach(two_h, frames[pb].cmag);
+        const float inf = __int_as_float(0x7f800000);
+        float lo[3] = {mine ? __fsub_rn(pi.x, reach) : inf, mine ? __fsub_rn(pi.y, reach) : inf,
+                       mine ? __fsub_rn(pi.z, reach) : inf};
+        float hi[3] = {mine ? __fadd_rn(pi.x, reach) : -inf, mine ? __fadd_rn(pi.y, reach) : -inf,
+                       mine ? __fadd_rn(pi.z, reach) : -inf};
+        float rmax = mine ? reach : 0.f;
+        for (int o = 4; o; o >>= 1) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                lo[a] = fminf(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
+                hi[a] = fmaxf(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], o));
             }
-            if (mt.w) {
-                for (u32 r = mt.y; r < mt.y + mt.z; ++r) {
-                    if (r == (u32)i) continue;
-                    if (member_in(pq[r], pi, two_h, two_h64, fb)) {
-                        if (FILL) {
-                            if (w < wend) idx[w] = r;   // never past this row
-                            ++w;
-                        } else {
-                            if (c < kNbCap) scratch[(size_t)i * kNbCap + c] = r;
-                            ++c;
-                        }
+            rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
+        }
+        const bool wide = __any_sync(
+            0xffffffffu,
+            fmaxf(fmaxf(hi[0] - lo[0], hi[1] - lo[1]), hi[2] - lo[2]) > kNbWide * rmax);
+        __syncwarp();
+        if ((lane & 7) == 0) {
+            oct[w][lane >> 3][0] = make_float4(lo[0], lo[1], lo[2], 0.f);
+            oct[w][lane >> 3][1] = make_float4(hi[0], hi[1], hi[2], 0.f);
+        }
+        sphere[w][lane] = make_float4(pi.x, pi.y, pi.z, mine ? __fmul_rn(reach, reach) : -1.f);
+        __syncwarp();
+        // 1e-5: far above the rounding of the FP32 distance, so that no
+        // neighbour is left out of the mask
+        const float thr = mine ? two_h * two_h * (1.f + 1e-5f) + 1e-36f : -1.f;
+        int staged = 0;
+        u32 base = cells[__shfl_sync(0xffffffffu, s0, lead)];
+        while (base < n1) {   // 32 cells of the pre-order, one per lane
+            const u32 n = base + lane;
+            const bool in = n < n1;
+            uint4 mt = make_uint4(n + 1, 0u, 0u, 0u);
+            bool hit = false;
+            if (in) {
+                const float4 b = box[n];
+                mt = meta[n];
+                const float bx = __fadd_rn(b.x, b.w), by = __fadd_rn(b.y, b.w),
+                            bz = __fadd_rn(b.z, b.w);
+#pragma unroll
+                for (int g = 0; g < 4; ++g) {
+                    const float4 l = oct[w][g][0], u = oct[w][g][1];
+                    hit = hit || (b.x <= u.x && bx >= l.x && b.y <= u.y && by >= l.y &&
+                                  b.z <= u.z && bz >= l.z);
+                }
+                if (wide && hit) {
+                    hit = false;
+                    for (int t = 0; t < 32 && !hit; ++t) {
+                        const float4 p = sphere[w][t];
+                        hit = cell_d2(b, p.x, p.y, p.z) <= p.w;
                     }
                 }
-                n = mt.x;
-            } else {
-                n = n + 1;
+            }
+            // cells inside the subtree of one that is not hit are not reached
+            const u32 skip = mt.x - base;   // first lane after this cell's subtree
+            const bool out = in && !hit;
+            const unsigned upto = skip >= 32u ? 0xffffffffu : (1u << skip) - 1u;
+            const unsigned from = lane == 31 ? 0u : 0xffffffffu << (lane + 1);
+            const unsigned unreached = __reduce_or_sync(0xffffffffu, out ? upto & from : 0u);
+            const u32 next = __reduce_max_sync(0xffffffffu, out ? mt.x : 0u);
+            const bool leaf = hit && mt.w && !((unreached >> lane) & 1u);
+            base = max(base + 32u, next);
+            // the members of the leaves reached, in order
+            const u32 m = leaf ? mt.z : 0u;
+            u32 end = m;
+            for (int o = 1; o < 32; o <<= 1) {
+                const u32 y = __shfl_up_sync(0xffffffffu, end, o);
+                if (lane >= o) end += y;
+            }
+            const u32 total = __shfl_sync(0xffffffffu, end, 31);
+            for (u32 q0 = 0; q0 < total; q0 += 32) {
+                const u32 q = q0 + lane;
+                int src = 0;   // the lane whose leaf holds candidate q: the first with end > q
+                for (int o = 16; o; o >>= 1) {
+                    const u32 e = __shfl_sync(0xffffffffu, end, src + o - 1);
+                    if (e <= q) src += o;
+                }
+                src = min(src, 31);
+                const u32 first = __shfl_sync(0xffffffffu, mt.y, src);
+                const u32 e = __shfl_sync(0xffffffffu, end, src);
+                const u32 len = __shfl_sync(0xffffffffu, m, src);
+                float4 p = far;
+                bool near = false;
+                if (q < total) {
+                    const u32 r = first + (q - (e - len));
+                    p = pq[r];
+                    p.w = __uint_as_float(r);
+                    near = wide;
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) {
+                        const float4 l = oct[w][g][0], u = oct[w][g][1];
+                        near = near || (p.x <= u.x && p.x >= l.x && p.y <= u.y && p.y >= l.y &&
+                                        p.z <= u.z && p.z >= l.z);
+                    }
+                }
+                const unsigned nm = __ballot_sync(0xffffffffu, near);
+                if (near) buf[w][staged + __popc(nm & ((1u << lane) - 1u))] = p;
+                staged += __popc(nm);
+                __syncwarp();
+                if (staged >= 32) {
+                    nb_take(buf[w], pi, two_h, two_h64, thr, (u32)i, list[w], lane, c, fb);
+                    __syncwarp();
+                    staged -= 32;
+                    if (lane < staged) buf[w][lane] = buf[w][32 + lane];
+                    __syncwarp();
+                }
             }
         }
-        if (!FILL) {
-            cnt[i] = c;
-            if (c > kNbCap) atomicAdd(n_over, 1ull);
-        } else if (w != wend) {
-            atomicAdd(fb_total, 1ull);   // internal-error counter in FILL
+        if (staged) {
+            if (lane >= staged) buf[w][lane] = far;
+            __syncwarp();
+            nb_take(buf[w], pi, two_h, two_h64, thr, (u32)i, list[w], lane, c, fb);
+            __syncwarp();
         }
     }
-    if (!FILL) {
-        for (int o = 16; o; o >>= 1) fb += __shfl_xor_sync(0xffffffffu, fb, o);
-        if ((threadIdx.x & 31) == 0 && fb) atomicAdd(fb_total, (unsigned long long)fb);
+    if (live) cnt[i] = c;
+    __syncwarp();
+    // the rows, one after the other, lanes along the row
+    const int rows = (int)min(32ll, np - i0);
+    for (int t = 0; t < rows; ++t) {
+        const u32 m = min(kNbCap, __shfl_sync(0xffffffffu, c, t));
+        for (u32 k = lane; k < m; k += 32) scratch[(size_t)(i0 + t) * kNbCap + k] = list[w][k][t];
+    }
+    const unsigned over = __ballot_sync(0xffffffffu, live && c > kNbCap);
+    for (int o = 16; o; o >>= 1) fb += __shfl_xor_sync(0xffffffffu, fb, o);
+    if (lane == 0) {
+        if (over) atomicAdd(n_over, (unsigned long long)__popc(over));
+        if (fb) atomicAdd(fb_total, (unsigned long long)fb);
     }
 }
 
-// Rows of at most kNbCap neighbours copied from the scratch into the CSR, one
-// warp per target; the others are listed for the filling walk.
-__global__ void k_nb_compact(long long np, const u32 *cnt, const u32 *off, const u32 *scratch,
-                             u32 *idx, u32 *over, unsigned long long *n_over)
+// The rows of the targets listed in only[0, n), a thread each.
+__global__ void __launch_bounds__(128) k_nb_fill(const float4 *pq, const float *h, long long n_only,
+                                                 long long np, const float4 *box,
+                                                 const uint4 *meta, Segs segs, const u32 *cells,
+                                                 const FrameRec *frames, const u32 *off, u32 *idx,
+                                                 unsigned long long *bad, const u32 *only)
 {
-    long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / 32;
-    int lane = threadIdx.x & 31;
-    if (i >= np) return;
-    u32 c = cnt[i];
-    if (c > kNbCap) {
-        if (lane == 0) over[atomicAdd(n_over, 1ull)] = (u32)i;
-        return;
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n_only) return;
+    const u32 i = only[t];
+    u32 s0 = 0u, s1 = (u32)np;
+    const u32 prob = segs.range(i, s0, s1);
+    const float4 pi = pq[i];
+    const float two_h = __fmul_rn(2.f, h[i]);
+    const double two_h64 = 2.0 * (double)h[i];
+    const float reach = nb_reach(two_h, frames[prob].cmag);
+    const float reach2 = __fmul_rn(reach, reach);
+    unsigned fb = 0;
+    u32 w = off[i];
+    const u32 wend = off[i + 1], n1 = cells[s1];
+    for (u32 n = cells[s0]; n < n1;) {
+        const uint4 mt = meta[n];
+        if (cell_d2(box[n], pi.x, pi.y, pi.z) > reach2) {
+            n = mt.x;
+            continue;
+        }
+        if (mt.w)
+            for (u32 r = mt.y; r < mt.y + mt.z; ++r)
+                if (r != i && member_in(pq[r], pi, two_h, two_h64, fb)) {
+                    if (w < wend) idx[w] = r;   // never past this row
+                    ++w;
+                }
+        n = mt.w ? mt.x : n + 1;
     }
-    u32 o = off[i];
-    for (u32 k = lane; k < c; k += 32) idx[o + k] = scratch[(size_t)i * kNbCap + k];
+    if (w != wend) atomicAdd(bad, 1ull);   // the counting walk's row
 }
 
-int build_neighbours(start_ctx *c)
+// Rows of at most kNbCap neighbours copied from the scratch into the CSR,
+// gridDim.y warps for the 32 consecutive rows of a group: lanes along the
+// output, which the rows share (a warp per row spent most of its time on the
+// latency of one 32-entry copy: 199 us at 2^20 particles, against 89 us).  The
+// others are listed for the filling walk.
+__global__ void __launch_bounds__(256) k_nb_compact(long long np, const u32 *cnt, const u32 *off,
+                                                    const u32 *__restrict__ scratch,
+                                                    u32 *__restrict__ idx, u32 *over,
+                                                    unsigned long long *n_over)
+{
+    const long long i0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / 32 * 32;
+    const int lane = threadIdx.x & 31;
+    if (i0 >= np) return;
+    const long long i = i0 + lane;
+    const u32 c = i < np ? cnt[i] : 0u;
+    const u32 o = off[i < np ? i : np];
+    if (c > kNbCap && blockIdx.y == 0) over[atomicAdd(n_over, 1ull)] = (u32)i;
+    const unsigned longer = __ballot_sync(0xffffffffu, c > kNbCap);
+    const u32 e0 = __shfl_sync(0xffffffffu, o, 0), e1 = off[min(i0 + 32, np)];
+#pragma unroll 4
+    for (u32 e = e0 + 32u * blockIdx.y; e < e1; e += 32u * gridDim.y) {
+        const u32 q = e + lane;
+        int src = 0;   // the last row that starts at or before entry q
+        for (int k = 16; k; k >>= 1) {
+            const u32 s = __shfl_sync(0xffffffffu, o, src + k);
+            if (s <= q) src += k;
+        }
+        const u32 s = __shfl_sync(0xffffffffu, o, src);
+        if (q < e1 && !((longer >> src) & 1u)) idx[q] = scratch[(size_t)(i0 + src) * kNbCap + (q - s)];
+    }
+}
+
+// frames: the problems' root cubes (device).
+int build_neighbours(start_ctx *c, const Segs &segs, const FrameRec *frames)
 {
     long long np = c->np;
     c->nb_total = 0;
@@ -139,10 +348,10 @@ int build_neighbours(start_ctx *c)
     unsigned long long *n_over = ctr + C_NB_OVER;
     ST_CUDA(c, cudaMemsetAsync(n_over, 0, sizeof(unsigned long long), c->stream));
     const Tree &t = c->pt;
-    k_neighbours<false><<<grid_for(np, 128), 128, 0, c->stream>>>(
-        c->pq.as<float4>(), c->ph.as<float>(), np, t.box.as<float4>(), t.meta.as<uint4>(), t.n,
-        c->fr.cmag, c->lcount.as<u32>(), nullptr, nullptr, fb, scratch.as<u32>(), n_over,
-        nullptr); ++c->launches;
+    k_neighbours<<<grid_for(np, 32 * kNbWarps), 32 * kNbWarps, 0, c->stream>>>(
+        c->pq.as<float4>(), c->ph.as<float>(), np, t.box.as<float4>(), t.meta.as<uint4>(), segs,
+        t.pos.as<u32>(), frames, c->lcount.as<u32>(), fb, scratch.as<u32>(), n_over);
+    ++c->launches;
     ST_CUDA(c, cudaGetLastError());
     // offsets in u64 first to detect overflow of the u32 CSR
     ST_TRY(ensure(c->loff, (np + 1) * sizeof(u64)));
@@ -159,14 +368,17 @@ int build_neighbours(start_ctx *c)
     if (over && ensure(olist, over * sizeof(u32)))
         return set_err(c, START_ENOMEM, "out of device memory (neighbour lists)");
     ST_CUDA(c, cudaMemsetAsync(n_over, 0, sizeof(unsigned long long), c->stream));
-    k_nb_compact<<<grid_for(np * 32, 256), 256, 0, c->stream>>>(
+    // four warps per group where the groups alone leave SMs idle (7 against 20 us
+    // at 2 k), one where they do not (89 against 131 us at 2^20)
+    k_nb_compact<<<dim3(grid_for(np, 256), np < (1 << 18) ? 4 : 1), 256, 0, c->stream>>>(
         np, c->lcount.as<u32>(), c->nb_off.as<u32>(), scratch.as<u32>(), c->nb_idx.as<u32>(),
-        over ? olist.as<u32>() : nullptr, n_over); ++c->launches;
+        over ? olist.as<u32>() : nullptr, n_over);
+    ++c->launches;
     if (over) {
-        k_neighbours<true><<<grid_for((long long)over, 128), 128, 0, c->stream>>>(
-            c->pq.as<float4>(), c->ph.as<float>(), (long long)over, t.box.as<float4>(),
-            t.meta.as<uint4>(), t.n, c->fr.cmag, nullptr, c->nb_off.as<u32>(),
-            c->nb_idx.as<u32>(), ctr + C_INTERNAL, nullptr, nullptr, olist.as<u32>());
+        k_nb_fill<<<grid_for((long long)over, 128), 128, 0, c->stream>>>(
+            c->pq.as<float4>(), c->ph.as<float>(), (long long)over, np, t.box.as<float4>(),
+            t.meta.as<uint4>(), segs, t.pos.as<u32>(), frames, c->nb_off.as<u32>(),
+            c->nb_idx.as<u32>(), ctr + C_INTERNAL, olist.as<u32>());
         ++c->launches;
     }
     ST_CUDA(c, cudaGetLastError());
