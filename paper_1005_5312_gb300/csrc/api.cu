@@ -225,7 +225,7 @@ __global__ void k_scatter_d(const double *in, const u32 *inv, long long n, doubl
 }
 
 // Morton-ordered particle records from the staged SoA inputs.
-__global__ void k_gather_particles(const float *pos, const float *h, const double *V,
+__global__ void k_gather_particles(const float *pos, Segs segs, const float *h, const double *V,
                                    const u32 *perm, long long n, float4 *pq, float *ph,
                                    double *Vm, float *nH, double *y, float *gam, u32 *inv,
                                    double *eL, float *eLs, double *Tg)
@@ -233,7 +233,10 @@ __global__ void k_gather_particles(const float *pos, const float *h, const doubl
     long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
     u32 i = perm[r];
-    pq[r] = make_float4(pos[i], pos[n + i], pos[2 * n + i], 0.f);
+    u32 lo = 0u, hi = (u32)n;
+    segs.range(i, lo, hi);
+    pq[r] = make_float4(pos[point_index(lo, hi, i, 0)], pos[point_index(lo, hi, i, 1)],
+                        pos[point_index(lo, hi, i, 2)], 0.f);
     ph[r] = h[i];
     if (V) Vm[r] = V[i];
     else Vm[r] = 0.0;
@@ -246,15 +249,17 @@ __global__ void k_gather_particles(const float *pos, const float *h, const doubl
     Tg[r] = 1e4;
 }
 
-__global__ void k_gather_sources(const float *pos, const double *L, const u32 *perm, long long n,
-                                 double L_unit, float4 *sq, double *sL)
+__global__ void k_gather_sources(const float *pos, Segs segs, const double *L, const u32 *perm,
+                                 long long n, double L_unit, float4 *sq, double *sL)
 {
     long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
     u32 i = perm[r];
     double Lj = L[i];
-    sq[r] = make_float4(pos[i], pos[n + i], pos[2 * n + i],
-                        __double2float_rn(__ddiv_rn(Lj, L_unit)));
+    u32 lo = 0u, hi = (u32)n;
+    segs.range(i, lo, hi);
+    sq[r] = make_float4(pos[point_index(lo, hi, i, 0)], pos[point_index(lo, hi, i, 1)],
+                        pos[point_index(lo, hi, i, 2)], __double2float_rn(__ddiv_rn(Lj, L_unit)));
     sL[r] = Lj;
 }
 
@@ -323,60 +328,25 @@ static void csr_to_input(long long n, const std::vector<O> &moff, const std::vec
 }
 
 // ---------------------------------------------------------------- batches
-// Merging one problem's structures into a batch's forest: plain copies, and
-// index arrays shifted by the problem's offsets (kNone kept).
-__global__ void k_shift_u32(const u32 *in, long long n, u32 add, u32 *out)
+// What a solve needs per target of a batch: the cells of its own source tree
+// and its problem's squared dilution floor.
+__global__ void k_batch_targets(long long np, Segs psegs, Segs ssegs, long long ns,
+                                const u32 *scells, const FrameRec *frames, uint2 *tr, float *rf2)
 {
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = in[i] == 0xffffffffu ? 0xffffffffu : in[i] + add;   // "none" kept
-}
-
-__global__ void k_shift_meta(const uint4 *in, long long n, u32 node0, u32 memb0, uint4 *out)
-{
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) {
-        uint4 m = in[i];
-        out[i] = make_uint4(m.x + node0, m.y + memb0, m.z, m.w);
-    }
-}
-
-__global__ void k_fill_range(uint2 *tr, float *rf2, long long n, uint2 r, float f)
-{
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) {
-        tr[i] = r;
-        rf2[i] = f;
-    }
-}
-
-extern "C" int start_destroy(start_ctx *c);
-
-int destroy_batch_parts(start_ctx *c)
-{
-    for (start_ctx *b : c->bsub) start_destroy(b);
-    c->bsub.clear();
-    return START_OK;
-}
-
-static int copy_dev(start_ctx *c, void *dst, const void *src, size_t bytes)
-{
-    if (!bytes) return START_OK;
-    return cuda_check(c, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToDevice, c->stream),
-                      "batch copy");
-}
-
-static int shift_copy(start_ctx *c, u32 *dst, const u32 *src, long long n, u32 add)
-{
-    if (n <= 0) return START_OK;
-    k_shift_u32<<<grid_for(n, 256), 256, 0, c->stream>>>(src, n, add, dst);
-    ++c->launches;
-    return cuda_check(c, cudaGetLastError(), "k_shift_u32");
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= np) return;
+    u32 lo = 0u, hi = (u32)np;
+    const u32 b = psegs.range((u32)i, lo, hi);
+    const u32 s0 = ssegs.n > 1 ? ssegs.start[b] : 0u;
+    const u32 s1 = ssegs.n > 1 ? ssegs.start[b + 1] : (u32)ns;
+    tr[i] = ns ? make_uint2(scells[s0], scells[s1]) : make_uint2(0u, 0u);
+    const double rf = 1e-6 * frames[b].side;
+    rf2[i] = (float)(rf * rf);
 }
 
 static void release_all(start_ctx *c)
 {
     c->rb_n = c->rb_geo_n = 0;
-    destroy_batch_parts(c);
     resident_reset(c);
     if (c->r_cap) cudaStreamDestroy(c->r_cap);
     c->r_cap = nullptr;
@@ -389,7 +359,8 @@ static void release_all(start_ctx *c)
                    &c->r_j, &c->r_up, &c->r_dl, &c->r_next, &c->r_tau, &c->r_pos, &c->r_lvl, &c->r_vid,
                    &c->m_st[0], &c->m_st[1], &c->m_ups, &c->m_fr, &c->m_hard, &c->m_part, &c->m_table,
                    &c->w_scratch, &c->w_over, &c->ctr_save, &c->g_hist, &c->gacc, &c->klum_big, &c->trange, &c->trf2,
-                   &c->rb_mask, &c->rb_geo, &c->rb_amax, &c->m_w[0], &c->m_w[1]};
+                   &c->rb_mask, &c->rb_geo, &c->rb_amax, &c->m_w[0], &c->m_w[1],
+                   &c->seg, &c->frames, &c->bounds, &c->Tg};
     for (DBuf *b : all) release(*b);
     tree_release(c->pt);
     tree_release(c->stree);
@@ -413,11 +384,20 @@ using namespace st;
 namespace {
 // What a build leaves on the device for the host to read.
 struct BuildNotes {
-    FrameRec frame;
     unsigned long long hist[3][kLevels + 1];   // cells per level: particles, sources, emitters
     u32 cursor[3][kLevels + 1];
     u32 long_runs;   // runs of equal leading key bits that the sort left
-    int bounds[8];
+};
+
+// The problems of a build: sizes and arrays (host or device), and the bounds
+// of their particles and sources in the stacked arrays.
+struct Problems {
+    int n;
+    const long long *n_p, *n_s;
+    const float *const *pos, *const *h, *const *src_pos;
+    const double *const *src_L;
+    const double *V;   // diffuse (one problem)
+    std::vector<u32> p0, s0;
 };
 
 struct Staged {
@@ -540,6 +520,191 @@ int start_destroy(start_ctx *c)
     return START_OK;
 }
 
+// Validation of staged inputs: the counts of bad values land in C_BAD_INPUT.
+static int check_inputs(start_ctx *c, const float *h, long long n_p, const double *L,
+                        long long n_s, const double *V)
+{
+    unsigned long long *bad = c->counters.as<unsigned long long>() + C_BAD_INPUT;
+    cudaStream_t s = c->stream;
+    if (n_p) { k_check_pos_h<<<grid_for(n_p, 256), 256, 0, s>>>(h, n_p, bad); ++c->launches; }
+    if (n_s) { k_check_nonneg_d<<<grid_for(n_s, 256), 256, 0, s>>>(L, n_s, bad, 0); ++c->launches; }
+    if (V && n_p) { k_check_nonneg_d<<<grid_for(n_p, 256), 256, 0, s>>>(V, n_p, bad, 1); ++c->launches; }
+    return cuda_check(c, cudaGetLastError(), "k_check");
+}
+
+// Names the first problem of a batch whose staged inputs are bad (error path).
+static int bad_problem(start_ctx *c, const Problems &q, const Staged &in, bool batch)
+{
+    unsigned long long *ctr = c->counters.as<unsigned long long>();
+    int code = START_EINVAL;
+    for (int b = 0; b < q.n; ++b) {
+        ST_CUDA(c, cudaMemsetAsync(ctr, 0, C_COUNT * sizeof(unsigned long long), c->stream));
+        const u32 p = q.p0[b], s = q.s0[b];
+        ST_TRY(check_inputs(c, in.h.as<float>() + p, q.n_p[b], in.L.as<double>() + s, q.n_s[b],
+                            q.V ? in.V.as<double>() : nullptr));
+        ST_TRY(compute_frames(c, in.pos.as<float>() + 3 * (size_t)p, q.n_p[b], Segs{},
+                              in.spos.as<float>() + 3 * (size_t)s, q.n_s[b], Segs{},
+                              c->bounds.as<int>(), c->frames.as<FrameRec>()));
+        const bool val = read_counter(c, C_BAD_INPUT) != 0;
+        if (val || read_counter(c, C_BAD_POS)) {
+            const std::string what = val ? "invalid values in h, src_L or V"
+                                         : "non-finite particle or source position";
+            code = set_err(c, START_EINVAL,
+                           batch ? "batch part " + std::to_string(b) + ": " + what : what);
+            break;
+        }
+    }
+    ST_CUDA(c, cudaMemsetAsync(ctr, 0, C_COUNT * sizeof(unsigned long long), c->stream));
+    return code;
+}
+
+// Frames, keys, sorts, trees and neighbour lists of one problem or a batch: the
+// problems are stacked, and every pass runs once over all of them (a batch of
+// sixteen 6 k problems built one after the other took 6.6 ms of launches and
+// waits that no problem fills the GPU with, against 1.0 ms).
+static int build_problems(start_ctx *c, Problems &q, bool diffuse, bool batch)
+{
+    cudaStream_t s = c->stream;
+    unsigned long long *ctr = c->counters.as<unsigned long long>();
+    const long long n_p = c->np, n_s = c->ns;
+    q.p0.assign(q.n + 1, 0u);
+    q.s0.assign(q.n + 1, 0u);
+    Segs ps, ss;
+    ps.n = ss.n = q.n;
+    ps.trees = ss.trees = 0;
+    for (int b = 0; b < q.n; ++b) {
+        q.p0[b + 1] = q.p0[b] + (u32)q.n_p[b];
+        q.s0[b + 1] = q.s0[b] + (u32)q.n_s[b];
+        ps.trees += q.n_p[b] > 0;
+        ss.trees += q.n_s[b] > 0;
+    }
+    ST_CUDA(c, cudaMemsetAsync(ctr, 0, C_COUNT * sizeof(unsigned long long), s));
+    phase_mark(c, START_PHASE_BUILD, false);
+    Staged in;
+    if (ensure(in.pos, 3 * n_p * sizeof(float)) || ensure(in.h, n_p * sizeof(float)) ||
+        ensure(in.spos, 3 * n_s * sizeof(float)) || ensure(in.L, n_s * sizeof(double)) ||
+        (diffuse && ensure(in.V, n_p * sizeof(double))))
+        return set_err(c, START_ENOMEM, "out of device memory (inputs)");
+    auto put = [&](void *dst, const void *src, size_t bytes) {
+        return bytes ? cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, s) : cudaSuccess;
+    };
+    for (int b = 0; b < q.n; ++b) {
+        const size_t p = q.p0[b], t = q.s0[b], m = (size_t)q.n_p[b], k = (size_t)q.n_s[b];
+        ST_CUDA(c, put(in.pos.as<float>() + 3 * p, q.pos[b], 3 * m * sizeof(float)));
+        ST_CUDA(c, put(in.h.as<float>() + p, q.h[b], m * sizeof(float)));
+        ST_CUDA(c, put(in.spos.as<float>() + 3 * t, q.src_pos[b], 3 * k * sizeof(float)));
+        ST_CUDA(c, put(in.L.as<double>() + t, q.src_L[b], k * sizeof(double)));
+    }
+    if (diffuse) ST_CUDA(c, put(in.V.p, q.V, n_p * sizeof(double)));
+    ST_TRY(check_inputs(c, in.h.as<float>(), n_p, in.L.as<double>(), n_s,
+                        diffuse ? in.V.as<double>() : nullptr));
+    if (n_p + n_s == 0 && !batch) {
+        c->pt.n = c->stree.n = c->et.n = 0;
+        c->nb_total = 0;
+        c->built = true;
+        return START_OK;
+    }
+    // the device's notes of a build: cells per level of the three trees and
+    // scratch; the host reads them once, with the frames, when the sizes are
+    // needed
+    if (ensure(c->flags, sizeof(BuildNotes)) || ensure(c->frames, q.n * sizeof(FrameRec)) ||
+        ensure(c->bounds, 8 * q.n * sizeof(int)) ||
+        (q.n > 1 && ensure(c->seg, 2 * (q.n + 1) * sizeof(u32))))
+        return set_err(c, START_ENOMEM, "out of device memory (inputs)");
+    if (q.n > 1) {
+        u32 *seg = c->seg.as<u32>();
+        ST_CUDA(c, put(seg, q.p0.data(), (q.n + 1) * sizeof(u32)));
+        ST_CUDA(c, put(seg + q.n + 1, q.s0.data(), (q.n + 1) * sizeof(u32)));
+        ps.start = seg;
+        ss.start = seg + q.n + 1;
+    }
+    BuildNotes *notes = c->flags.as<BuildNotes>();
+    FrameRec *frames = c->frames.as<FrameRec>();
+    ST_CUDA(c, cudaMemsetAsync(notes, 0, sizeof(BuildNotes), s));
+    ST_TRY(compute_frames(c, in.pos.as<float>(), n_p, ps, in.spos.as<float>(), n_s, ss,
+                          c->bounds.as<int>(), frames));
+
+    // keys, stable sorts, Morton-ordered records
+    size_t P = (size_t)(n_p ? n_p : 1), S = (size_t)(n_s ? n_s : 1);
+    if (ensure(c->pkey, P * 8) || ensure(c->tk[1], P * 8) || ensure(c->porig, P * 4) ||
+        ensure(c->pinv, P * 4) || ensure(c->pq, P * 16) || ensure(c->ph, P * 4) ||
+        ensure(c->nH, P * 4) || ensure(c->y, P * 8) || ensure(c->V, P * 8) || ensure(c->Tg, P * 8) ||
+        ensure(c->gam, P * 4) || ensure(c->eL, P * 8) || ensure(c->eLs, P * 4) ||
+        ensure(c->skey, S * 8) || ensure(c->tv[1], S * 8) || ensure(c->sorig, S * 4) ||
+        ensure(c->sq, S * 16) || ensure(c->sL, S * 8) ||
+        (batch && (ensure(c->trange, P * 8) || ensure(c->trf2, P * 4))))
+        return set_err(c, START_ENOMEM, "out of device memory (inputs)");
+    u64 *pks = c->tk[1].as<u64>(), *sks = c->tv[1].as<u64>();
+    ST_TRY(morton_keys(c, in.pos.as<float>(), n_p, ps, frames, c->pkey.as<u64>()));
+    ST_TRY(morton_keys(c, in.spos.as<float>(), n_s, ss, frames, c->skey.as<u64>()));
+    BuildNotes bn;
+    std::vector<FrameRec> fr(q.n);
+    for (int attempt = 0;; ++attempt) {
+        ST_TRY(sort_keys(c, c->pkey.as<u64>(), n_p, ps, q.p0, pks, c->porig.as<u32>(),
+                         c->sort_all_bits, &notes->long_runs));
+        ST_TRY(sort_keys(c, c->skey.as<u64>(), n_s, ss, q.s0, sks, c->sorig.as<u32>(),
+                         c->sort_all_bits, &notes->long_runs));
+        ST_TRY(tree_census(c, c->pt, pks, n_p, c->p.ptree_leaf, ps, notes->hist[0]));
+        ST_TRY(tree_census(c, c->stree, sks, n_s, c->p.src_leaf, ss, notes->hist[1]));
+        c->et.n = 0;
+        if (diffuse)
+            ST_TRY(tree_census(c, c->et, pks, n_p, c->p.src_leaf, ps, notes->hist[2]));
+        unsigned long long bad[C_COUNT];
+        ST_CUDA(c, cudaMemcpyAsync(&bn, notes, sizeof(bn), cudaMemcpyDeviceToHost, s));
+        ST_CUDA(c, cudaMemcpyAsync(fr.data(), frames, q.n * sizeof(FrameRec),
+                                   cudaMemcpyDeviceToHost, s));
+        ST_CUDA(c, cudaMemcpyAsync(bad, ctr, sizeof(bad), cudaMemcpyDeviceToHost, s));
+        ST_CUDA(c, cudaStreamSynchronize(s));
+        if (bad[C_BAD_INPUT] || bad[C_BAD_POS]) return bad_problem(c, q, in, batch);
+        if (!bn.long_runs) break;
+        if (attempt) return set_err(c, START_ECUDA, "internal inconsistency (sort)");
+        c->sort_all_bits = true;   // tight clumps: all bits, also in the next builds
+        ST_CUDA(c, cudaMemsetAsync(notes->hist, 0, sizeof(bn.hist), s));
+        ST_CUDA(c, cudaMemsetAsync(&notes->long_runs, 0, sizeof(bn.long_runs), s));
+    }
+    if (n_p) {
+        k_gather_particles<<<grid_for(n_p, 256), 256, 0, s>>>(
+            in.pos.as<float>(), ps, in.h.as<float>(), diffuse ? in.V.as<double>() : nullptr,
+            c->porig.as<u32>(), n_p, c->pq.as<float4>(), c->ph.as<float>(), c->V.as<double>(),
+            c->nH.as<float>(), c->y.as<double>(), c->gam.as<float>(), c->pinv.as<u32>(),
+            c->eL.as<double>(), c->eLs.as<float>(), c->Tg.as<double>());
+        ++c->launches;
+    }
+    if (n_s) {
+        k_gather_sources<<<grid_for(n_s, 256), 256, 0, s>>>(
+            in.spos.as<float>(), ss, in.L.as<double>(), c->sorig.as<u32>(), n_s, c->p.L_unit,
+            c->sq.as<float4>(), c->sL.as<double>());
+        ++c->launches;
+    }
+    ST_CUDA(c, cudaGetLastError());
+    for (int a = 0; a < 3; ++a) c->fr.lo[a] = fr[0].lo[a];
+    c->fr.side = fr[0].side;
+    c->fr.cmag = 0.f;   // the filters' magnitude bound covers every problem
+    for (int b = 0; b < q.n; ++b)
+        if (q.n_p[b] + q.n_s[b] > 0) c->fr.cmag = std::max(c->fr.cmag, fr[b].cmag);
+    ST_TRY(tree_emit(c, c->pt, pks, n_p, ps, frames, bn.hist[0], notes->hist[0],
+                     notes->cursor[0], false));
+    ST_TRY(tree_emit(c, c->stree, sks, n_s, ss, frames, bn.hist[1], notes->hist[1],
+                     notes->cursor[1], true));
+    ST_TRY(tree_moments(c, c->stree, c->sq.as<float4>(), c->sL.as<double>(), c->p.L_unit));
+    if (diffuse)
+        ST_TRY(tree_emit(c, c->et, pks, n_p, ps, frames, bn.hist[2], notes->hist[2],
+                         notes->cursor[2], true));
+    if (batch && n_p) {
+        k_batch_targets<<<grid_for(n_p, 256), 256, 0, s>>>(
+            n_p, ps, ss, n_s, c->stree.pos.as<u32>(), frames, c->trange.as<uint2>(),
+            c->trf2.as<float>());
+        ++c->launches;
+        ST_CUDA(c, cudaGetLastError());
+    }
+    ST_TRY(build_neighbours(c, ps, frames));
+    phase_mark(c, START_PHASE_BUILD, true);
+    ST_CUDA(c, cudaGetLastError());
+    if (read_counter(c, C_INTERNAL)) return set_err(c, START_ECUDA, "internal inconsistency (trees or neighbour lists)");
+    c->built = true;
+    return START_OK;
+}
+
 int start_build_trees(start_ctx *c, const float *pos, const float *h, long long n_p,
                       const float *src_pos, const double *src_L, long long n_s, const double *V,
                       unsigned flags)
@@ -560,108 +725,8 @@ int start_build_trees(start_ctx *c, const float *pos, const float *h, long long 
     c->np = n_p;
     c->ns = n_s;
     c->diffuse = diffuse;
-    cudaStream_t s = c->stream;
-    unsigned long long *ctr = c->counters.as<unsigned long long>();
-    ST_CUDA(c, cudaMemsetAsync(ctr, 0, C_COUNT * sizeof(unsigned long long), s));
-
-    phase_mark(c, START_PHASE_BUILD, false);
-    Staged in;
-    ST_TRY(stage_in(c, in.pos, pos, 3 * n_p * sizeof(float)));
-    ST_TRY(stage_in(c, in.h, h, n_p * sizeof(float)));
-    ST_TRY(stage_in(c, in.spos, src_pos, 3 * n_s * sizeof(float)));
-    ST_TRY(stage_in(c, in.L, src_L, n_s * sizeof(double)));
-    if (diffuse) ST_TRY(stage_in(c, in.V, V, n_p * sizeof(double)));
-    if (n_p) { k_check_pos_h<<<grid_for(n_p, 256), 256, 0, s>>>(in.h.as<float>(), n_p, ctr + C_BAD_INPUT); ++c->launches; }
-    if (n_s) { k_check_nonneg_d<<<grid_for(n_s, 256), 256, 0, s>>>(in.L.as<double>(), n_s, ctr + C_BAD_INPUT, 0); ++c->launches; }
-    if (diffuse && n_p) { k_check_nonneg_d<<<grid_for(n_p, 256), 256, 0, s>>>(in.V.as<double>(), n_p, ctr + C_BAD_INPUT, 1); ++c->launches; }
-    if (n_p + n_s == 0) {
-        c->pt.n = c->stree.n = c->et.n = 0;
-        c->nb_total = 0;
-        c->built = true;
-        return START_OK;
-    }
-    // the device's notes of a build: frame, cells per level of the three trees,
-    // and scratch; the host reads them once, when the sizes are needed
-    if (ensure(c->flags, sizeof(BuildNotes)))
-        return set_err(c, START_ENOMEM, "out of device memory (inputs)");
-    BuildNotes *notes = c->flags.as<BuildNotes>();
-    ST_CUDA(c, cudaMemsetAsync(notes, 0, sizeof(BuildNotes), s));
-    ST_TRY(compute_frame(c, in.pos.as<float>(), n_p, in.spos.as<float>(), n_s, notes->bounds,
-                         &notes->frame));
-
-    // particles: keys, stable sort, Morton-ordered records
-    size_t P = (size_t)(n_p ? n_p : 1), S = (size_t)(n_s ? n_s : 1);
-    if (ensure(c->pkey, P * 8) || ensure(c->tk[1], P * 8) || ensure(c->porig, P * 4) ||
-        ensure(c->pinv, P * 4) || ensure(c->pq, P * 16) || ensure(c->ph, P * 4) ||
-        ensure(c->nH, P * 4) || ensure(c->y, P * 8) || ensure(c->V, P * 8) || ensure(c->Tg, P * 8) ||
-        ensure(c->gam, P * 4) || ensure(c->eL, P * 8) || ensure(c->eLs, P * 4) ||
-        ensure(c->skey, S * 8) || ensure(c->tv[1], S * 8) || ensure(c->sorig, S * 4) ||
-        ensure(c->sq, S * 16) || ensure(c->sL, S * 8))
-        return set_err(c, START_ENOMEM, "out of device memory (inputs)");
-    const FrameRec *frame = &notes->frame;   // device address
-    const Segs one;
-    u64 *pks = c->tk[1].as<u64>(), *sks = c->tv[1].as<u64>();
-    if (n_p) ST_TRY(morton_keys(c, in.pos.as<float>(), n_p, frame, c->pkey.as<u64>()));
-    if (n_s) ST_TRY(morton_keys(c, in.spos.as<float>(), n_s, frame, c->skey.as<u64>()));
-    BuildNotes bn;
-    for (int attempt = 0;; ++attempt) {
-        ST_TRY(sort_keys(c, c->pkey.as<u64>(), n_p, pks, c->porig.as<u32>(), c->sort_all_bits,
-                         &notes->long_runs));
-        ST_TRY(sort_keys(c, c->skey.as<u64>(), n_s, sks, c->sorig.as<u32>(), c->sort_all_bits,
-                         &notes->long_runs));
-        ST_TRY(tree_census(c, c->pt, pks, n_p, c->p.ptree_leaf, one, notes->hist[0]));
-        ST_TRY(tree_census(c, c->stree, sks, n_s, c->p.src_leaf, one, notes->hist[1]));
-        c->et.n = 0;
-        if (diffuse)
-            ST_TRY(tree_census(c, c->et, pks, n_p, c->p.src_leaf, one, notes->hist[2]));
-        unsigned long long bad[C_COUNT];
-        ST_CUDA(c, cudaMemcpyAsync(&bn, notes, sizeof(bn), cudaMemcpyDeviceToHost, s));
-        ST_CUDA(c, cudaMemcpyAsync(bad, ctr, sizeof(bad), cudaMemcpyDeviceToHost, s));
-        ST_CUDA(c, cudaStreamSynchronize(s));
-        if (bad[C_BAD_INPUT] || bad[C_BAD_POS]) {
-            ST_CUDA(c, cudaMemsetAsync(ctr, 0, C_COUNT * sizeof(unsigned long long), s));
-            return set_err(c, START_EINVAL, bad[C_BAD_INPUT]
-                                                ? "invalid values in h, src_L or V"
-                                                : "non-finite particle or source position");
-        }
-        if (!bn.long_runs) break;
-        if (attempt) return set_err(c, START_ECUDA, "internal inconsistency (sort)");
-        c->sort_all_bits = true;   // tight clumps: all bits, also in the next builds
-        ST_CUDA(c, cudaMemsetAsync(notes->hist, 0, sizeof(bn.hist), s));
-        ST_CUDA(c, cudaMemsetAsync(&notes->long_runs, 0, sizeof(bn.long_runs), s));
-    }
-    if (n_p) {
-        k_gather_particles<<<grid_for(n_p, 256), 256, 0, s>>>(
-            in.pos.as<float>(), in.h.as<float>(), diffuse ? in.V.as<double>() : nullptr,
-            c->porig.as<u32>(), n_p, c->pq.as<float4>(), c->ph.as<float>(), c->V.as<double>(),
-            c->nH.as<float>(), c->y.as<double>(), c->gam.as<float>(), c->pinv.as<u32>(),
-            c->eL.as<double>(), c->eLs.as<float>(), c->Tg.as<double>());
-        ++c->launches;
-    }
-    if (n_s) {
-        k_gather_sources<<<grid_for(n_s, 256), 256, 0, s>>>(in.spos.as<float>(), in.L.as<double>(),
-                                                            c->sorig.as<u32>(), n_s, c->p.L_unit,
-                                                            c->sq.as<float4>(), c->sL.as<double>());
-        ++c->launches;
-    }
-    ST_CUDA(c, cudaGetLastError());
-    for (int a = 0; a < 3; ++a) c->fr.lo[a] = bn.frame.lo[a];
-    c->fr.side = bn.frame.side;
-    c->fr.cmag = bn.frame.cmag;
-    ST_TRY(tree_emit(c, c->pt, pks, n_p, one, frame, bn.hist[0], notes->hist[0],
-                     notes->cursor[0], false));
-    ST_TRY(tree_emit(c, c->stree, sks, n_s, one, frame, bn.hist[1], notes->hist[1],
-                     notes->cursor[1], true));
-    ST_TRY(tree_moments(c, c->stree, c->sq.as<float4>(), c->sL.as<double>(), c->p.L_unit));
-    if (diffuse)
-        ST_TRY(tree_emit(c, c->et, pks, n_p, one, frame, bn.hist[2], notes->hist[2],
-                         notes->cursor[2], true));
-    ST_TRY(build_neighbours(c, one, frame));
-    phase_mark(c, START_PHASE_BUILD, true);
-    ST_CUDA(c, cudaGetLastError());
-    if (read_counter(c, C_INTERNAL)) return set_err(c, START_ECUDA, "internal inconsistency (trees or neighbour lists)");
-    c->built = true;
-    return START_OK;
+    Problems q{1, &n_p, &n_s, &pos, &h, &src_pos, &src_L, diffuse ? V : nullptr, {}, {}};
+    return build_problems(c, q, diffuse, false);
 }
 
 int start_build_batch(start_ctx *c, int nb, const long long *n_p, const long long *n_s,
@@ -681,116 +746,18 @@ int start_build_batch(start_ctx *c, int nb, const long long *n_p, const long lon
         if (n_p[b] < 0 || n_s[b] < 0) return set_err(c, START_EINVAL, "negative size");
         P += n_p[b];
         S += n_s[b];
+        if ((n_p[b] && (!pos[b] || !h[b])) || (n_s[b] && (!src_pos[b] || !src_L[b])))
+            return set_err(c, START_EINVAL, "batch part " + std::to_string(b) + ": NULL input array");
     }
     if (P >= START_MAX_N || S >= START_MAX_N)
         return set_err(c, START_ERANGE, "a batch holds below 2^30 particles and sources");
-    // every problem built on its own (its frame, trees and neighbour lists), in
-    // contexts that share this one's stream and parameters
-    while ((int)c->bsub.size() < nb) {
-        start_ctx *b = nullptr;
-        start_params q = c->p;
-        q.timing = 0;
-        int rc = start_create(&b, &q);
-        if (rc != START_OK) return set_err(c, rc, "batch: creating a part");
-        c->bsub.push_back(b);
-    }
-    long long N = 0, NB = 0;
-    float cmag = 0.f;
-    for (int b = 0; b < nb; ++b) {
-        start_ctx *q = c->bsub[b];
-        q->p = c->p;
-        q->p.timing = 0;
-        q->stream = c->stream;
-        int rc = start_build_trees(q, pos[b], h[b], n_p[b], src_pos[b], src_L[b], n_s[b], nullptr,
-                                   0u);
-        if (rc != START_OK) return set_err(c, rc, "batch part " + std::to_string(b) + ": " + q->err);
-        N += q->stree.n;
-        NB += q->nb_total;
-        if (q->np + q->ns > 0 && q->fr.cmag > cmag) cmag = q->fr.cmag;
-        c->launches += q->launches;
-        q->launches = 0;
-    }
-    if (N >= (1LL << 31)) return set_err(c, START_ERANGE, "a batch's forest is too large");
-    size_t Pz = (size_t)(P ? P : 1), Sz = (size_t)(S ? S : 1), Nz = (size_t)(N ? N : 1);
-    Tree &t = c->stree;
-    if (ensure(c->pq, Pz * 16) || ensure(c->ph, Pz * 4) || ensure(c->porig, Pz * 4) ||
-        ensure(c->pinv, Pz * 4) || ensure(c->pkey, Pz * 8) || ensure(c->nH, Pz * 4) ||
-        ensure(c->y, Pz * 8) || ensure(c->V, Pz * 8) || ensure(c->Tg, Pz * 8) ||
-        ensure(c->gam, Pz * 4) || ensure(c->eL, Pz * 8) || ensure(c->eLs, Pz * 4) ||
-        ensure(c->nb_off, (Pz + 1) * 4) || ensure(c->nb_idx, (size_t)(NB ? NB : 1) * 4) ||
-        ensure(c->sq, Sz * 16) || ensure(c->sL, Sz * 8) || ensure(c->sorig, Sz * 4) ||
-        ensure(c->skey, Sz * 8) || ensure(t.box, Nz * 16) || ensure(t.meta, Nz * 16) ||
-        ensure(t.cube, Nz * 32) || ensure(t.level, Nz * 4) || ensure(t.parent, Nz * 4) ||
-        ensure(t.leafof, Sz * 4) || ensure(t.vsrc, Nz * 16) || ensure(t.L, Nz * 8) ||
-        ensure(t.M, Nz * 24) || ensure(c->trange, Pz * 8) || ensure(c->trf2, Pz * 4))
-        return set_err(c, START_ENOMEM, "out of device memory (batch)");
-    long long p0 = 0, s0 = 0, n0 = 0, e0 = 0;
-    for (int b = 0; b < nb; ++b) {
-        start_ctx *q = c->bsub[b];
-        const long long np = q->np, ns = q->ns, nn = q->stree.n, ne = q->nb_total;
-        if (np) {
-            ST_TRY(copy_dev(c, c->pq.as<float4>() + p0, q->pq.p, np * 16));
-            ST_TRY(copy_dev(c, c->ph.as<float>() + p0, q->ph.p, np * 4));
-            ST_TRY(copy_dev(c, c->pkey.as<u64>() + p0, q->pkey.p, np * 8));
-            ST_TRY(copy_dev(c, c->V.as<double>() + p0, q->V.p, np * 8));
-            ST_TRY(copy_dev(c, c->nH.as<float>() + p0, q->nH.p, np * 4));
-            ST_TRY(copy_dev(c, c->y.as<double>() + p0, q->y.p, np * 8));
-            ST_TRY(copy_dev(c, c->gam.as<float>() + p0, q->gam.p, np * 4));
-            ST_TRY(copy_dev(c, c->Tg.as<double>() + p0, q->Tg.p, np * 8));
-            ST_TRY(shift_copy(c, c->porig.as<u32>() + p0, q->porig.as<u32>(), np, (u32)p0));
-            ST_TRY(shift_copy(c, c->pinv.as<u32>() + p0, q->pinv.as<u32>(), np, (u32)p0));
-            ST_TRY(shift_copy(c, c->nb_off.as<u32>() + p0, q->nb_off.as<u32>(), np, (u32)e0));
-            ST_TRY(shift_copy(c, c->nb_idx.as<u32>() + e0, q->nb_idx.as<u32>(), ne, (u32)p0));
-            const double rf = 1e-6 * q->fr.side;
-            k_fill_range<<<grid_for(np, 256), 256, 0, c->stream>>>(
-                c->trange.as<uint2>() + p0, c->trf2.as<float>() + p0, np,
-                make_uint2((u32)n0, (u32)(n0 + nn)), (float)(rf * rf));
-            ++c->launches;
-        }
-        if (ns) {
-            ST_TRY(copy_dev(c, c->sq.as<float4>() + s0, q->sq.p, ns * 16));
-            ST_TRY(copy_dev(c, c->sL.as<double>() + s0, q->sL.p, ns * 8));
-            ST_TRY(copy_dev(c, c->skey.as<u64>() + s0, q->skey.p, ns * 8));
-            ST_TRY(shift_copy(c, c->sorig.as<u32>() + s0, q->sorig.as<u32>(), ns, (u32)s0));
-            ST_TRY(shift_copy(c, t.leafof.as<u32>() + s0, q->stree.leafof.as<u32>(), ns, (u32)n0));
-        }
-        if (nn) {
-            const Tree &u = q->stree;
-            ST_TRY(copy_dev(c, t.box.as<float4>() + n0, u.box.p, nn * 16));
-            ST_TRY(copy_dev(c, t.cube.as<double>() + 4 * n0, u.cube.p, nn * 32));
-            ST_TRY(copy_dev(c, t.level.as<int>() + n0, u.level.p, nn * 4));
-            ST_TRY(copy_dev(c, t.vsrc.as<float4>() + n0, u.vsrc.p, nn * 16));
-            ST_TRY(copy_dev(c, t.L.as<double>() + n0, u.L.p, nn * 8));
-            ST_TRY(copy_dev(c, t.M.as<double>() + 3 * n0, u.M.p, nn * 24));
-            ST_TRY(shift_copy(c, t.parent.as<u32>() + n0, u.parent.as<u32>(), nn, (u32)n0));
-            k_shift_meta<<<grid_for(nn, 256), 256, 0, c->stream>>>(
-                u.meta.as<uint4>(), nn, (u32)n0, (u32)s0, t.meta.as<uint4>() + n0);
-            ++c->launches;
-        }
-        p0 += np;
-        s0 += ns;
-        n0 += nn;
-        e0 += ne;
-    }
-    u32 etot = (u32)NB;
-    ST_CUDA(c, cudaMemcpyAsync(c->nb_off.as<u32>() + P, &etot, 4, cudaMemcpyHostToDevice,
-                               c->stream));
-    if (P) {
-        ST_CUDA(c, cudaMemsetAsync(c->eL.p, 0, P * 8, c->stream));
-        ST_CUDA(c, cudaMemsetAsync(c->eLs.p, 0, P * 4, c->stream));
-    }
-    ST_CUDA(c, cudaStreamSynchronize(c->stream));   // the stacked values above are on the host
     c->np = P;
     c->ns = S;
-    c->nb_total = NB;
     c->diffuse = false;
-    c->pt.n = 0;          // the problems' particle trees stay in their parts
-    c->et.n = 0;
-    t.n = N;
-    c->fr = c->bsub[0]->fr;
-    c->fr.cmag = cmag;    // the filters' magnitude bound covers every problem
+    Problems q{nb, n_p, n_s, pos, h, src_pos, src_L, nullptr, {}, {}};
+    ST_TRY(build_problems(c, q, false, true));
+    c->pt.n = 0;          // the trees of the problems' particles are no single tree
     c->nbatch = nb;
-    c->built = true;
     return START_OK;
 }
 

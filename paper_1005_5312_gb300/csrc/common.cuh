@@ -100,6 +100,13 @@ struct Frame {
     float cmag;                // bound on |coordinate| of any point or cube corner
 };
 
+// Coordinate a of point i in the positions of a batch: problem after problem,
+// each x[m], y[m], z[m]; [lo, hi) are the points of i's problem.
+__device__ __forceinline__ size_t point_index(u32 lo, u32 hi, long long i, int a)
+{
+    return 3 * (size_t)lo + (size_t)a * (hi - lo) + (size_t)(i - lo);
+}
+
 }  // namespace st
 
 constexpr int kLevelBatch = 4;   // memoised march: frontier levels issued per host round trip
@@ -179,7 +186,7 @@ struct start_ctx {
     // target walks only its problem's range (trange, uint2 per target) with its
     // problem's dilution floor (trf2, float per target)
     int nbatch = 0;
-    std::vector<start_ctx *> bsub;     // contexts the problems are built in
+    st::DBuf seg, frames, bounds;      // problem bounds (u32), root cubes and their scratch
     st::DBuf trange, trf2;
 
     // memoised march: per chain link (virtual source, particle)
@@ -299,11 +306,12 @@ void phase_mark(start_ctx *c, int phase, bool end);
 // scan_sort.cu
 int exclusive_scan_u32(start_ctx *c, const u32 *in, u32 *out, long long n, u32 *total_dev);
 int exclusive_scan_u32_to_u64(start_ctx *c, const u32 *in, u64 *out, long long n);
-int sort_keys(start_ctx *c, const u64 *keys, long long n, u64 *sorted, u32 *perm, bool all_bits,
-              u32 *longer);
-int compute_frame(start_ctx *c, const float *ppos, long long np, const float *spos, long long ns,
-                  int *mm, FrameRec *fr);
-int morton_keys(start_ctx *c, const float *pos_soa, long long n, const FrameRec *fr, u64 *keys);
+int sort_keys(start_ctx *c, const u64 *keys, long long n, const Segs &segs,
+              const std::vector<u32> &start, u64 *sorted, u32 *perm, bool all_bits, u32 *longer);
+int compute_frames(start_ctx *c, const float *ppos, long long np, const Segs &psegs,
+                   const float *spos, long long ns, const Segs &ssegs, int *mm, FrameRec *fr);
+int morton_keys(start_ctx *c, const float *pos, long long n, const Segs &segs,
+                const FrameRec *frames, u64 *keys);
 
 // tree.cu
 int tree_census(start_ctx *c, Tree &t, const u64 *keys, long long n, int leaf, const Segs &segs,

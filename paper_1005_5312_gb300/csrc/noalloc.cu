@@ -25,8 +25,9 @@ namespace st {
 
 // Kernels of the regular path (scan_sort.cu), reused unchanged with
 // pointers into the fixed scratch.
-__global__ void k_bbox_init(int *mm);
-__global__ void k_bbox(const float *pos, long long n, int *mm, unsigned long long *bad);
+__global__ void k_bbox_init(int *mm, int problems);
+__global__ void k_bbox(const float *pos, long long n, Segs segs, int *mm,
+                       unsigned long long *bad);
 void rs_tile_hist(const u64 *keys, long long n, int shift, u32 *hist, int nblocks,
                   cudaStream_t s);
 void rs_tile_scatter(const u64 *kin, const u32 *vin, u64 *kout, u32 *vout, long long n, int shift,
@@ -202,8 +203,8 @@ extern "C" int start_morton_order_noalloc(const float *pos, long long n, unsigne
 
     // the array keeps the previous call's contents: reset the counter
     if (cudaMemsetAsync(bad, 0, sizeof(*bad), s) != cudaSuccess) return START_ECUDA;
-    k_bbox_init<<<1, 32, 0, s>>>(mm);
-    k_bbox<<<grid_for(n, 256, 1024), 256, 0, s>>>(pos, n, mm, bad);
+    k_bbox_init<<<1, 32, 0, s>>>(mm, 1);
+    k_bbox<<<grid_for(n, 256, 1024), 256, 0, s>>>(pos, n, Segs{}, mm, bad);
     k_frame_dev<<<1, 1, 0, s>>>(mm, frame, frame_out);
     k_morton_dev<<<grid_for(n, 256), 256, 0, s>>>(pos, n, frame, ka, reinterpret_cast<u64 *>(keys_out),
                                                   perm_out);

@@ -199,12 +199,12 @@ __global__ void __launch_bounds__(kRsThreads) k_rs_hist(const u64 *keys, long lo
 
 // Stable scatter: within a tile the items are ranked in index order
 // (warp-major, then round, then lane) with warp match/popc.  vin NULL: the
-// values are the items' indices.
+// values are the items' indices, from v0 on.
 template <int IPT>
 __global__ void __launch_bounds__(kRsThreads) k_rs_scatter(const u64 *kin, const u32 *vin,
                                                            u64 *kout, u32 *vout, long long n,
                                                            int shift, const u32 *offs,
-                                                           int nblocks)
+                                                           int nblocks, u32 v0)
 {
     __shared__ u32 wcnt[kRsWarps][256];
     __shared__ u32 base[256];
@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(kRsThreads) k_rs_scatter(const u64 *kin, const
         long long idx = wbase + r * 32 + lane;
         bool valid = idx < n;
         k[r] = valid ? kin[idx] : 0ull;
-        v[r] = !valid ? 0u : vin ? vin[idx] : (u32)idx;
+        v[r] = !valid ? 0u : vin ? vin[idx] : v0 + (u32)idx;
         int d = valid ? (int)((k[r] >> shift) & 255u) : 256;
         dg[r] = d;
         unsigned peers = __match_any_sync(0xffffffffu, d);
@@ -263,7 +263,7 @@ void rs_tile_hist(const u64 *keys, long long n, int shift, u32 *hist, int nblock
 void rs_tile_scatter(const u64 *kin, const u32 *vin, u64 *kout, u32 *vout, long long n, int shift,
                      const u32 *offs, int nblocks, cudaStream_t s)
 {
-    k_rs_scatter<16><<<nblocks, kRsThreads, 0, s>>>(kin, vin, kout, vout, n, shift, offs, nblocks);
+    k_rs_scatter<16><<<nblocks, kRsThreads, 0, s>>>(kin, vin, kout, vout, n, shift, offs, nblocks, 0u);
 }
 
 // Sorting up to kRankSort keys by counting: the place of an item is the
@@ -272,39 +272,49 @@ void rs_tile_scatter(const u64 *kin, const u32 *vin, u64 *kout, u32 *vout, long 
 // (every lane reads the same key: a broadcast).  The count is n^2 comparisons,
 // but in one launch over the whole chip: 8 us at 2 k keys, where eight radix
 // passes by one block took 55 us; the four passes of a larger sort take 90 us
-// at 23 k keys.
+// at 23 k keys.  blockIdx.y: the problem of a batch; problems with more keys
+// are left to the radix passes.
 constexpr long long kRankSort = 16384;
 constexpr int kRankTile = 2048;
 
-__global__ void __launch_bounds__(256) k_rank_sort(const u64 *kin, int n, u64 *kout, u32 *perm)
+__global__ void __launch_bounds__(256) k_rank_sort(const u64 *keys, int n_all, Segs segs,
+                                                   u64 *sorted, u32 *perm)
 {
     __shared__ __align__(16) u64 tile[kRankTile];
     __shared__ u32 part[8][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int i = blockIdx.x * 32 + lane;
-    const u64 key = i < n ? kin[i] : 0ull;
-    u32 below = 0;
-    for (int t0 = 0; t0 < n; t0 += kRankTile) {
-        __syncthreads();
-        for (int j = threadIdx.x; j < kRankTile; j += 256)
-            tile[j] = t0 + j < n ? kin[t0 + j] : ~0ull;   // above every key
-        __syncthreads();
-        const int j0 = w * (kRankTile / 8);
+    for (int b = blockIdx.y; b < segs.n; b += gridDim.y) {
+        const u32 lo = segs.n > 1 ? segs.start[b] : 0u;
+        const u32 m = segs.n > 1 ? segs.start[b + 1] - lo : (u32)n_all;
+        if (blockIdx.x * 32 >= m || m > kRankSort) continue;   // block-uniform
+        const int n = (int)m;
+        const u64 *kin = keys + lo;
+        const u64 key = i < n ? kin[i] : 0ull;
+        u32 below = 0;
+        for (int t0 = 0; t0 < n; t0 += kRankTile) {
+            __syncthreads();
+            for (int j = threadIdx.x; j < kRankTile; j += 256)
+                tile[j] = t0 + j < n ? kin[t0 + j] : ~0ull;   // above every key
+            __syncthreads();
+            const int j0 = w * (kRankTile / 8);
 #pragma unroll 4
-        for (int j = 0; j < kRankTile / 8; j += 2) {
-            const ulonglong2 q = *reinterpret_cast<const ulonglong2 *>(&tile[j0 + j]);
-            const int g = t0 + j0 + j;
-            below += q.x < key || (q.x == key && g < i);
-            below += q.y < key || (q.y == key && g + 1 < i);
+            for (int j = 0; j < kRankTile / 8; j += 2) {
+                const ulonglong2 q = *reinterpret_cast<const ulonglong2 *>(&tile[j0 + j]);
+                const int g = t0 + j0 + j;
+                below += q.x < key || (q.x == key && g < i);
+                below += q.y < key || (q.y == key && g + 1 < i);
+            }
         }
-    }
-    part[w][lane] = below;
-    __syncthreads();
-    if (w == 0 && i < n) {
-        u32 r = 0;
-        for (int k = 0; k < 8; ++k) r += part[k][lane];
-        kout[r] = key;
-        perm[r] = (u32)i;
+        part[w][lane] = below;
+        __syncthreads();
+        if (w == 0 && i < n) {
+            u32 r = 0;
+            for (int k = 0; k < 8; ++k) r += part[k][lane];
+            sorted[lo + r] = key;
+            perm[lo + r] = lo + (u32)i;
+        }
+        __syncthreads();
     }
 }
 
@@ -341,7 +351,7 @@ __global__ void k_sort_runs(u64 *keys, u32 *vals, long long n, u32 *longer)
 
 template <int IPT>
 static int rs_pass(start_ctx *c, const u64 *ka, const u32 *va, u64 *kb, u32 *vb, long long n,
-                   int shift)
+                   int shift, u32 v0)
 {
     const int nblocks = (int)((n + kRsThreads * IPT - 1) / (kRsThreads * IPT));
     ST_TRY(ensure(c->hist, (size_t)2 * 256 * nblocks * sizeof(u32)));
@@ -351,26 +361,20 @@ static int rs_pass(start_ctx *c, const u64 *ka, const u32 *va, u64 *kb, u32 *vb,
     ST_CUDA(c, cudaGetLastError());
     ST_TRY(exclusive_scan_u32(c, hist, offs, (long long)256 * nblocks, nullptr));
     k_rs_scatter<IPT><<<nblocks, kRsThreads, 0, c->stream>>>(ka, va, kb, vb, n, shift, offs,
-                                                             nblocks);
+                                                             nblocks, v0);
     c->launches += 2;
     return cuda_check(c, cudaGetLastError(), "k_rs_scatter");
 }
 
 // Sorted keys and the input index of every rank (stable: equal keys in input
-// order) of n keys in input order.  More than kRankSort keys: four radix passes
-// over the leading 32 bits, after which only particles within 2^-10.67 of the
-// box of each other share a run (sorted by insertion); runs that are too long
-// are counted in `longer`, which the caller cleared, and the caller sorts
-// again with all_bits: eight passes.
-int sort_keys(start_ctx *c, const u64 *keys, long long n, u64 *sorted, u32 *perm, bool all_bits,
-              u32 *longer)
+// order) of one set of n keys from index v0 on by radix passes: four over the
+// leading 32 bits, after which only particles within 2^-10.67 of the box of
+// each other share a run (sorted by insertion); runs that are too long are
+// counted in `longer`, which the caller cleared, and the caller sorts again
+// with all_bits: eight passes.
+static int radix_sort(start_ctx *c, const u64 *keys, long long n, u32 v0, u64 *sorted, u32 *perm,
+                      bool all_bits, u32 *longer)
 {
-    if (n <= 0) return START_OK;
-    if (n <= kRankSort) {
-        k_rank_sort<<<grid_for(n, 32), 256, 0, c->stream>>>(keys, (int)n, sorted, perm);
-        ++c->launches;
-        return cuda_check(c, cudaGetLastError(), "k_rank_sort");
-    }
     ST_TRY(ensure(c->tk[0], n * sizeof(u64)));
     ST_TRY(ensure(c->tv[0], n * sizeof(u32)));
     u64 *tk = c->tk[0].as<u64>();
@@ -381,8 +385,8 @@ int sort_keys(start_ctx *c, const u64 *keys, long long n, u64 *sorted, u32 *perm
         const u32 *va = pass == 0 ? nullptr : (pass & 1 ? tv : perm);
         u64 *kb = pass & 1 ? sorted : tk;
         u32 *vb = pass & 1 ? perm : tv;
-        ST_TRY(n < kRsSmallTiles ? rs_pass<4>(c, ka, va, kb, vb, n, shift)
-                                 : rs_pass<16>(c, ka, va, kb, vb, n, shift));
+        ST_TRY(n < kRsSmallTiles ? rs_pass<4>(c, ka, va, kb, vb, n, shift, v0)
+                                 : rs_pass<16>(c, ka, va, kb, vb, n, shift, v0));
     }
     // four or eight passes: the result is in (sorted, perm)
     if (!all_bits) {
@@ -390,6 +394,32 @@ int sort_keys(start_ctx *c, const u64 *keys, long long n, u64 *sorted, u32 *perm
         ++c->launches;
     }
     return cuda_check(c, cudaGetLastError(), "k_sort_runs");
+}
+
+// Sorts the n keys of every problem on its own (start: host copy of the
+// problems' bounds): all problems of at most kRankSort keys in one launch, the
+// larger ones one after the other.
+int sort_keys(start_ctx *c, const u64 *keys, long long n, const Segs &segs,
+              const std::vector<u32> &start, u64 *sorted, u32 *perm, bool all_bits, u32 *longer)
+{
+    if (n <= 0) return START_OK;
+    long long small = 0;   // the largest problem sorted by counting
+    for (int b = 0; b < segs.n; ++b) {
+        const long long m = (long long)start[b + 1] - start[b];
+        if (m <= kRankSort && m > small) small = m;
+    }
+    if (small) {
+        k_rank_sort<<<dim3(grid_for(small, 32), segs.n < 65535 ? segs.n : 65535), 256, 0, c->stream>>>(keys, (int)n, segs,
+                                                                              sorted, perm);
+        ++c->launches;
+        ST_CUDA(c, cudaGetLastError());
+    }
+    for (int b = 0; b < segs.n; ++b) {
+        const long long lo = start[b], m = (long long)start[b + 1] - lo;
+        if (m > kRankSort)
+            ST_TRY(radix_sort(c, keys + lo, m, (u32)lo, sorted + lo, perm + lo, all_bits, longer));
+    }
+    return START_OK;
 }
 
 // ---------------------------------------------------------------- frame
@@ -400,56 +430,72 @@ __device__ __forceinline__ int f2ord(float f)
 }
 __device__ __forceinline__ float ord2f(int i) { return __int_as_float(i >= 0 ? i : i ^ 0x7fffffff); }
 
-__global__ void k_bbox_init(int *mm)
+// Bounds of the problems' points (six ordered ints each, mm[8 b ..]).
+__global__ void k_bbox_init(int *mm, int problems)
 {
-    if (threadIdx.x < 3) mm[threadIdx.x] = 0x7fffffff;
-    else if (threadIdx.x < 6) mm[threadIdx.x] = (int)0x80000000;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= 8 * problems) return;
+    mm[t] = (t & 7) < 3 ? 0x7fffffff : (int)0x80000000;
 }
 
-__global__ void k_bbox(const float *pos, long long n, int *mm, unsigned long long *bad)
+// Widens the bounds of every problem by its points: the problems' positions
+// one after the other, each x[m], y[m], z[m]; a row of blocks per problem.
+__global__ void k_bbox(const float *pos_all, long long n_all, Segs segs, int *mm_all,
+                       unsigned long long *bad)
 {
-    float lo[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, hi[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX};
-    unsigned long long nbad = 0;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            float v = pos[(long long)a * n + i];
-            if (!isfinite(v)) { ++nbad; continue; }
-            lo[a] = fminf(lo[a], v);
-            hi[a] = fmaxf(hi[a], v);
-        }
-    }
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        for (int o = 16; o; o >>= 1) {
-            lo[a] = fminf(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
-            hi[a] = fmaxf(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], o));
-        }
-    }
-    for (int o = 16; o; o >>= 1) nbad += __shfl_xor_sync(0xffffffffu, nbad, o);
-    // one set of atomics per block
     __shared__ int bound[6];
-    if (threadIdx.x < 6) bound[threadIdx.x] = threadIdx.x < 3 ? 0x7fffffff : (int)0x80000000;
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) {
+    for (int b = blockIdx.y; b < segs.n; b += gridDim.y) {
+        const long long p0 = segs.n > 1 ? segs.start[b] : 0;
+        const long long n = segs.n > 1 ? (long long)segs.start[b + 1] - p0 : n_all;
+        const float *pos = pos_all + 3 * p0;
+        if ((long long)blockIdx.x * blockDim.x >= n) continue;   // block-uniform
+        float lo[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, hi[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX};
+        unsigned long long nbad = 0;
+        for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+             i += (long long)gridDim.x * blockDim.x) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                float v = pos[(long long)a * n + i];
+                if (!isfinite(v)) { ++nbad; continue; }
+                lo[a] = fminf(lo[a], v);
+                hi[a] = fmaxf(hi[a], v);
+            }
+        }
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            atomicMin(&bound[a], f2ord(lo[a]));
-            atomicMax(&bound[3 + a], f2ord(hi[a]));
+            for (int o = 16; o; o >>= 1) {
+                lo[a] = fminf(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
+                hi[a] = fmaxf(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], o));
+            }
         }
-        if (nbad) atomicAdd(bad, nbad);
+        for (int o = 16; o; o >>= 1) nbad += __shfl_xor_sync(0xffffffffu, nbad, o);
+        // one set of atomics per block
+        if (threadIdx.x < 6) bound[threadIdx.x] = threadIdx.x < 3 ? 0x7fffffff : (int)0x80000000;
+        __syncthreads();
+        if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                atomicMin(&bound[a], f2ord(lo[a]));
+                atomicMax(&bound[3 + a], f2ord(hi[a]));
+            }
+            if (nbad) atomicAdd(bad, nbad);
+        }
+        __syncthreads();
+        if (threadIdx.x < 3) atomicMin(&mm_all[8 * b + threadIdx.x], bound[threadIdx.x]);
+        else if (threadIdx.x < 6) atomicMax(&mm_all[8 * b + threadIdx.x], bound[threadIdx.x]);
+        __syncthreads();
     }
-    __syncthreads();
-    if (threadIdx.x < 3) atomicMin(&mm[threadIdx.x], bound[threadIdx.x]);
-    else if (threadIdx.x < 6) atomicMax(&mm[threadIdx.x], bound[threadIdx.x]);
 }
 
-// The root cube from the bounds mm: lower corner, largest extent (1 when it
-// is 0), keys per length, and a bound on every coordinate of a point or a cube
-// corner (FP64, never contracted).
-__global__ void k_frame(const int *mm, FrameRec *fr)
+// The root cube of every problem from its bounds: lower corner, largest extent
+// (1 when it is 0), keys per length, and a bound on every coordinate of a point
+// or a cube corner (FP64, never contracted).
+__global__ void k_frame(const int *mm_all, FrameRec *frames, int problems)
 {
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b >= problems) return;
+    const int *mm = mm_all + 8 * b;
+    FrameRec *fr = frames + b;
     double side = 0.0, mag;
     double lo[3];
     for (int a = 0; a < 3; ++a) {
@@ -469,16 +515,22 @@ __global__ void k_frame(const int *mm, FrameRec *fr)
     fr->pad = 0.f;
 }
 
-// Issues the frame of np particles and ns sources (mm: six ints of scratch);
-// non-finite positions are counted in C_BAD_POS.
-int compute_frame(start_ctx *c, const float *ppos, long long np, const float *spos, long long ns,
-                  int *mm, FrameRec *fr)
+// Issues the frames of the problems' np particles and ns sources (mm: eight
+// ints of scratch each); non-finite positions are counted in C_BAD_POS.
+int compute_frames(start_ctx *c, const float *ppos, long long np, const Segs &psegs,
+                   const float *spos, long long ns, const Segs &ssegs, int *mm, FrameRec *fr)
 {
     unsigned long long *bad = c->counters.as<unsigned long long>() + C_BAD_POS;
-    k_bbox_init<<<1, 32, 0, c->stream>>>(mm); ++c->launches;
-    if (np) { k_bbox<<<grid_for(np, 256, 1024), 256, 0, c->stream>>>(ppos, np, mm, bad); ++c->launches; }
-    if (ns) { k_bbox<<<grid_for(ns, 256, 1024), 256, 0, c->stream>>>(spos, ns, mm, bad); ++c->launches; }
-    k_frame<<<1, 1, 0, c->stream>>>(mm, fr); ++c->launches;
+    const int nb = psegs.n, rows = nb < 65535 ? nb : 65535;
+    k_bbox_init<<<grid_for(8 * nb, 256), 256, 0, c->stream>>>(mm, nb);
+    if (np)
+        k_bbox<<<dim3(grid_for(np, 256, nb > 1 ? 64 : 1024), rows), 256, 0, c->stream>>>(
+            ppos, np, psegs, mm, bad);
+    if (ns)
+        k_bbox<<<dim3(grid_for(ns, 256, nb > 1 ? 64 : 1024), rows), 256, 0, c->stream>>>(
+            spos, ns, ssegs, mm, bad);
+    k_frame<<<grid_for(nb, 64), 64, 0, c->stream>>>(mm, fr, nb);
+    c->launches += 2 + (np > 0) + (ns > 0);
     return cuda_check(c, cudaGetLastError(), "k_frame");
 }
 
@@ -494,25 +546,29 @@ __device__ __forceinline__ u64 spread3(u64 v)
     return v;
 }
 
-__global__ void k_morton(const float *pos, long long n, const FrameRec *fr, u64 *keys)
+__global__ void k_morton(const float *pos, long long n, Segs segs, const FrameRec *frames,
+                         u64 *keys)
 {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
+    u32 lo = 0u, hi = (u32)n;
+    const FrameRec *fr = frames + segs.range((u32)i, lo, hi);
     u64 q[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        double t = floor(__dmul_rn(__dsub_rn((double)pos[(long long)a * n + i], fr->lo[a]),
-                                   fr->scale));
+        const float x = pos[point_index(lo, hi, i, a)];
+        double t = floor(__dmul_rn(__dsub_rn((double)x, fr->lo[a]), fr->scale));
         t = fmin(fmax(t, 0.0), 2097151.0);
         q[a] = (u64)t;
     }
     keys[i] = (spread3(q[0]) << 2) | (spread3(q[1]) << 1) | spread3(q[2]);
 }
 
-int morton_keys(start_ctx *c, const float *pos_soa, long long n, const FrameRec *fr, u64 *keys)
+int morton_keys(start_ctx *c, const float *pos, long long n, const Segs &segs,
+                const FrameRec *frames, u64 *keys)
 {
     if (n <= 0) return START_OK;
-    k_morton<<<grid_for(n, 256), 256, 0, c->stream>>>(pos_soa, n, fr, keys); ++c->launches;
+    k_morton<<<grid_for(n, 256), 256, 0, c->stream>>>(pos, n, segs, frames, keys); ++c->launches;
     return cuda_check(c, cudaGetLastError(), "k_morton");
 }
 

@@ -1,0 +1,84 @@
+"""Batches built in one set of passes, where the stacked arrays are awkward:
+problems of one or a few particles (several in one group of 32 targets), empty
+problems at either end, problems without sources, one problem alone in its
+batch, problems beyond the counting sort beside small ones, duplicates and
+tight clumps.  Each problem's neighbour sets, Gamma and counts are those of
+the same problem built alone.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def S():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1005_5312_gb300 as S
+    S.build()
+    return S
+
+
+def problem(n_p, n_s, seed, clump=0):
+    rng = np.random.default_rng(seed)
+    pos = (rng.uniform(0.0, 1.0 + seed % 3, (3, n_p)) - seed).astype(np.float32)
+    if clump:
+        pos[:, :clump] = pos[:, :1] + np.float32(1e-5) * rng.uniform(0, 1, (3, clump)).astype(np.float32)
+        pos[:, 1] = pos[:, 0]
+    h = np.full(n_p, 0.5 * (1.0 + seed % 3) * (30.0 / (4.2 * max(n_p, 30))) ** (1 / 3), np.float32)
+    src = (rng.uniform(0.0, 1.0 + seed % 3, (3, n_s)) - seed).astype(np.float32)
+    return pos, h, src, rng.lognormal(0.0, 1.0, n_s) * 1e48
+
+
+@pytest.mark.parametrize("sizes", [
+    [(1, 1), (3, 2), (5, 0), (2, 7), (1, 1), (40, 3)],
+    [(0, 0), (100, 5), (0, 3), (77, 1), (0, 0)],
+    [(500, 20)],
+    [(17000, 30), (300, 17000), (16384, 4), (20000, 9)],
+    [(16390, 5, 900), (64, 5, 40), (4097, 5, 300)],
+])
+def test_batch_parts_are_the_problems_alone(S, sizes):
+    probs = [problem(s[0], s[1], b, *s[2:]) for b, s in enumerate(sizes)]
+    n_HI = [np.random.default_rng(b).uniform(0, 1e-3, s[0]).astype(np.float32)
+            for b, s in enumerate(sizes)]
+    off = np.cumsum([0] + [s[0] for s in sizes])
+    ctx = S.Context()
+    for _ in range(2):
+        ctx.build_batch(probs)
+    g = np.zeros(max(off[-1], 1), np.float32)
+    ctx.rt_solve(0.7, n_HI=np.concatenate(n_HI), gamma_out=g)
+    st = ctx.stats()
+    noff, nidx = ctx.neighbors()
+    rays = 0
+    for b, (pos, h, src, L) in enumerate(probs):
+        one = S.Context()
+        one.build_trees(pos, h, src, L)
+        ga = np.zeros(max(len(h), 1), np.float32)
+        one.rt_solve(0.7, n_HI=n_HI[b], gamma_out=ga)
+        rays += one.stats()["rays"]
+        assert np.array_equal(g[off[b]:off[b + 1]], ga[:len(h)]), b
+        if len(h) == 0:
+            continue
+        oa, ia = one.neighbors()
+        lo, hi = int(off[b]), int(off[b + 1])
+        assert np.array_equal(noff[lo:hi + 1] - noff[lo], oa), b
+        assert np.array_equal(nidx[int(noff[lo]):int(noff[hi])] - lo, ia), b
+    assert st["rays"] == rays
+
+
+def test_bad_input_names_its_part(S):
+    probs = [problem(50, 3, 1), problem(60, 4, 2), problem(10, 1, 3)]
+    for k, what in ((1, "invalid values"), (2, "non-finite particle or source position")):
+        bad = [list(p) for p in probs]
+        if k == 1:
+            bad[k][1] = bad[k][1].copy()
+            bad[k][1][7] = -1.0
+        else:
+            bad[k][2] = bad[k][2].copy()
+            bad[k][2][1, 0] = np.nan
+        ctx = S.Context()
+        with pytest.raises(S.StartError, match=f"batch part {k}: {what}"):
+            ctx.build_batch(bad)
+        ctx.build_batch(probs)   # the context is usable afterwards
