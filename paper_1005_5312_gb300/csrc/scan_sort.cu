@@ -269,18 +269,22 @@ void rs_tile_scatter(const u64 *kin, const u32 *vin, u64 *kout, u32 *vout, long 
 // Sorting up to kRankSort keys by counting: the place of an item is the
 // number of keys below its own, and of equal keys before it.  A block places
 // 32 items, its eight warps counting an eighth of each staged tile of keys
-// (every lane reads the same key: a broadcast).  The count is n^2 comparisons,
-// but in one launch over the whole chip: 8 us at 2 k keys, where eight radix
-// passes by one block took 55 us; the four passes of a larger sort take 90 us
-// at 23 k keys.  blockIdx.y: the problem of a batch; problems with more keys
-// are left to the radix passes.
+// (every lane reads the same keys: a broadcast) -- first the leading 32 bits
+// alone, four keys per read, then, where other keys share an item's leading
+// bits, those keys in full.  The count is n^2 comparisons, but in one launch
+// over the whole chip: 5 us at 2 k keys, where eight radix passes by one block
+// took 55 us; the four passes of a larger sort take 90 us at 23 k keys.  On
+// sixteen problems of 3 to 12 k keys: 346 us with full keys throughout, against
+// 218 us.  blockIdx.y: the problem of a batch; problems with more keys are
+// left to the radix passes.
 constexpr long long kRankSort = 16384;
-constexpr int kRankTile = 2048;
+constexpr int kRankTile = 4096;
+constexpr int kKeyHigh = 32, kKeyLow = 3 * kLevels - kKeyHigh;
 
 __global__ void __launch_bounds__(256) k_rank_sort(const u64 *keys, int n_all, Segs segs,
                                                    u64 *sorted, u32 *perm)
 {
-    __shared__ __align__(16) u64 tile[kRankTile];
+    __shared__ __align__(16) u32 tile[kRankTile];
     __shared__ u32 part[8][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int i = blockIdx.x * 32 + lane;
@@ -291,21 +295,36 @@ __global__ void __launch_bounds__(256) k_rank_sort(const u64 *keys, int n_all, S
         const int n = (int)m;
         const u64 *kin = keys + lo;
         const u64 key = i < n ? kin[i] : 0ull;
-        u32 below = 0;
+        const u32 high = (u32)(key >> kKeyLow);
+        u32 below = 0, same = 0;
         for (int t0 = 0; t0 < n; t0 += kRankTile) {
+            const int len = min(kRankTile, n - t0);
+            const int per = (len + 31) / 32 * 4;   // keys per warp, a multiple of four
             __syncthreads();
-            for (int j = threadIdx.x; j < kRankTile; j += 256)
-                tile[j] = t0 + j < n ? kin[t0 + j] : ~0ull;   // above every key
+            for (int j = threadIdx.x; j < per * 8; j += 256)
+                tile[j] = j < len ? (u32)(kin[t0 + j] >> kKeyLow) : 0xffffffffu;   // padding
             __syncthreads();
-            const int j0 = w * (kRankTile / 8);
+            // the padding counts as neither below nor, for items that are not at
+            // the very top of the range, the same (those take the full pass)
+            const uint4 *t4 = reinterpret_cast<const uint4 *>(tile + w * per);
 #pragma unroll 4
-            for (int j = 0; j < kRankTile / 8; j += 2) {
-                const ulonglong2 q = *reinterpret_cast<const ulonglong2 *>(&tile[j0 + j]);
-                const int g = t0 + j0 + j;
-                below += q.x < key || (q.x == key && g < i);
-                below += q.y < key || (q.y == key && g + 1 < i);
+            for (int j = 0; j < per / 4; ++j) {
+                const uint4 q = t4[j];
+                below += (q.x < high) + (q.y < high) + (q.z < high) + (q.w < high);
+                same += (q.x == high) + (q.y == high) + (q.z == high) + (q.w == high);
             }
         }
+        part[w][lane] = same;
+        __syncthreads();
+        same = 0;
+        for (int k = 0; k < 8; ++k) same += part[k][lane];
+        if (__any_sync(0xffffffffu, i < n && same > 1u)) {   // alike in all warps
+            for (int j = w; j < n; j += 8) {
+                const u64 q = kin[j];
+                if ((u32)(q >> kKeyLow) == high) below += q < key || (q == key && j < i);
+            }
+        }
+        __syncthreads();
         part[w][lane] = below;
         __syncthreads();
         if (w == 0 && i < n) {
@@ -321,7 +340,6 @@ __global__ void __launch_bounds__(256) k_rank_sort(const u64 *keys, int n_all, S
 // Completes an order by the leading kKeyHigh bits: each run of equal leading
 // bits is sorted by insertion (stable) by the thread at its first item; a run
 // of more than kRunMax items is counted in `longer` and left.
-constexpr int kKeyHigh = 32, kKeyLow = 3 * kLevels - kKeyHigh;
 constexpr int kRunMax = 32;
 
 __global__ void k_sort_runs(u64 *keys, u32 *vals, long long n, u32 *longer)
