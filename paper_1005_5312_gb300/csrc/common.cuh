@@ -165,7 +165,8 @@ struct start_ctx {
     // solve workspace
     st::DBuf lcount;  // u32 per target
     st::DBuf loff;    // u64 [np + 1]
-    st::DBuf w_scratch, w_over;   // one-walk lists: kWalkRow ids per target; longer rows
+    st::DBuf w_scratch, w_over;   // one-walk lists: the parts' ids; parts with more of them
+    st::DBuf w_off;               // u64 offsets of the parts
     st::DBuf ctr_save;            // counters before a memoised-march attempt (retries)
     bool walk_scratch = false;    // the last count walk also filled w_scratch
     unsigned long long walk_nover = 0;

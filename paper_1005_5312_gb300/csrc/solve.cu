@@ -115,7 +115,7 @@ struct SlotRows {
 // (tree tag, node id of the accepted cell or of the leaf holding the member),
 // so every target's row is sorted by it.  MODE 0 counts, 1 writes raw
 // entries (tree tag | member flag | id), 2 writes canonical ids, 3 counts and
-// writes the first kWalkRow canonical ids into a fixed-size scratch row.
+// writes the first canonical ids into a fixed-size scratch row.
 template <int MODE, class Rows>
 __device__ __forceinline__ void walk_tree(const TreeView &t, float4 p, float th2f, double th2d,
                                           float cmag, u32 self, u32 tag, CanonBase cb, u32 &c,
@@ -141,7 +141,7 @@ __device__ __forceinline__ void walk_tree(const TreeView &t, float4 p, float th2
         int a = accept_32(b, th2f, p.x, p.y, p.z, cmag);
         if (a < 0) {
             a = accept_64(t.cube + 4 * (size_t)n, th2d, p.x, p.y, p.z) ? 1 : 0;
-            ++fb;
+            if (n >= t.lo) ++fb;   // cells before the range belong to another walk's
         }
         const bool in = n >= t.lo;
         if (a) {
@@ -251,13 +251,60 @@ __device__ __forceinline__ void walk_tree_warp(const TreeView &t, float4 p, bool
     }
 }
 
-constexpr u32 kWalkRow = 1024;                 // scratch row of the one-walk lists
-constexpr size_t kWalkScratchMax = 1ull << 30;   // bytes: larger problems count first
+// One-walk lists: ids kept per target, at least kWalkRow and, where the scratch
+// stays within kWalkScratchMax bytes, up to kWalkRowMax; larger problems (whose
+// kWalkRow ids per target exceed it) count first.
+constexpr u32 kWalkRow = 1024, kWalkRowMax = 4096;
+constexpr size_t kWalkScratchMax = 2ull << 30;
 
-// Targets [t0, t1), or when only is set the listed targets only[0, t1 - t0)
-// that lie in [lo, hi) (MODE 2).  MODE 3: the row of target i goes to
-// ent[(i - t0) kWalkRow ...], its length to cnt[i], and targets with longer
-// rows are appended to over[].
+// A target's walk cut into `n` parts, each its own range of depth-first cells
+// and its own thread, so that a row is the parts' rows one after the other.
+// Half of a row lies around the target in a tree that holds it (the emitters):
+// the parts end at the target's own leaf and at the cells of its ancestor
+// `climb` levels up; other trees are cut evenly.
+constexpr int kWalkParts = 4;
+
+struct WalkParts {
+    int n = 1;
+    u32 cap = kWalkRow;               // ids kept per part by the counting walk
+    const u32 *leaf_e = nullptr, *parent_e = nullptr;
+    int climb = 0;
+};
+
+__device__ __forceinline__ void walk_part(const WalkParts &w, TreeView &st_, TreeView &et_,
+                                          long long i, int p)
+{
+    if (w.n == 1) return;
+    if (et_.n == 0) {
+        u32 a = 0, b = st_.n;
+        if (st_.trange) {
+            const uint2 r = st_.trange[i];
+            a = r.x;
+            b = r.y;
+        }
+        const u32 len = b - a;
+        st_.lo = a + (u32)((u64)len * p / w.n);
+        st_.hi = a + (u32)((u64)len * (p + 1) / w.n);
+        return;
+    }
+    const u32 own = w.leaf_e[i];
+    u32 a = own;
+    for (int k = 0; k < w.climb; ++k) {
+        const u32 up = w.parent_e[a];
+        if (up == kNone) break;
+        a = up;
+    }
+    const u32 last = et_.meta[a].x;
+    if (p > 0) st_.hi = 0u;   // the point sources go with the first part
+    et_.lo = p == 0 ? 0u : p == 1 ? a : p == 2 ? own : last;
+    et_.hi = p == 0 ? a : p == 1 ? own : p == 2 ? last : et_.n;
+}
+
+// Targets [t0, t1), part blockIdx.y of each, or when only is set the listed
+// parts of targets only[0, t1 - t0) (target x parts + part) of targets in
+// [lo, hi) (MODE 2).  off and cnt are indexed by part.  MODE 3: the ids of a
+// part go to ent[part x cap ...], their number to cnt, and longer parts are
+// appended to over[].
 template <int MODE>
 __global__ void __launch_bounds__(128) k_walk(const float4 *pq, long long t0, long long t1,
                                               TreeView st_, TreeView et_, CanonBase scb,
@@ -266,28 +313,32 @@ __global__ void __launch_bounds__(128) k_walk(const float4 *pq, long long t0, lo
                                               u32 *ent, u32 *tgt, u32 *ord,
                                               unsigned long long *fb_total, const u32 *only,
                                               long long lo, long long hi, u32 *over,
-                                              unsigned long long *n_over)
+                                              unsigned long long *n_over, WalkParts parts)
 {
     constexpr bool FILL = MODE != 0;
     constexpr bool COUNT = MODE == 0 || MODE == 3;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     long long i = -1;
+    int part = blockIdx.y;
     if (!only) {
         if (t0 + t < t1) i = t0 + t;
     } else if (t < t1 - t0) {
-        const long long k = (long long)only[t];
+        const long long k = (long long)only[t] / parts.n;
+        part = (int)(only[t] % parts.n);
         if (k >= lo && k < hi) i = k;
     }
+    const long long v = i * parts.n + part;   // this part's index
+    if ((MODE == 2 || MODE == 3) && i >= 0) walk_part(parts, st_, et_, i, part);
     unsigned fb = 0;
     const bool live = i >= 0;
     // the warp-cooperative walk (both trees or none; not over a batch's forest)
     const bool warp = st_.level != nullptr && st_.trange == nullptr;
     u32 c = 0;
     const u64 w0 = !live ? 0ull
-                         : (MODE == 3 ? (u64)(i - t0) * kWalkRow : (FILL ? off[i] - base : 0ull));
+                         : (MODE == 3 ? (u64)v * parts.cap : (FILL ? off[v] - base : 0ull));
     u64 w = w0;
     const u64 wend = !live ? 0ull
-                           : (MODE == 3 ? w0 + kWalkRow : (FILL ? off[i + 1] - base : 0ull));
+                           : (MODE == 3 ? w0 + parts.cap : (FILL ? off[v + 1] - base : 0ull));
     if (live || warp) {                         // warp: every lane takes part
         float4 p = live ? pq[i] : make_float4(0.f, 0.f, 0.f, 0.f);
         const u32 self = live ? (u32)i : kNone;
@@ -320,10 +371,10 @@ __global__ void __launch_bounds__(128) k_walk(const float4 *pq, long long t0, lo
     }
     if (live) {
         if (MODE == 0) {
-            cnt[i] = c;
+            cnt[v] = c;
         } else if (MODE == 3) {
-            cnt[i] = (u32)(w - w0);
-            if (w - w0 > kWalkRow) over[atomicAdd(n_over, 1ull)] = (u32)i;
+            cnt[v] = (u32)(w - w0);
+            if (w - w0 > parts.cap) over[atomicAdd(n_over, 1ull)] = (u32)v;
         } else if (w != wend) {
             atomicAdd(fb_total, 1ull);   // internal-error counter in FILL
         }
@@ -705,42 +756,91 @@ static void launch_march(const MarchArgs &a, cudaStream_t s, int nsm)
     k_march<G><<<(unsigned)blocks, 256, 0, s>>>(a);
 }
 
+// The parts the one-walk lists cut every target's walk into.  A walk is a chain
+// of dependent reads, and at the sizes that use one-walk lists (up to 2^19
+// targets) one thread per target leaves the SMs waiting: 225 us for 23 k
+// targets and 430 cells, 0.95 ms for 43 k emitting targets, 0.83 ms for 262 k
+// targets and 1510 cells, against 80 us, 0.70 and 0.69 ms in four parts (the
+// rows longer than 1024, walked again by a few threads, took another 1.1 ms of
+// the second).  Trees below kWalkCells cells per problem are walked whole (16
+// sources: 57 us either way, and a launch less), and so is the warp-cooperative
+// walk, which shares one traversal per warp.
+constexpr long long kWalkCells = 128;
+
+static WalkParts walk_parts(start_ctx *c)
+{
+    WalkParts w;
+    const long long members = c->ns + (c->walk_emit ? c->np : 0);
+    size_t cap = kWalkScratchMax / sizeof(u32) / (size_t)(c->np ? c->np : 1);
+    cap = std::min<size_t>(std::max<size_t>(cap, kWalkRow), kWalkRowMax);
+    const long long cells = c->stree.n + (c->walk_emit ? c->et.n : 0);
+    if (!c->p.walk_warp && cells >= kWalkCells * std::max(1, c->nbatch)) w.n = kWalkParts;
+    // a row holds at most one cell or member per member
+    w.cap = (u32)std::min<size_t>(cap / w.n, (size_t)std::max<long long>(members, 4));
+    if (c->walk_emit) {
+        w.leaf_e = c->et.leafof.as<u32>();
+        w.parent_e = c->et.parent.as<u32>();
+        w.climb = (int)c->et.lvl_off.size() / 2;
+    }
+    return w;
+}
+
+// Row offsets from the parts' offsets.
+__global__ void k_row_offsets(const u64 *poff, long long np, int parts, u64 *off)
+{
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i <= np) off[i] = poff[i * parts];
+}
+
 // Interaction-list counts of every target and their exclusive scan (loff).
 // one_walk (memoised march, scratch within kWalkScratchMax): the counting
-// walk also writes the canonical ids into a scratch row per target, so the
-// slot fill becomes a copy (walk_fill_slots).
+// walk also writes the canonical ids into a scratch row per part of a target,
+// so the slot fill becomes a copy (walk_fill_slots).
 static int walk_count(start_ctx *c, float theta, const TreeView &sv, const TreeView &ev,
                       unsigned long long *total, bool one_walk = false)
 {
     long long np = c->np;
     cudaStream_t s = c->stream;
     unsigned long long *ctr = c->counters.as<unsigned long long>();
-    ST_TRY(ensure(c->lcount, np * sizeof(u32)));
     ST_TRY(ensure(c->loff, (np + 1) * sizeof(u64)));
     c->walk_scratch = false;
     c->walk_nover = 0;
+    const WalkParts parts = walk_parts(c);
+    const long long nv = np * parts.n;
     one_walk = one_walk && (size_t)np * kWalkRow * sizeof(u32) <= kWalkScratchMax;
-    if (one_walk && (ensure(c->w_scratch, (size_t)np * kWalkRow * sizeof(u32)) ||
-                     ensure(c->w_over, (size_t)np * sizeof(u32))))
+    if (one_walk && (ensure(c->w_scratch, (size_t)nv * parts.cap * sizeof(u32)) ||
+                     ensure(c->w_over, (size_t)nv * sizeof(u32)) ||
+                     (parts.n > 1 && ensure(c->w_off, (nv + 1) * sizeof(u64)))))
         one_walk = false;   // no room: count, then fill
+    ST_TRY(ensure(c->lcount, (one_walk ? nv : np) * sizeof(u32)));
     if (one_walk) {
         u32 SN = (u32)c->stree.n, NS = (u32)c->ns, EN = (u32)(c->walk_emit ? c->et.n : 0);
         CanonBase scb{0u, SN}, ecb{SN + NS, SN + NS + EN};
         ST_CUDA(c, cudaMemsetAsync(ctr + C_WALK_OVER, 0, sizeof(unsigned long long), s));
-        k_walk<3><<<grid_for(np, 128), 128, 0, s>>>(
+        k_walk<3><<<dim3(grid_for(np, 128), parts.n), 128, 0, s>>>(
             c->pq.as<float4>(), 0, np, sv, ev, scb, ecb, theta * theta,
             (double)theta * (double)theta, c->fr.cmag, c->lcount.as<u32>(), nullptr, 0ull,
             c->w_scratch.as<u32>(), nullptr, nullptr, ctr + C_WALK_FB, nullptr, 0, 0,
-            c->w_over.as<u32>(), ctr + C_WALK_OVER);
+            c->w_over.as<u32>(), ctr + C_WALK_OVER, parts);
+        ST_CUDA(c, cudaGetLastError());
+        DBuf &po = parts.n > 1 ? c->w_off : c->loff;   // the parts' offsets
+        ST_TRY(exclusive_scan_u32_to_u64(c, c->lcount.as<u32>(), po.as<u64>(), nv));
+        if (parts.n > 1) {
+            k_row_offsets<<<grid_for(np + 1, 256), 256, 0, s>>>(po.as<u64>(), np, parts.n,
+                                                                c->loff.as<u64>());
+            ++c->launches;
+        }
     } else {
         k_walk<0><<<grid_for(np, 128), 128, 0, s>>>(
             c->pq.as<float4>(), 0, np, sv, ev, CanonBase{}, CanonBase{}, theta * theta,
             (double)theta * (double)theta, c->fr.cmag, c->lcount.as<u32>(), nullptr, 0ull,
-            nullptr, nullptr, nullptr, ctr + C_WALK_FB, nullptr, 0, 0, nullptr, nullptr);
+            nullptr, nullptr, nullptr, ctr + C_WALK_FB, nullptr, 0, 0, nullptr, nullptr,
+            WalkParts{});
+        ST_CUDA(c, cudaGetLastError());
+        ST_TRY(exclusive_scan_u32_to_u64(c, c->lcount.as<u32>(), c->loff.as<u64>(), np));
     }
     ++c->launches;
     ST_CUDA(c, cudaGetLastError());
-    ST_TRY(exclusive_scan_u32_to_u64(c, c->lcount.as<u32>(), c->loff.as<u64>(), np));
     ST_CUDA(c, cudaMemcpyAsync(total, c->loff.as<u64>() + np, sizeof(*total),
                                cudaMemcpyDeviceToHost, s));
     if (one_walk)
@@ -760,7 +860,7 @@ static int walk_fill(start_ctx *c, float theta, const TreeView &sv, const TreeVi
         c->pq.as<float4>(), t0, t1, sv, ev, CanonBase{}, CanonBase{}, theta * theta,
         (double)theta * (double)theta, c->fr.cmag, nullptr, c->loff.as<u64>(), base,
         c->pent.as<u32>(), c->ptgt.as<u32>(), c->pord.as<u32>(), ctr + C_INTERNAL, nullptr, 0, 0,
-        nullptr, nullptr);
+        nullptr, nullptr, WalkParts{});
     ++c->launches;
     return cuda_check(c, cudaGetLastError(), "k_walk");
 }
@@ -774,28 +874,32 @@ static TreeView emitter_view(start_ctx *c);
 // written straight into the first slots (the vid and ord buffers, which the
 // caller sized); the first hop knows each row's target, so the pair slots'
 // particle is not stored.
-// The rows of targets [t0, t1) from the one-walk scratch (rows of at most
-// kWalkRow ids; longer rows were filled in place by a second walk), copied
-// to their slots with their order keys, one warp per target.
+// The rows of targets [t0, t1) from the one-walk scratch (parts of at most
+// cap ids; longer parts were filled in place by a second walk), copied to
+// their slots with their order keys, one warp per target.
 __global__ void k_walk_compact(long long t0, long long t1, u64 base, const u32 *cnt,
-                               const u64 *off, const u32 *scratch, u32 *vid, u32 SN, u32 NS,
-                               u32 EN, const u32 *leaf_s, const u32 *leaf_e, u32 *key)
+                               const u64 *off, int parts, u32 cap, const u32 *scratch, u32 *vid,
+                               u32 SN, u32 NS, u32 EN, const u32 *leaf_s, const u32 *leaf_e,
+                               u32 *key)
 {
     const long long i = t0 + ((long long)blockIdx.x * blockDim.x + threadIdx.x) / 32;
     const int lane = threadIdx.x & 31;
     if (i >= t1) return;
-    const u32 c = cnt[i];
-    const u64 o = off[i] - base;
-    const u32 *src = scratch + (size_t)i * kWalkRow;
-    for (u32 k = lane; k < c; k += 32) {
-        u32 v = c <= kWalkRow ? src[k] : vid[o + k];
-        if (c <= kWalkRow) vid[o + k] = v;
-        u32 q;
-        if (v < SN) q = v;
-        else if ((v -= SN) < NS) q = leaf_s[v];
-        else if ((v -= NS) < EN) q = 0x80000000u | v;
-        else q = 0x80000000u | leaf_e[v - EN];
-        key[o + k] = q;
+    for (int p = 0; p < parts; ++p) {
+        const long long r = i * parts + p;
+        const u32 c = cnt[r];
+        const u64 o = off[r] - base;
+        const u32 *src = scratch + (size_t)r * cap;
+        for (u32 k = lane; k < c; k += 32) {
+            u32 v = c <= cap ? src[k] : vid[o + k];
+            if (c <= cap) vid[o + k] = v;
+            u32 q;
+            if (v < SN) q = v;
+            else if ((v -= SN) < NS) q = leaf_s[v];
+            else if ((v -= NS) < EN) q = 0x80000000u | v;
+            else q = 0x80000000u | leaf_e[v - EN];
+            key[o + k] = q;
+        }
     }
 }
 
@@ -806,19 +910,21 @@ int walk_fill_slots(start_ctx *c, float theta, long long t0, long long t1, u64 b
     u32 SN = (u32)c->stree.n, NS = (u32)c->ns, EN = (u32)(c->walk_emit ? c->et.n : 0);
     CanonBase scb{0u, SN}, ecb{SN + NS, SN + NS + EN};
     if (c->walk_scratch) {
-        if (c->walk_nover) {   // the longer rows, walked again straight into their slots
+        const WalkParts parts = walk_parts(c);
+        const u64 *po = parts.n > 1 ? c->w_off.as<u64>() : c->loff.as<u64>();
+        if (c->walk_nover) {   // the longer parts, walked again straight into their slots
             long long m = (long long)c->walk_nover;
             k_walk<2><<<grid_for(m, 128), 128, 0, c->stream>>>(
                 c->pq.as<float4>(), 0, m, source_view(c), emitter_view(c), scb, ecb,
                 theta * theta, (double)theta * (double)theta, c->fr.cmag, nullptr,
-                c->loff.as<u64>(), base, c->m_vid.as<u32>(), nullptr, nullptr, ctr + C_INTERNAL,
-                c->w_over.as<u32>(), t0, t1, nullptr, nullptr);
+                po, base, c->m_vid.as<u32>(), nullptr, nullptr, ctr + C_INTERNAL,
+                c->w_over.as<u32>(), t0, t1, nullptr, nullptr, parts);
             ++c->launches;
         }
         k_walk_compact<<<grid_for((t1 - t0) * 32, 256), 256, 0, c->stream>>>(
-            t0, t1, base, c->lcount.as<u32>(), c->loff.as<u64>(), c->w_scratch.as<u32>(),
-            c->m_vid.as<u32>(), SN, NS, EN, c->stree.leafof.as<u32>(), c->et.leafof.as<u32>(),
-            c->m_ord.as<u32>());
+            t0, t1, base, c->lcount.as<u32>(), po, parts.n, parts.cap,
+            c->w_scratch.as<u32>(), c->m_vid.as<u32>(), SN, NS, EN, c->stree.leafof.as<u32>(),
+            c->et.leafof.as<u32>(), c->m_ord.as<u32>());
         ++c->launches;
         return cuda_check(c, cudaGetLastError(), "k_walk_compact");
     }
@@ -828,7 +934,7 @@ int walk_fill_slots(start_ctx *c, float theta, long long t0, long long t1, u64 b
         c->pq.as<float4>(), t0, t1, source_view(c), emitter_view(c), scb, ecb, theta * theta,
         (double)theta * (double)theta, c->fr.cmag, nullptr, c->loff.as<u64>(), base,
         c->m_vid.as<u32>(), nullptr, c->m_ord.as<u32>(), ctr + C_INTERNAL, nullptr, 0, 0, nullptr,
-        nullptr);
+        nullptr, WalkParts{});
     ++c->launches;
     return cuda_check(c, cudaGetLastError(), "k_walk");
 }
@@ -1126,7 +1232,7 @@ static int run_grouped(start_ctx *c, float theta, float *gout_dev, long long max
             c->pq.as<float4>(), 0, np, source_view(c), emitter_view(c), CanonBase{}, CanonBase{},
             theta * theta, (double)theta * (double)theta, c->fr.cmag, c->lcount.as<u32>(),
             nullptr, 0ull, nullptr, nullptr, nullptr, ctr + C_WALK_FB_GROUP, nullptr, 0, 0,
-            nullptr, nullptr);
+            nullptr, nullptr, WalkParts{});
         ++c->launches;
         ST_CUDA(c, cudaGetLastError());
         ST_TRY(exclusive_scan_u32_to_u64(c, c->lcount.as<u32>(), c->loff.as<u64>(), np));
@@ -1203,7 +1309,7 @@ int run_solve(start_ctx *c, float theta, float *gout_dev)
     std::vector<unsigned long long> hist;
     bool grouped = false;
     unsigned long long total = 0;
-    if (memo && (size_t)np * kWalkRow * sizeof(u32) > kWalkScratchMax) {
+    if (memo && (size_t)np * kWalkRow * sizeof(u32) > kWalkScratchMax) {   // above 2^19 targets
         // a large problem: the sampled histogram first; a solve that clearly
         // needs groups skips the counting walk over every target
         ST_TRY(group_histogram(c, theta, hist));
