@@ -406,13 +406,20 @@ __device__ __forceinline__ int accept_32(float4 box, float th2, float px, float 
     // walk must take bit-identical decisions
     float l = box.w;
     float hx = __fadd_rn(box.x, l), hy = __fadd_rn(box.y, l), hz = __fadd_rn(box.z, l);
-    float dx = px < box.x ? __fsub_rn(box.x, px) : (px > hx ? __fsub_rn(px, hx) : 0.f);
-    float dy = py < box.y ? __fsub_rn(box.y, py) : (py > hy ? __fsub_rn(py, hy) : 0.f);
-    float dz = pz < box.z ? __fsub_rn(box.z, pz) : (pz > hz ? __fsub_rn(pz, hz) : 0.f);
+    float dx = fmaxf(fmaxf(__fsub_rn(box.x, px), __fsub_rn(px, hx)), 0.f);
+    float dy = fmaxf(fmaxf(__fsub_rn(box.y, py), __fsub_rn(py, hy)), 0.f);
+    float dz = fmaxf(fmaxf(__fsub_rn(box.z, pz), __fsub_rn(pz, hz)), 0.f);
     float d2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
     float l2 = __fmul_rn(l, l);
     float t = __fmul_rn(th2, d2);
     float m = __fsub_rn(t, l2);
+    // a wide margin decides without the bound below: for d >= cmag / 600 that
+    // is at most 2u (3.4641 x 1801 + 9) (t + l2) < 7.5e-4 (t + l2)
+    if (__fmul_rn(d2, 360000.f) >= __fmul_rn(cmag, cmag)) {
+        const float w = __fmul_rn(1e-3f, __fadd_rn(t, l2));
+        if (m > w) return 1;
+        if (m < -w) return 0;
+    }
     // error bound: coordinates of the cube and of its far side carry up to
     // 3u*cmag each; every rounded operation adds u of its result.
     float d = __fsqrt_rn(d2);

@@ -70,44 +70,38 @@ struct RawRows {
 struct SlotRows {
     u32 *ent;             // canonical ids
     u32 *key = nullptr;   // their order keys, when set (the slots' keys)
-    u64 g = 0;            // group (w / 4) of the buffered entries
-    int lo = 0, hi = 0;   // buffered positions [lo, hi) of the group
+    u64 at = 0;           // place of the next entry
+    u32 held = 0;         // entries in the buffer (the last ones, oldest first at 4 - held)
     u32 e0 = 0, e1 = 0, e2 = 0, e3 = 0, k0 = 0, k1 = 0, k2 = 0, k3 = 0;
-    __device__ __forceinline__ static void store4(u32 *dst, u64 b, int lo, int hi, u32 v0, u32 v1,
-                                                  u32 v2, u32 v3)
+    __device__ __forceinline__ void store(u64 b, u32 v0, u32 v1, u32 v2, u32 v3, u32 *dst) const
     {
-        if (lo == 0 && hi == 4) {
-            *reinterpret_cast<uint4 *>(dst + b) = make_uint4(v0, v1, v2, v3);
-        } else {
-            if (lo <= 0 && 0 < hi) dst[b] = v0;
-            if (lo <= 1 && 1 < hi) dst[b + 1] = v1;
-            if (lo <= 2 && 2 < hi) dst[b + 2] = v2;
-            if (lo <= 3 && 3 < hi) dst[b + 3] = v3;
-        }
+        // the held entries end at place b
+        if (held >= 4) dst[b - 4] = v0;
+        if (held >= 3) dst[b - 3] = v1;
+        if (held >= 2) dst[b - 2] = v2;
+        if (held >= 1) dst[b - 1] = v3;
     }
     __device__ __forceinline__ void flush()
     {
-        if (hi <= lo) return;
-        u64 b = g * 4;
-        store4(ent, b, lo, hi, e0, e1, e2, e3);
-        if (key) store4(key, b, lo, hi, k0, k1, k2, k3);
-        lo = hi = 0;
+        store(at, e0, e1, e2, e3, ent);
+        if (key) store(at, k0, k1, k2, k3, key);
+        held = 0;
     }
     __device__ __forceinline__ void put(u64 w, u32 e, u32 kk)
     {
-        u64 gw = w >> 2;
-        int k = (int)(w & 3);
-        if (hi > lo && gw != g) flush();
-        if (hi <= lo) {
-            g = gw;
-            lo = k;
+        e0 = e1, e1 = e2, e2 = e3, e3 = e;
+        if (key) k0 = k1, k1 = k2, k2 = k3, k3 = kk;
+        ++held;
+        at = w + 1;
+        if ((at & 3) == 0) {   // the end of an aligned group
+            if (held == 4) {
+                *reinterpret_cast<uint4 *>(ent + (at - 4)) = make_uint4(e0, e1, e2, e3);
+                if (key) *reinterpret_cast<uint4 *>(key + (at - 4)) = make_uint4(k0, k1, k2, k3);
+                held = 0;
+            } else {
+                flush();
+            }
         }
-        if (k == 0) e0 = e, k0 = kk;
-        if (k == 1) e1 = e, k1 = kk;
-        if (k == 2) e2 = e, k2 = kk;
-        if (k == 3) e3 = e, k3 = kk;
-        hi = k + 1;
-        if (hi == 4) flush();
     }
 };
 
@@ -131,45 +125,70 @@ __device__ __forceinline__ void walk_tree(const TreeView &t, float4 p, float th2
         n = r.x;
         end = r.y < end ? r.y : end;
     }
+    // the records of the cell after the current one's subtree are requested
+    // before its test: most cells are accepted, leaves or outside the range, and
+    // the walk is a chain of these reads (filling walks of the 128^3 diffuse step:
+    // 56.0 against 50.8 ms; 48.0 with SlotRows shifting its buffer)
+    uint4 mt = make_uint4(0u, 0u, 0u, 0u);
+    float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (n < end) {
+        mt = t.meta[n];
+        b = t.box[n];
+    }
     while (n < end) {
-        uint4 mt = t.meta[n];
-        if (mt.x <= t.lo) {   // the whole subtree lies before the range
-            n = mt.x;
-            continue;
+        const u32 skip = mt.x;
+        uint4 mt2 = mt;
+        float4 b2 = b;
+        if (skip < end) {
+            mt2 = t.meta[skip];
+            b2 = t.box[skip];
         }
-        float4 b = t.box[n];
-        int a = accept_32(b, th2f, p.x, p.y, p.z, cmag);
-        if (a < 0) {
-            a = accept_64(t.cube + 4 * (size_t)n, th2d, p.x, p.y, p.z) ? 1 : 0;
-            if (n >= t.lo) ++fb;   // cells before the range belong to another walk's
-        }
-        const bool in = n >= t.lo;
-        if (a) {
-            if (in && FILL) {
-                if (w < wend) {   // never past this row
-                    u32 e = (MODE >= 2) ? ((mt.w && mt.z == 1u) ? cb.memb0 + mt.y : cb.node0 + n)
-                                        : (n | tag);
-                    rows.put(w, e, okey | n);
-                }
-                ++w;
-            } else if (in) {
-                ++c;
+        bool open = false;
+        if (skip > t.lo) {   // else the whole subtree lies before the range
+            int a = accept_32(b, th2f, p.x, p.y, p.z, cmag);
+            if (a < 0) {
+                a = accept_64(t.cube + 4 * (size_t)n, th2d, p.x, p.y, p.z) ? 1 : 0;
+                if (n >= t.lo) ++fb;   // cells before the range belong to another walk's
             }
-            n = mt.x;
-        } else if (mt.w) {
-            for (u32 r = mt.y; in && r < mt.y + mt.z; ++r) {
-                if (r == self) continue;
-                if (FILL) {
-                    if (w < wend)
-                        rows.put(w, (MODE >= 2) ? cb.memb0 + r : (kEntrySrc | tag | r), okey | n);
+            const bool in = n >= t.lo;
+            if (a) {
+                if (in && FILL) {
+                    if (w < wend) {   // never past this row
+                        u32 e = (MODE >= 2) ? ((mt.w && mt.z == 1u) ? cb.memb0 + mt.y
+                                                                    : cb.node0 + n)
+                                            : (n | tag);
+                        rows.put(w, e, okey | n);
+                    }
                     ++w;
-                } else {
+                } else if (in) {
                     ++c;
                 }
+            } else if (mt.w) {
+                for (u32 r = mt.y; in && r < mt.y + mt.z; ++r) {
+                    if (r == self) continue;
+                    if (FILL) {
+                        if (w < wend)
+                            rows.put(w, (MODE >= 2) ? cb.memb0 + r : (kEntrySrc | tag | r),
+                                     okey | n);
+                        ++w;
+                    } else {
+                        ++c;
+                    }
+                }
+            } else {
+                open = true;
             }
-            n = mt.x;
-        } else {
+        }
+        if (open) {
             n = n + 1;
+            if (n < end) {
+                mt = t.meta[n];
+                b = t.box[n];
+            }
+        } else {
+            n = skip;
+            mt = mt2;
+            b = b2;
         }
     }
 }
@@ -792,6 +811,19 @@ __global__ void k_row_offsets(const u64 *poff, long long np, int parts, u64 *off
     if (i <= np) off[i] = poff[i * parts];
 }
 
+// Offsets of the parts and of the rows from the parts' counts (lcount).
+static int part_offsets(start_ctx *c, const WalkParts &parts)
+{
+    DBuf &po = parts.n > 1 ? c->w_off : c->loff;   // the parts' offsets
+    ST_TRY(exclusive_scan_u32_to_u64(c, c->lcount.as<u32>(), po.as<u64>(), c->np * parts.n));
+    if (parts.n > 1) {
+        k_row_offsets<<<grid_for(c->np + 1, 256), 256, 0, c->stream>>>(po.as<u64>(), c->np,
+                                                                       parts.n, c->loff.as<u64>());
+        ++c->launches;
+    }
+    return cuda_check(c, cudaGetLastError(), "k_row_offsets");
+}
+
 // Interaction-list counts of every target and their exclusive scan (loff).
 // one_walk (memoised march, scratch within kWalkScratchMax): the counting
 // walk also writes the canonical ids into a scratch row per part of a target,
@@ -823,13 +855,7 @@ static int walk_count(start_ctx *c, float theta, const TreeView &sv, const TreeV
             c->w_scratch.as<u32>(), nullptr, nullptr, ctr + C_WALK_FB, nullptr, 0, 0,
             c->w_over.as<u32>(), ctr + C_WALK_OVER, parts);
         ST_CUDA(c, cudaGetLastError());
-        DBuf &po = parts.n > 1 ? c->w_off : c->loff;   // the parts' offsets
-        ST_TRY(exclusive_scan_u32_to_u64(c, c->lcount.as<u32>(), po.as<u64>(), nv));
-        if (parts.n > 1) {
-            k_row_offsets<<<grid_for(np + 1, 256), 256, 0, s>>>(po.as<u64>(), np, parts.n,
-                                                                c->loff.as<u64>());
-            ++c->launches;
-        }
+        ST_TRY(part_offsets(c, parts));
     } else {
         k_walk<0><<<grid_for(np, 128), 128, 0, s>>>(
             c->pq.as<float4>(), 0, np, sv, ev, CanonBase{}, CanonBase{}, theta * theta,
@@ -1094,9 +1120,9 @@ __global__ void k_set_evals(unsigned long long *ctr, unsigned long long evals,
 // whenever k's walk lists v, so only the method's own boundary links leave
 // the lists -- splitting by target would cut every chain at the edge of the
 // target range.  Groups are planned from a histogram of the pairs over
-// kGroupBins equal ranges of cell index, taken on every stride-th target
-// (4 up to 4 M targets, then about a million samples: at most 64); each
-// group's exact count comes from its own counting walk, and a group that
+// kGroupBins equal ranges of cell index, taken on every stride-th target (65 k
+// samples, at least every 256th: half a million samples planned no better and
+// took 11 against 2 ms on the 128^3 diffuse step); each group's exact count comes from its own counting walk, and a group that
 // exceeds the plan by half is halved.
 constexpr int kGroupBins = 2048;
 
@@ -1171,7 +1197,7 @@ static int group_histogram(start_ctx *c, float theta, std::vector<unsigned long 
     ST_TRY(ensure(c->g_hist, kGroupBins * sizeof(unsigned long long)));
     unsigned long long *d = c->g_hist.as<unsigned long long>();
     ST_CUDA(c, cudaMemsetAsync(d, 0, kGroupBins * sizeof(unsigned long long), c->stream));
-    const int stride = (int)std::min<long long>(64, std::max<long long>(4, c->np >> 20));
+    const int stride = (int)std::min<long long>(256, std::max<long long>(4, c->np >> 16));
     const long long ns = (c->np + stride - 1) / stride;
     k_walk_hist<<<grid_for(ns, 128), 128, 0, c->stream>>>(
         c->pq.as<float4>(), c->np, stride, source_view(c), emitter_view(c), theta * theta,
