@@ -263,12 +263,15 @@ __global__ void k_gather_sources(const float *pos, Segs segs, const double *L, c
     sL[r] = Lj;
 }
 
+// (not when a value was found bad: the state stays as it was)
 __global__ void k_set_state(const float *nH_in, const double *y_in, const u32 *inv, long long n,
-                            float *nH, double *y, float4 *pq)
+                            float *nH, double *y, float4 *pq, double *Tg,
+                            const unsigned long long *bad)
 {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    if (i >= n || *bad) return;
     u32 r = inv[i];
+    Tg[r] = 1e4;
     double yy = y_in ? y_in[i] : 1.0;
     float nh = nH_in[i];
     nH[r] = nh;
@@ -296,6 +299,17 @@ static unsigned long long read_counter(start_ctx *c, int slot)
                     cudaMemcpyDeviceToHost, c->stream);
     cudaStreamSynchronize(c->stream);
     return v;
+}
+
+// The solve's error counters in one copy and one wait.
+static int finish_call(start_ctx *c, const char *internal)
+{
+    unsigned long long v[C_COUNT];
+    ST_CUDA(c, cudaMemcpyAsync(v, c->counters.p, sizeof(v), cudaMemcpyDeviceToHost, c->stream));
+    ST_CUDA(c, cudaStreamSynchronize(c->stream));
+    if (v[C_INTERNAL]) return set_err(c, START_ECUDA, internal);
+    if (v[C_CHAIN_OVF]) return set_err(c, START_ECHAIN, "a ray exceeded hop_cap");
+    return START_OK;
 }
 
 static int check_bad(start_ctx *c, const char *what)
@@ -778,13 +792,12 @@ int start_set_state(start_ctx *c, const float *n_H, const double *y)
     if (y) ST_TRY(stage_in(c, in.V, y, n * sizeof(double)));
     k_check_nonneg_f<<<grid_for(n, 256), 256, 0, c->stream>>>(in.h.as<float>(), n, ctr + C_BAD_INPUT); ++c->launches;
     if (y) { k_check_unit_d<<<grid_for(n, 256), 256, 0, c->stream>>>(in.V.as<double>(), n, ctr + C_BAD_INPUT); ++c->launches; }
-    ST_TRY(check_bad(c, "n_H or y"));
-    k_set_state<<<grid_for(n, 256), 256, 0, c->stream>>>(in.h.as<float>(), y ? in.V.as<double>() : nullptr,
-                                                        c->pinv.as<u32>(), n, c->nH.as<float>(),
-                                                        c->y.as<double>(), c->pq.as<float4>()); ++c->launches;
-    k_fill_d<<<grid_for(n, 256), 256, 0, c->stream>>>(c->Tg.as<double>(), n, 1e4); ++c->launches;
+    k_set_state<<<grid_for(n, 256), 256, 0, c->stream>>>(
+        in.h.as<float>(), y ? in.V.as<double>() : nullptr, c->pinv.as<u32>(), n, c->nH.as<float>(),
+        c->y.as<double>(), c->pq.as<float4>(), c->Tg.as<double>(), ctr + C_BAD_INPUT);
+    ++c->launches;
     ST_CUDA(c, cudaGetLastError());
-    ST_CUDA(c, cudaStreamSynchronize(c->stream));
+    ST_TRY(check_bad(c, "n_H or y"));   // waits: the inputs are the caller's again
     c->has_state = true;
     return START_OK;
 }
@@ -866,9 +879,7 @@ int start_rt_solve(start_ctx *c, const float *n_HI, float theta, float *gamma_ou
         if (resident_eligible(c)) ST_TRY(resident_build(c, theta));
     }
     if (gamma_out && !dev_out) ST_TRY(copy_out(c, gamma_out, c->stage.p, n * sizeof(float)));
-    ST_CUDA(c, cudaStreamSynchronize(c->stream));
-    if (read_counter(c, C_INTERNAL)) return set_err(c, START_ECUDA, "internal inconsistency (interaction lists)");
-    if (read_counter(c, C_CHAIN_OVF)) return set_err(c, START_ECHAIN, "a ray exceeded hop_cap");
+    ST_TRY(finish_call(c, "internal inconsistency (interaction lists)"));
     c->solved = true;
     return START_OK;
 }
@@ -972,9 +983,7 @@ int start_h2_dissociation(start_ctx *c, const float *n_H2, float theta, double k
     }
     c->kappa_LW = kappa_LW;
     ST_TRY(run_h2_dissociation(c, nd, theta, dst));
-    ST_CUDA(c, cudaStreamSynchronize(c->stream));
-    if (read_counter(c, C_INTERNAL)) return set_err(c, START_ECUDA, "internal inconsistency");
-    if (read_counter(c, C_CHAIN_OVF)) return set_err(c, START_ECHAIN, "a ray exceeded hop_cap");
+    ST_TRY(finish_call(c, "internal inconsistency"));
     if (!dev_out) ST_TRY(copy_out(c, kdis_out, dst, n * sizeof(float)));
     return START_OK;
 }

@@ -830,12 +830,21 @@ __global__ void __launch_bounds__(128) k_memo_tail(MemoArgs a, long long max_ite
     if (fbs) atomicAdd(&a.m.counters[C_MARCH_FB], fbs);
 }
 
+// Chain links of the march: the slots allocated, which the host reads only
+// after the first round (cap: all that were kept when they overflowed).
+__device__ __forceinline__ long long slot_count(const unsigned long long *nslots, long long cap)
+{
+    const long long n = (long long)*nslots;
+    return n < cap ? n : cap;
+}
+
 // Links claimed by another thread during the same launch: read the slot the
 // claimant wrote (visible after the launch boundary).
 __global__ void k_memo_resolve(MemoArgs a)
 {
+    // after the tail: every slot from the frontier on
     const u32 fbase = a.dlv ? (u32)a.dlv[0] : a.fbase;
-    const long long nf = a.dlv ? (long long)a.dlv[1] : a.nf;
+    const long long nf = a.dlv ? (long long)a.dlv[1] : slot_count(a.nslots, a.cap) - fbase;
     for (long long it = (long long)blockIdx.x * blockDim.x + threadIdx.x; it < nf;
          it += (long long)gridDim.x * blockDim.x) {
         u32 s = a.fr ? a.fr[it] : fbase + (u32)it;
@@ -917,8 +926,10 @@ constexpr int kGammaU = 2;   // pairs per lane in flight in the rows of a group
 
 // The march's states widened for the counting form: one link, no
 // compensation term.
-__global__ void k_memo_widen(long long n, const uint2 *__restrict__ st, uint4 *__restrict__ w)
+__global__ void k_memo_widen(const unsigned long long *nslots, long long cap,
+                             const uint2 *__restrict__ st, uint4 *__restrict__ w)
 {
+    const long long n = slot_count(nslots, cap);
     for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < n;
          s += (long long)gridDim.x * blockDim.x) {
         const uint2 v = st[s];
@@ -931,11 +942,13 @@ __global__ void k_memo_widen(long long n, const uint2 *__restrict__ st, uint4 *_
 // rounds: plain stores, stream-ordered launches of the same grid), and its
 // slots whose chains are still open after this round.
 template <int G, int R>
-__global__ void __launch_bounds__(256) k_memo_jump8(long long n, const uint2 *__restrict__ st,
+__global__ void __launch_bounds__(256) k_memo_jump8(const unsigned long long *nslots, long long cap,
+                                                    const uint2 *__restrict__ st,
                                                     uint2 *__restrict__ st2,
                                                     unsigned long long *ctr,
                                                     unsigned long long *part)
 {
+    const long long n = slot_count(nslots, cap);
     const long long s0 = (long long)blockIdx.x * (256 * R) + threadIdx.x;
     const u32 n32 = (u32)n;
     uint2 me[R];
@@ -992,11 +1005,14 @@ __global__ void __launch_bounds__(256) k_memo_jump8(long long n, const uint2 *__
 
 // One round of the counting form; part[2 b ..] of block b as above.
 template <int G>
-__global__ void __launch_bounds__(256, 2) k_memo_jump(long long n, const uint4 *__restrict__ st,
-                                                    uint4 *__restrict__ st2,
-                                                    unsigned long long *ctr,
-                                                    unsigned long long *part)
+__global__ void __launch_bounds__(256, 2) k_memo_jump(const unsigned long long *nslots,
+                                                       long long cap,
+                                                       const uint4 *__restrict__ st,
+                                                       uint4 *__restrict__ st2,
+                                                       unsigned long long *ctr,
+                                                       unsigned long long *part)
 {
+    const long long n = slot_count(nslots, cap);
     const long long s0 = (long long)blockIdx.x * (256 * kJumpR) + threadIdx.x;
     uint4 me[kJumpR];
     unsigned go = 0;   // bit r: slot r advances this round
@@ -1472,7 +1488,6 @@ static int memo_attempt(start_ctx *c, const MarchArgs &m, float theta, size_t ca
         for (int k = 0; k < 4 * kLevelBatch; ++k) cudaEventCreate(&c->lev_ev[k]);
     double hop_ms = 0.0, link_ms = 0.0, jump_ms = 0.0;
     long long max_iter = m.hop_cap + 1;
-    unsigned long long nslots_host = (unsigned long long)m.npairs;   // slots after the levels
     // device frontier {fbase, nf, total} after the slot counters
     unsigned long long *dlv = ctr + C_LEVEL;
     static_assert(C_LEVEL + 3 <= C_COUNT, "level state inside the counters");
@@ -1531,7 +1546,6 @@ static int memo_attempt(start_ctx *c, const MarchArgs &m, float theta, size_t ca
         }
         a.fbase = (u32)lv[0];
         a.nf = (long long)lv[1];
-        nslots_host = lv[2];
         // every chain ended (possibly inside the last batch, whose later
         // levels then launched over an empty frontier and did nothing)
         if (a.nf == 0) break;
@@ -1545,23 +1559,12 @@ static int memo_attempt(start_ctx *c, const MarchArgs &m, float theta, size_t ca
             ev(1);
             ++c->launches;
             ST_CUDA(c, cudaGetLastError());
-            unsigned long long tail_cap = 0;
-            ST_CUDA(c, cudaMemcpyAsync(both, ctr + C_SLOTS, sizeof(both), cudaMemcpyDeviceToHost,
-                                       s));
-            ST_CUDA(c, cudaMemcpyAsync(&tail_cap, ctr + C_TAIL_CAP, sizeof(tail_cap),
-                                       cudaMemcpyDeviceToHost, s));
-            ST_CUDA(c, cudaStreamSynchronize(s));
-            if (both[1]) {
-                overflow = true;
-                return START_OK;
-            }
-            if (tail_cap) return set_err(c, START_ECHAIN, "a chain exceeded hop_cap");
-            a.nf = (long long)(both[0] - a.fbase);
             ev(2);
-            k_memo_resolve<<<grid_for(a.nf, 256), 256, 0, s>>>(a);
+            // (its slots, an overflow or a cut chain are read with the counts of
+            // the first pointer-jumping round)
+            k_memo_resolve<<<fixed_grid, 256, 0, s>>>(a);
             ev(3);
             ++c->launches;
-            nslots_host = both[0];
             pending = 1;   // read after the first pointer-jumping round
             break;
         }
@@ -1594,45 +1597,37 @@ static int memo_attempt(start_ctx *c, const MarchArgs &m, float theta, size_t ca
         c->hop_ms += hop_ms;
         c->link_ms += link_ms;
     }
-    long long nslots = (long long)nslots_host;
-    c->memo_slots = nslots;
-    if (t0 == 0 && t1 == c->np && m.npairs > 0) {
-        c->memo_off_frac = (double)(nslots - m.npairs) / (double)m.npairs;
-        c->memo_off_theta = theta;
-    }
-    c->memo_evals += (unsigned long long)nslots;
-    c->memo_links += (unsigned long long)nslots;
     // pointer jumping
     const bool wide = memo_counts_links(c);
     if (wide && (ensure(c->m_w[0], cap * 16) || ensure(c->m_w[1], cap * 16)))
         return set_err(c, START_ENOMEM, "out of device memory (memoised march)");
     int b = 0;
-    const long long jblocks = (long long)grid_for(nslots, 256 * (wide ? kJumpR : kJumpR8));
+    const long long jblocks = (long long)grid_for((long long)cap, 256 * (wide ? kJumpR : kJumpR8));
     const long long nparts = wide ? jblocks : jblocks * 8;   // per block / per warp
     if (ensure(c->m_part, (size_t)nparts * 16))
         return set_err(c, START_ENOMEM, "out of device memory (memoised march)");
     ST_CUDA(c, cudaMemsetAsync(c->m_part.p, 0, (size_t)nparts * 16, s));
     if (wide) {
-        k_memo_widen<<<grid_for(nslots, 256), 256, 0, s>>>(nslots, c->m_st[0].as<uint2>(),
-                                                           c->m_w[0].as<uint4>());
+        k_memo_widen<<<grid_for((long long)cap, 256), 256, 0, s>>>(
+            a.nslots, (long long)cap, c->m_st[0].as<uint2>(), c->m_w[0].as<uint4>());
         ++c->launches;
     }
     static_assert(C_JUMP_LEFT == C_JUMP_MOVED + 1, "adjacent counters");
     // the counting form runs until every chain is closed; the 8-byte form
     // until few slots are open, whose chains the Gamma sum follows itself
-    const unsigned long long few = wide ? 0ull : (unsigned long long)(kJumpOpen * (double)nslots);
-    long long rounds = 0;
+    unsigned long long few = 0ull;
+    long long rounds = 0, nslots = 0;
     unsigned long long jc[2] = {0, 0};
     for (int round = 0; round < 40; ++round) {
         ST_CUDA(c, cudaMemsetAsync(ctr + C_JUMP_MOVED, 0, sizeof(jc), s));
         if (timing) cudaEventRecord(c->hev[0], s);
         if (wide)
             k_memo_jump<kJumpG><<<(unsigned)jblocks, 256, 0, s>>>(
-                nslots, c->m_w[b].as<uint4>(), c->m_w[b ^ 1].as<uint4>(), ctr,
+                a.nslots, (long long)cap, c->m_w[b].as<uint4>(), c->m_w[b ^ 1].as<uint4>(), ctr,
                 c->m_part.as<unsigned long long>());
         else
             k_memo_jump8<kJumpG, kJumpR8><<<(unsigned)jblocks, 256, 0, s>>>(
-                nslots, c->m_st[b].as<uint2>(), c->m_st[b ^ 1].as<uint2>(), ctr,
+                a.nslots, (long long)cap, c->m_st[b].as<uint2>(), c->m_st[b ^ 1].as<uint2>(), ctr,
                 c->m_part.as<unsigned long long>());
         if (timing) cudaEventRecord(c->hev[1], s);
         k_sum_jump_counts<<<grid_for(nparts, 1024, 4 * (long long)nsm), 1024, 0, s>>>(
@@ -1641,8 +1636,18 @@ static int memo_attempt(start_ctx *c, const MarchArgs &m, float theta, size_t ca
         ++rounds;
         ST_CUDA(c, cudaGetLastError());
         b ^= 1;
-        ST_CUDA(c, cudaMemcpyAsync(jc, ctr + C_JUMP_MOVED, sizeof(jc), cudaMemcpyDeviceToHost, s));
+        unsigned long long v[C_COUNT];
+        ST_CUDA(c, cudaMemcpyAsync(v, ctr, sizeof(v), cudaMemcpyDeviceToHost, s));
         ST_CUDA(c, cudaStreamSynchronize(s));
+        if (v[C_MEMO_OVF]) {   // in the tail
+            overflow = true;
+            return START_OK;
+        }
+        if (v[C_TAIL_CAP]) return set_err(c, START_ECHAIN, "a chain exceeded hop_cap");
+        jc[0] = v[C_JUMP_MOVED];
+        jc[1] = v[C_JUMP_LEFT];
+        nslots = (long long)v[C_SLOTS];
+        if (!wide) few = (unsigned long long)(kJumpOpen * (double)nslots);
         if (timing) {
             float ms = 0.f;
             if (cudaEventElapsedTime(&ms, c->hev[0], c->hev[1]) == cudaSuccess) jump_ms += ms;
@@ -1657,6 +1662,13 @@ static int memo_attempt(start_ctx *c, const MarchArgs &m, float theta, size_t ca
         if (cudaEventElapsedTime(&ms, c->lev_ev[2], c->lev_ev[3]) == cudaSuccess) c->link_ms += ms;
         else cudaGetLastError();
     }
+    c->memo_slots = nslots;
+    if (t0 == 0 && t1 == c->np && m.npairs > 0) {
+        c->memo_off_frac = (double)(nslots - m.npairs) / (double)m.npairs;
+        c->memo_off_theta = theta;
+    }
+    c->memo_evals += (unsigned long long)nslots;
+    c->memo_links += (unsigned long long)nslots;
     c->jump_rounds += rounds;
     // own state read per slot and round, and what the rounds moved beyond
     // that: per advancing slot one successor read and the write, the extra
