@@ -209,7 +209,7 @@ struct start_ctx {
 
     // resident chains (reuse_chains = 1): the link forest of the last full
     // solve in chain-end-first level order, replayed as a CUDA graph
-    st::DBuf r_j, r_up, r_dl, r_next, r_tau, r_pos, r_lvl, r_vid;
+    st::DBuf r_j, r_up, r_dl, r_next, r_tau, r_pos, r_lvl, r_vid, r_w;
     std::vector<long long> r_lvl_off;  // first position of each depth level
     bool r_valid = false;
     float r_theta = -1.f;

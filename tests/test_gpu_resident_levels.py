@@ -1,0 +1,49 @@
+"""Resident steps over chains whose depth levels are few or many links deep:
+lines of particles (levels of a link per source, all taken by one block),
+lines beside a lattice (both kinds of level) and a lattice.  Each later step
+against a full solve of the same state.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def particles(line, side, seed):
+    rng = np.random.default_rng(seed)
+    g = np.stack(np.meshgrid(*[np.arange(side)] * 3, indexing="ij")).reshape(3, -1)
+    pos = g + 0.5 + rng.uniform(-0.25, 0.25, g.shape)
+    h = np.full(pos.shape[1], 1.02)
+    x = np.stack([np.arange(line) + side + 1.0, np.full(line, 0.5), np.full(line, 0.5)])
+    x = x + rng.uniform(-0.05, 0.05, x.shape)
+    return (np.concatenate([pos, x], 1).astype(np.float32),
+            np.concatenate([h, np.full(line, 1.05)]).astype(np.float32))
+
+
+@pytest.mark.parametrize("line,side,n_s", [(5, 0, 1), (700, 0, 3), (300, 12, 40), (0, 30, 64)])
+def test_later_steps_match_full_solves(line, side, n_s):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1005_5312_gb300 as S
+    S.build()
+    pos, h = particles(line, side, line + side)
+    n = pos.shape[1]
+    rng = np.random.default_rng(n)
+    src = rng.uniform(0.0, 0.4, (3, n_s)).astype(np.float32) * np.float32(max(side, 1))
+    L = rng.lognormal(0.0, 1.0, n_s) * 1e48
+    n_H = np.full(n, 1e-3, np.float32)
+    ctx = S.Context(reuse_chains=1, sigma_cm2=1.0, len_unit_cm=10.0)
+    full = S.Context(sigma_cm2=1.0, len_unit_cm=10.0, link_counts=1)
+    for c in (ctx, full):
+        c.build_trees(pos, h, src, L)
+    for step in range(3):
+        y = rng.uniform(0.0, 1.0, n)
+        g = [np.zeros(n, np.float32) for _ in range(2)]
+        for c, out in zip((ctx, full), g):
+            c.set_state(n_H, y)
+            c.rt_solve(0.8, gamma_out=out)
+        # the same links summed from the other end in double-float: a few
+        # roundings of tau (below 10) and of each contribution
+        np.testing.assert_allclose(g[0], g[1], rtol=1e-5)
+        assert ctx.stats()["rays"] == full.stats()["rays"]
