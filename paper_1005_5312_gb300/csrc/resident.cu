@@ -49,6 +49,58 @@ __global__ void k_res_place(const uint4 *st, long long n, u32 *cursor, u32 *pos)
     if (s < n) pos[s] = atomicAdd(&cursor[st[s].y & ~kStableBit], 1u);
 }
 
+// The same for chains of fewer than kResDepths links: a block places 4096 slots
+// at once, keeping those of one depth in slot order.  A row's links of one depth
+// then lie side by side, and so do their successors, one depth earlier in the
+// upstream row: with a claim per slot the rows in flight shuffled each level,
+// and the gathers of a step took a sector per link (1.63 against 1.29 ms per
+// step on 64^3 x 1024 sources).
+constexpr int kResDepths = 256, kResTileRounds = 16;
+
+__global__ void __launch_bounds__(256) k_res_place_tiles(const uint4 *st, long long n, u32 *cursor,
+                                                         u32 *pos)
+{
+    __shared__ u32 wcnt[8][kResDepths];
+    __shared__ u32 base[kResDepths];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int k = threadIdx.x; k < 8 * kResDepths; k += 256) (&wcnt[0][0])[k] = 0u;
+    __syncthreads();
+    const unsigned below = (1u << lane) - 1u;
+    const long long s0 =
+        (long long)blockIdx.x * (256 * kResTileRounds) + warp * (32 * kResTileRounds) + lane;
+    u32 rank[kResTileRounds];
+    int depth[kResTileRounds];
+#pragma unroll
+    for (int r = 0; r < kResTileRounds; ++r) {
+        const long long s = s0 + 32 * r;
+        const bool valid = s < n;
+        const int d = valid ? (int)(st[s].y & ~kStableBit) : kResDepths;
+        depth[r] = d;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        const u32 before = valid ? wcnt[warp][d] : 0u;
+        __syncwarp();
+        if (valid && lane == __ffs(peers) - 1) wcnt[warp][d] = before + __popc(peers);
+        __syncwarp();
+        rank[r] = before + __popc(peers & below);
+    }
+    __syncthreads();
+    {
+        const int d = threadIdx.x;
+        u32 run = 0;
+        for (int w = 0; w < 8; ++w) {
+            const u32 t = wcnt[w][d];
+            wcnt[w][d] = run;
+            run += t;
+        }
+        base[d] = run ? atomicAdd(&cursor[d], run) : 0u;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kResTileRounds; ++r)
+        if (depth[r] < kResDepths)
+            pos[s0 + 32 * r] = base[depth[r]] + wcnt[warp][depth[r]] + rank[r];
+}
+
 __global__ void k_res_fill(long long n, const u32 *pos, const u32 *sj, const u32 *nx0,
                            const float *dl, u32 *rj, u32 *rup, float *rdl, u32 *rnext)
 {
@@ -215,7 +267,11 @@ int resident_build(start_ctx *c, float theta)
     c->r_lvl_off[D + 1] = run;
     if (run != S || hh[0] != 0) return set_err(c, START_ECUDA, "internal inconsistency (chain depths)");
     ST_CUDA(c, cudaMemcpyAsync(cursor, start.data(), (D + 2) * sizeof(u32), cudaMemcpyHostToDevice, s));
-    k_res_place<<<grid_for(S, 256), 256, 0, s>>>(st, S, cursor, pos.as<u32>());
+    if (D < kResDepths)
+        k_res_place_tiles<<<grid_for(S, 256 * kResTileRounds), 256, 0, s>>>(st, S, cursor,
+                                                                           pos.as<u32>());
+    else
+        k_res_place<<<grid_for(S, 256), 256, 0, s>>>(st, S, cursor, pos.as<u32>());
     k_res_pair_targets<<<grid_for(c->np * 32, 256), 256, 0, s>>>(c->np, c->loff.as<u64>(),
                                                                  c->m_j.as<u32>());
     ++c->launches;
