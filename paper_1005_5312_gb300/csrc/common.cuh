@@ -191,6 +191,7 @@ struct start_ctx {
     st::DBuf trange, trf2;
 
     // memoised march: per chain link (virtual source, particle)
+    st::DBuf m_vs;   // float4 virtual sources of the solve by canonical id
     st::DBuf m_vid, m_j, m_ord, m_st[2], m_ups, m_fr, m_hard, m_part, m_table, m_nx0, m_dl;
     // upstream candidate sets per particle and direction bin (row_bins = N:
     // 6 N^2 u64 masks per particle), each particle's largest neighbour

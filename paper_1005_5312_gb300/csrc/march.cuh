@@ -70,7 +70,8 @@ __device__ __forceinline__ int dir_bin(float x, float y, float z, int N)
         s = x;
         t = y;
     }
-    const float hn = 0.5f * (float)N / mj;
+    // (2 ulp: the bins' cones are widened by far more)
+    const float hn = __fdividef(0.5f * (float)N, mj);
     const int iu = min(N - 1, max(0, (int)((s + mj) * hn)));
     const int iv = min(N - 1, max(0, (int)((t + mj) * hn)));
     return (f * N + iu) * N + iv;

@@ -63,6 +63,7 @@ struct __align__(16) HEntry {
 struct MemoArgs {
     MarchArgs m;
     u32 SN, NS, EN;                 // source-tree nodes, sources, emitter-tree nodes
+    const float4 *vs;               // virtual sources by canonical id
     u32 *svid, *sj;                 // slot: virtual source id, particle (the particle of
                                     // a pair slot is its row's target; not stored)
     u32 *sord;                      // slot: order key of its virtual source (rows are
@@ -114,16 +115,47 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long x)
     return x;
 }
 
-__device__ __forceinline__ float4 vsource(const MemoArgs &a, u32 vid)
+// Position and L / L_unit of virtual source vid.  The four kinds lie in one
+// array (k_virtual_sources): a warp's pairs mix cells and members, and a branch
+// per kind made it read them one kind after the other (later hops 56.9 against
+// 55.2 ms, first hop 158.7 against 157.2 on the 128^3 diffuse step).
+__device__ __forceinline__ float4 vsource(const MemoArgs &a, u32 vid) { return a.vs[vid]; }
+
+__global__ void k_virtual_sources(const float4 *svsrc, u32 SN, const float4 *ssrc, u32 NS,
+                                  const float4 *evsrc, u32 EN, const float4 *pq, const float *eLs,
+                                  long long n, float4 *vs)
 {
-    if (vid < a.SN) return a.m.svsrc[vid];
-    vid -= a.SN;
-    if (vid < a.NS) return a.m.ssrc[vid];
-    vid -= a.NS;
-    if (vid < a.EN) return a.m.evsrc[vid];
-    vid -= a.EN;
-    float4 q = a.m.pq[vid];
-    return make_float4(q.x, q.y, q.z, a.m.eLs[vid]);
+    const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (v >= n) return;
+    u32 k = (u32)v;
+    float4 r;
+    if (k < SN) {
+        r = svsrc[k];
+    } else if ((k -= SN) < NS) {
+        r = ssrc[k];
+    } else if ((k -= NS) < EN) {
+        r = evsrc[k];
+    } else {
+        k -= EN;
+        r = pq[k];
+        r.w = eLs[k];
+    }
+    vs[v] = r;
+}
+
+// The virtual sources of a solve in canonical order.
+int memo_sources(start_ctx *c)
+{
+    const u32 SN = (u32)c->stree.n, NS = (u32)c->ns, EN = (u32)(c->walk_emit ? c->et.n : 0);
+    const long long n = (long long)SN + NS + EN + (c->walk_emit ? c->np : 0);
+    if (ensure(c->m_vs, (size_t)(n ? n : 1) * sizeof(float4)))
+        return set_err(c, START_ENOMEM, "out of device memory (memoised march)");
+    if (n == 0) return START_OK;
+    k_virtual_sources<<<grid_for(n, 256), 256, 0, c->stream>>>(
+        c->stree.vsrc.as<float4>(), SN, c->sq.as<float4>(), NS, c->et.vsrc.as<float4>(), EN,
+        c->pq.as<float4>(), c->eLs.as<float>(), n, c->m_vs.as<float4>());
+    ++c->launches;
+    return cuda_check(c, cudaGetLastError(), "k_virtual_sources");
 }
 
 __device__ __forceinline__ unsigned long long link_key(u32 vid, u32 k)
@@ -510,13 +542,14 @@ __global__ void __launch_bounds__(32 * W, 32 / W) k_memo_hop_rows(MemoArgs a)
     const unsigned me = 1u << lane;
     const long long i = a.t0 + ((long long)blockIdx.x * blockDim.x + threadIdx.x) / 32;
     if (i >= a.t1) return;   // warp-uniform
-    const u64 r0 = a.off[i] - a.base, r1 = a.off[i + 1] - a.base;
-    if (r1 <= r0) return;
+    // slot ids are 32-bit, rows shorter than 2^31
+    const u32 r0 = (u32)(a.off[i] - a.base), len = (u32)(a.off[i + 1] - a.off[i]);
+    if (len == 0) return;
     const float4 pj = a.m.pq[i];
     const u32 s0 = a.m.nb_off[i], s1 = a.m.nb_off[i + 1];
     if (s1 - s0 > (u32)kRowNB) {   // the whole row takes the global-memory path
-        for (u64 p0 = r0; p0 < r1; p0 += 32)
-            warp_append(p0 + lane < r1, (u32)(p0 + lane), (u32)i, a.hard, a.nhard);
+        for (u32 k = 0; k < len; k += 32)
+            warp_append(k + lane < len, r0 + k + lane, (u32)i, a.hard, a.nhard);
         return;
     }
     bool odd = false;   // a distinct neighbour whose FP32 offset underflowed
@@ -530,9 +563,10 @@ __global__ void __launch_bounds__(32 * W, 32 / W) k_memo_hop_rows(MemoArgs a)
     const int nbins = 6 * a.m.rbn * a.m.rbn;
     const bool count = (i & 63) == 0;   // candidate statistics on every 64th row
     unsigned cand = 0;
-    for (u64 p0 = r0; p0 < r1; p0 += 32) {   // warp-uniform: the list appends below
-        const u64 p = p0 + lane;
-        const bool valid = p < r1;
+    const unsigned long long *masks = a.m.rbm + (u64)i * nbins;
+    for (u32 k0 = 0; k0 < len; k0 += 32) {   // warp-uniform: the list appends below
+        const u32 p = r0 + k0 + lane;
+        const bool valid = k0 + lane < len;
         u32 up = kNone, nx = kNone;
         bool hard = false;
         u32 vid = 0;
@@ -549,7 +583,7 @@ __global__ void __launch_bounds__(32 * W, 32 / W) k_memo_hop_rows(MemoArgs a)
             um = all;
             if (nbins && bn > amax) {
                 const unsigned long long bm =
-                    a.m.rbm[(u64)i * nbins + dir_bin(bx, by, bz, a.m.rbn)];
+                    masks[dir_bin(bx, by, bz, a.m.rbn)];
                 if (bm) um = bm;
             }
         }
@@ -598,16 +632,16 @@ __global__ void __launch_bounds__(32 * W, 32 / W) k_memo_hop_rows(MemoArgs a)
                 if (a.nx0) a.nx0[p] = nx;
             }
         }
-        warp_append(hard, (u32)p, (u32)i, a.hard, a.nhard);
+        warp_append(hard, p, (u32)i, a.hard, a.nhard);
         // links found in up's row are done; the others are listed for
         // k_memo_link's table, marked as searched
-        append_miss(a, valid && !hard && up != kNone && nx == kNone, (u32)p, up | kRowMiss);
+        append_miss(a, valid && !hard && up != kNone && nx == kNone, p, up | kRowMiss);
     }
     if (count) {   // warp-uniform
         for (int o = 16; o; o >>= 1) cand += __shfl_xor_sync(0xffffffffu, cand, o);
         if (lane == 0) {
             atomicAdd(&a.m.counters[C_ROW_CAND], (unsigned long long)cand);
-            atomicAdd(&a.m.counters[C_ROW_NB], (unsigned long long)nst * (r1 - r0));
+            atomicAdd(&a.m.counters[C_ROW_NB], (unsigned long long)nst * len);
         }
     }
 }
@@ -914,15 +948,14 @@ constexpr int kJumpR = 6;    // counting form: slots per thread (independent loa
 constexpr int kJumpG = 3;    // successor reads per slot and round
 constexpr int kJumpR8 = 12;  // 8-byte form: slots per thread
 // Rounds of the 8-byte form: another one runs while more than this share of
-// the slots is open.  The Gamma sum follows the open chains block by block; of
-// chain lengths spread evenly, a share p left open means 1 / (2 (1 - p))
-// blocks to follow per pair, and a round costs about as much as 16 of them
-// (GB300, jumping + Gamma: 2.6 against 2.9 ms with a second round on 64^3 x
-// 1024 sources, p = 0.91; 9.4 against 10.2 ms with three rounds on 1.7 M x 500
-// sources, p = 0.96; 7.2 against 5.4 ms with three on 128^3 x 64 sources,
-// p = 0.98; 147 against 165 ms at half open on the 128^3 diffuse step).
-constexpr double kJumpOpen = 0.97;
-constexpr int kGammaU = 2;   // pairs per lane in flight in the rows of a group
+// the slots is open, the Gamma sum follows the open chains block by block.
+// Jumping + Gamma, one round against two (GB300): 2.5 against 2.7 ms on 64^3 x
+// 1024 sources (0.990 open after the first), 50 against 54 ms on 1.7 M x 40 k
+// (0.989), 0.35 against 0.35 ms on 41^3 x 256 (0.995), but 9.8 against 8.4 ms on
+// 1.7 M x 500 (0.999) and 7.2 against 4.5 ms on 128^3 x 64 (0.9998; a third
+// round, 0.979 open after the second, 4.9 ms).
+constexpr double kJumpOpen = 0.995;
+constexpr int kGammaU = 3;   // pairs per lane in flight in the rows of a group
 
 // The march's states widened for the counting form: one link, no
 // compensation term.
@@ -1201,8 +1234,13 @@ __device__ __forceinline__ float spec_lookup(const float *tab, float sidx)
 // group, the groups in row order: acc carries each target's compensated sums
 // (sum, compensation, heating sum, its compensation) from one group to the
 // next; the first group starts from zero and the last one writes Gamma.
+// (Registers are kept low for occupancy: the reads of open chains wait on L2.
+// Rows of one warp 1.60 ms at 40 registers, 1.41 at 32, on 64^3 x 1024 sources;
+// the short rows of a group, three pairs per lane, 76 / 31 ms at 51 registers on
+// the 128^3 diffuse step / 1.7 M x 40 k, 77 / 34 at 64; two pairs 78 / 32 at 51,
+// 83 / 29 at 42; one pair 97 / 31 at 32.)
 template <int MODE, int LANES, bool WIDE>
-__global__ void __launch_bounds__(256) k_memo_gamma(MemoArgs a, const u64 *off, long long t0,
+__global__ void __launch_bounds__(256, WIDE ? 4 : LANES == 32 ? 8 : 5) k_memo_gamma(MemoArgs a, const u64 *off, long long t0,
                                                      long long t1, u64 base, float conv,
                                                      const u32 *porig, float *gam, float *gout,
                                                      GammaExtra x, float4 *acc, int first,
@@ -1227,9 +1265,9 @@ __global__ void __launch_bounds__(256) k_memo_gamma(MemoArgs a, const u64 *off, 
             hsum = q.z;
             hcmp = q.w;
         }
-        // pairs per lane in flight: two in the short rows of a group (82 against
-        // 97 ms on the 128^3 diffuse step), one where a warp has the whole row
-        // (1.63 against 1.83 ms on 64^3 x 1024 sources)
+        // pairs per lane in flight: three in the short rows of a group (above),
+        // one where a warp has the whole row (1.63 against 1.83 ms with two on
+        // 64^3 x 1024 sources)
         constexpr int U = WIDE || LANES == 32 ? 1 : kGammaU;
         for (u64 e = e0; e < e1; e += LANES * U) {   // uniform within the lane group
             float v[U], hv[U], tau[U];
@@ -1435,6 +1473,7 @@ static int memo_attempt(start_ctx *c, const MarchArgs &m, float theta, size_t ca
     a.SN = (u32)c->stree.n;
     a.NS = (u32)c->ns;
     a.EN = (u32)(c->walk_emit ? c->et.n : 0);
+    a.vs = c->m_vs.as<float4>();
     a.ts = {c->stree.box.as<float4>(), c->stree.meta.as<uint4>(), c->stree.cube.as<double>(),
             c->stree.parent.as<u32>(), a.SN};
     a.te = {c->et.box.as<float4>(), c->et.meta.as<uint4>(), c->et.cube.as<double>(),
@@ -1702,6 +1741,7 @@ int memo_gamma(start_ctx *c, const MarchArgs &m, long long t0, long long t1, u64
     a.SN = (u32)c->stree.n;
     a.NS = (u32)c->ns;
     a.EN = (u32)(c->walk_emit ? c->et.n : 0);
+    a.vs = c->m_vs.as<float4>();
     a.svid = c->m_vid.as<u32>();
     a.state = c->m_st[c->memo_final].as<uint2>();
     a.cap = (u32)c->memo_slots;   // chain links of the march

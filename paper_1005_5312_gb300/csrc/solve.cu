@@ -22,6 +22,7 @@ namespace st {
 
 int run_memo(start_ctx *c, const MarchArgs &m, float theta, long long t0, long long t1,
              u64 base);
+int memo_sources(start_ctx *c);
 int memo_gamma(start_ctx *c, const MarchArgs &m, long long t0, long long t1, u64 base,
                float conv, float *gout, bool first, bool last);
 
@@ -1324,6 +1325,7 @@ int run_solve(start_ctx *c, float theta, float *gout_dev)
     c->walk_emit = c->diffuse && !kdis;               // LW photons come from point sources
     if (np == 0) return START_OK;
     if (c->walk_emit) ST_TRY(refresh_emitters(c));
+    if (memo) ST_TRY(memo_sources(c));
     // L / L_unit / (4 pi r^2), r in length units -> photons cm^-2 s^-1; for
     // k_dis times 1.13e8 kappa_LW (Eq. H2ss)
     double conv_d = c->p.L_unit / (c->p.len_unit_cm * c->p.len_unit_cm);
