@@ -426,46 +426,86 @@ __global__ void __launch_bounds__(32 * W) k_row_bins(MarchArgs m, const float4 *
     }
     if (lane == 0) ramax[i] = sqrtf(amax2);
     // per neighbour: unit offset e_k and t_k = |r_k - r_j| / (2 amax) + eta
-    // (over the staged record; 2 marks an entry at the target's own position)
-    // and sqrt(1 - t_k^2) (over the half distance); with a_k = acos t_k,
-    // k passes the closer-than test for the whole bin iff theta_k < a_k - rho
-    // (a_k > rho), i.e. cos theta_k > cos(a_k - rho) = t_k cos rho + sqrt(1 -
-    // t_k^2) sin rho; the qualifying neighbour of largest cos theta_k sets L
+    // (over the staged record) and sqrt(1 - t_k^2) (over the half distance);
+    // with a_k = acos t_k, k passes the closer-than test for the whole bin iff
+    // theta_k < a_k - rho (a_k > rho: t_k is at most 0.501 and rho below 0.7),
+    // i.e. cos theta_k > cos(a_k - rho) = t_k cos rho + sqrt(1 - t_k^2) sin rho;
+    // the qualifying neighbour of largest cos theta_k sets L.  An entry at the
+    // target's own position (e = 0) gets t = 2: it never qualifies.
     const float inv = 0.5f * rsqrtf(amax2);
-    for (int q = lane; q < nst; q += 32) {
-        const float an = 2.f * nba[w][q].w;
-        const float t = an < kFar ? an * inv + kBinEta : 2.f;
-        nbp[w][q].x = t;
-        nba[w][q].w = sqrtf(fmaxf(0.f, 1.f - t * t));
+    unsigned at_own[2] = {0u, 0u};   // such entries, by list offset
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int q = 32 * h + lane;
+        bool own = false;
+        if (q < nst) {
+            const float an = 2.f * nba[w][q].w;
+            own = !(an < kFar);
+            const float t = own ? 2.f : an * inv + kBinEta;
+            nbp[w][q].x = t;
+            nba[w][q].w = own ? 0.f : sqrtf(fmaxf(0.f, 1.f - t * t));
+        }
+        at_own[h] = __ballot_sync(0xffffffffu, own);
     }
     __syncwarp();
-    for (int b = lane; b < nbins; b += 32) {
-        const float4 g = geo[2 * b];
-        const float cr = g.w, sr = geo[2 * b + 1].x, rho = geo[2 * b + 1].y;
-        float best = -2.f;   // cos theta of the qualifying neighbour nearest the axis
+    // three bins per lane at a time: a neighbour is read once for all three (one
+    // bin at a time: 311 against 195 us for the 108 k particles of a batch)
+    for (int b0 = lane; b0 < nbins; b0 += 96) {
+        float4 g[3];
+        float sr[3], rho[3], best[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const int b = min(b0 + 32 * j, nbins - 1);
+            g[j] = geo[2 * b];
+            const float4 r = geo[2 * b + 1];
+            sr[j] = r.x;
+            rho[j] = r.y;
+            best[j] = -2.f;   // cos theta of the qualifying neighbour nearest the axis
+        }
+#pragma unroll 2
         for (int q = 0; q < nst; ++q) {
             const float4 u = nba[w][q];
             const float t = nbp[w][q].x;
-            const float ct = u.x * g.x + u.y * g.y + u.z * g.z;
-            const float thr = t * cr + u.w * sr;
-            if (t < cr && ct > thr + 1e-5f) best = fmaxf(best, ct);
-        }
-        unsigned long long mk = 0ull;
-        if (best > -2.f) {
-            // L = cos(theta + rho) of that neighbour (its sine from above: L
-            // from below); k can win only if theta_k <= acos(L - eta) + rho
-            const float sn = sqrtf(fmaxf(0.f, 1.f - best * best) + 1e-6f);
-            const float L = best <= -cr ? -1.f : best * cr - sn * sr;
-            const float Lp = L - kBinEta;
-            const float ang = Lp <= -1.f ? 4.f : acosf(Lp) + rho;
-            const float cmin = ang >= 3.14159f ? -2.f : cosf(ang) - 1e-5f;
-            for (int q = 0; q < nst; ++q) {
-                const float4 u = nba[w][q];
-                const float ct = u.x * g.x + u.y * g.y + u.z * g.z;
-                if (nbp[w][q].x < 1.5f && ct >= cmin) mk |= 1ull << q;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const float ct = u.x * g[j].x + u.y * g[j].y + u.z * g[j].z;
+                const float thr = t * g[j].w + (u.w * sr[j] + 1e-5f);
+                if (ct > thr) best[j] = fmaxf(best[j], ct);
             }
         }
-        row[b] = mk;
+        float cmin[3];   // k can win only if theta_k <= acos(L - eta) + rho
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            // L = cos(theta + rho) of that neighbour (its sine from above: L
+            // from below)
+            const float cr = g[j].w;
+            const float sn = sqrtf(fmaxf(0.f, 1.f - best[j] * best[j]) + 1e-6f);
+            const float L = best[j] <= -cr ? -1.f : best[j] * cr - sn * sr[j];
+            const float Lp = L - kBinEta;
+            const float ang = Lp <= -1.f ? 4.f : acosf(Lp) + rho[j];
+            cmin[j] = ang >= 3.14159f ? -2.f : cosf(ang) - 1e-5f;
+        }
+        unsigned mk[3][2] = {};
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int q1 = min(32, nst - 32 * h);
+#pragma unroll 2
+            for (int q = 0; q < q1; ++q) {
+                const float4 u = nba[w][32 * h + q];
+                const unsigned bit = 1u << q;
+#pragma unroll
+                for (int j = 0; j < 3; ++j)
+                    if (u.x * g[j].x + u.y * g[j].y + u.z * g[j].z >= cmin[j]) mk[j][h] |= bit;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const int b = b0 + 32 * j;
+            if (b >= nbins) continue;
+            const unsigned long long m2 =
+                (unsigned long long)(mk[j][1] & ~at_own[1]) << 32 | (mk[j][0] & ~at_own[0]);
+            row[b] = best[j] > -2.f ? m2 : 0ull;   // no qualifying neighbour: test them all
+        }
     }
 }
 
