@@ -4,10 +4,10 @@
 //
 // A warp takes 32 targets in Morton order, spatial neighbours, and walks the
 // particle tree once for all of them: 32 consecutive cells of the pre-order at
-// a time, one per lane, are tested against the boxes around the spheres of the
-// targets' four octets, and the skip pointers of those outside tell which of
-// the 32 the walk reaches and where it goes on.  The members of the leaves it
-// reaches are read one per lane, those inside a box are staged, and every lane
+// a time, one per lane, are tested against the box around the targets'
+// spheres, and the skip pointers of those outside tell which of the 32 the walk
+// reaches and where it goes on.  The members of the leaves it reaches are read
+// one per lane, those inside the box are staged, and every lane
 // tests its own target against each staged member (a broadcast read), first
 // without branches into a bit mask, then its few candidates by the FP32-filtered
 // exact test with an FP64 fallback.  The walk keeps the first kNbCap neighbours
@@ -15,8 +15,10 @@
 // and only targets with more neighbours than that walk again, a thread each, to
 // fill their rows.  (One walk per thread for every target, a chain of dependent
 // cell and member reads: 1570 us at 2^20 particles, 157 us at 2 k, where it
-// left most of the chip idle, against 1266 and 54 us; staging each octet's
-// members apart makes the tests fewer but the staging dearer: 1617 us.)
+// left most of the chip idle, against 1150 and 54 us.  Tighter boxes, of the
+// targets' octets, stage fewer members but cost more than they save: 1266 us;
+// of their quads 1560; staging each octet's members apart 1617.  The test as |p|^2
+// + t.p in three FMAs takes more registers than it saves issue: 1417.)
 #include "common.cuh"
 
 namespace st {
@@ -41,9 +43,9 @@ __device__ __forceinline__ bool member_in(float4 pk, float4 pi, float two_h, dou
 
 constexpr u32 kNbCap = 48;   // neighbours kept per target by the counting walk
 constexpr int kNbWarps = 4;
-// an octet of targets whose box is wider than this many times their largest
-// reach straddles a jump of the Morton curve (eight lattice neighbours span
-// three): its group tests the cells against each target's own sphere
+// a group of targets whose box is wider than this many times their largest
+// reach straddles a jump of the Morton curve (32 lattice neighbours span four):
+// it tests the cells against each target's own sphere
 constexpr float kNbWide = 6.f;
 
 // Squared distance from p to a cell's cube (FP32, rounded to nearest).
@@ -97,7 +99,6 @@ k_neighbours(const float4 *pq, const float *h, long long np, const float4 *box, 
 {
     __shared__ float4 buf[kNbWarps][64];      // staged members: position, index
     __shared__ float4 sphere[kNbWarps][32];   // the targets' positions and squared reaches
-    __shared__ float4 oct[kNbWarps][4][2];    // the octets' boxes: lower, upper corner
     __shared__ u32 list[kNbWarps][kNbCap][33];
     const float4 far = make_float4(1e30f, 1e30f, 1e30f, 0.f);   // no target's neighbour
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -131,7 +132,7 @@ k_neighbours(const float4 *pq, const float *h, long long np, const float4 *box, 
         float hi[3] = {mine ? __fadd_rn(pi.x, reach) : -inf, mine ? __fadd_rn(pi.y, reach) : -inf,
                        mine ? __fadd_rn(pi.z, reach) : -inf};
         float rmax = mine ? reach : 0.f;
-        for (int o = 4; o; o >>= 1) {
+        for (int o = 16; o; o >>= 1) {
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 lo[a] = fminf(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
@@ -139,14 +140,9 @@ k_neighbours(const float4 *pq, const float *h, long long np, const float4 *box, 
             }
             rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
         }
-        const bool wide = __any_sync(
-            0xffffffffu,
-            fmaxf(fmaxf(hi[0] - lo[0], hi[1] - lo[1]), hi[2] - lo[2]) > kNbWide * rmax);
+        const bool wide =
+            fmaxf(fmaxf(hi[0] - lo[0], hi[1] - lo[1]), hi[2] - lo[2]) > kNbWide * rmax;
         __syncwarp();
-        if ((lane & 7) == 0) {
-            oct[w][lane >> 3][0] = make_float4(lo[0], lo[1], lo[2], 0.f);
-            oct[w][lane >> 3][1] = make_float4(hi[0], hi[1], hi[2], 0.f);
-        }
         sphere[w][lane] = make_float4(pi.x, pi.y, pi.z, mine ? __fmul_rn(reach, reach) : -1.f);
         __syncwarp();
         // 1e-5: far above the rounding of the FP32 distance, so that no
@@ -162,14 +158,9 @@ k_neighbours(const float4 *pq, const float *h, long long np, const float4 *box, 
             if (in) {
                 const float4 b = box[n];
                 mt = meta[n];
-                const float bx = __fadd_rn(b.x, b.w), by = __fadd_rn(b.y, b.w),
-                            bz = __fadd_rn(b.z, b.w);
-#pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    const float4 l = oct[w][g][0], u = oct[w][g][1];
-                    hit = hit || (b.x <= u.x && bx >= l.x && b.y <= u.y && by >= l.y &&
-                                  b.z <= u.z && bz >= l.z);
-                }
+                hit = b.x <= hi[0] && __fadd_rn(b.x, b.w) >= lo[0] && b.y <= hi[1] &&
+                      __fadd_rn(b.y, b.w) >= lo[1] && b.z <= hi[2] &&
+                      __fadd_rn(b.z, b.w) >= lo[2];
                 if (wide && hit) {
                     hit = false;
                     for (int t = 0; t < 32 && !hit; ++t) {
@@ -212,13 +203,8 @@ k_neighbours(const float4 *pq, const float *h, long long np, const float4 *box, 
                     const u32 r = first + (q - (e - len));
                     p = pq[r];
                     p.w = __uint_as_float(r);
-                    near = wide;
-#pragma unroll
-                    for (int g = 0; g < 4; ++g) {
-                        const float4 l = oct[w][g][0], u = oct[w][g][1];
-                        near = near || (p.x <= u.x && p.x >= l.x && p.y <= u.y && p.y >= l.y &&
-                                        p.z <= u.z && p.z >= l.z);
-                    }
+                    near = p.x <= hi[0] && p.x >= lo[0] && p.y <= hi[1] && p.y >= lo[1] &&
+                           p.z <= hi[2] && p.z >= lo[2];
                 }
                 const unsigned nm = __ballot_sync(0xffffffffu, near);
                 if (near) buf[w][staged + __popc(nm & ((1u << lane) - 1u))] = p;
