@@ -16,10 +16,12 @@
 //   R_heat(tau) = (1/D) int (u - 1) u^-3 e^(-tau u^-3) du
 // in the same roles (Eq. gother for the heating).
 //
-// Each integral is tabulated on the host as ln F on a grid in
-// s = ln(1 + tau / tau0), by composite 6-point Gauss-Legendre (the blackbody
-// over u in [1, 1 + 80/a], beyond which the spectrum is below e^-80 of its
-// peak); the per-pair reduction interpolates linearly in s.
+// Each integral is tabulated as ln F on a grid in s = ln(1 + tau / tau0), by
+// composite 6-point Gauss-Legendre (the blackbody over u in [1, 1 + 80/a], beyond
+// which the spectrum is below e^-80 of its peak) in FP64, a thread per grid
+// point that takes the nodes in order (on the host the 12.6 million exponentials
+// of a blackbody held up the first solve with a new temperature for 38 ms,
+// against 1.4 ms); the per-pair reduction interpolates linearly in s.
 #include <math.h>
 
 #include <vector>
@@ -37,27 +39,6 @@ const double kGx[6] = {-0.9324695142031521, -0.6612093864662645, -0.238619186083
 const double kGw[6] = {0.1713244923791704, 0.3607615730481386, 0.4679139345726910,
                        0.4679139345726910, 0.3607615730481386, 0.1713244923791704};
 
-// ln of the two integrals of a spectrum given by its quadrature nodes (weight
-// w_j, u_j), normalised by z, at every grid point; into tab[0, kSpecN) and
-// tab[kSpecN, 2 kSpecN).
-void tabulate(const std::vector<double> &w, const std::vector<double> &u, double z, float *tab)
-{
-    std::vector<double> iu3(u.size());
-    for (size_t j = 0; j < u.size(); ++j) iu3[j] = 1.0 / (u[j] * u[j] * u[j]);
-    const double ds = log1p(kSpecTauMax / kSpecTau0) / (kSpecN - 1);
-    for (int k = 0; k < kSpecN; ++k) {
-        double tau = kSpecTau0 * expm1(k * ds);
-        double fi = 0.0, fh = 0.0;
-        for (size_t j = 0; j < u.size(); ++j) {
-            double v = w[j] * iu3[j] * exp(-tau * iu3[j]);
-            fi += v;
-            fh += v * (u[j] - 1.0);
-        }
-        tab[k] = (float)log(fmax(fi / z, 1e-300));
-        tab[kSpecN + k] = (float)log(fmax(fh / z, 1e-300));
-    }
-}
-
 // nodes and weights of composite Gauss-Legendre over [lo, hi]
 void gl_nodes(double lo, double hi, int panels, std::vector<double> &x, std::vector<double> &w)
 {
@@ -72,11 +53,63 @@ void gl_nodes(double lo, double hi, int panels, std::vector<double> &x, std::vec
 }
 }  // namespace
 
+// ln of the two integrals of a spectrum given by its n quadrature nodes (weight
+// w_j and u_j, then u_j^-3), normalised by z, at every grid point; into tab[0, kSpecN)
+// and tab[kSpecN, 2 kSpecN).
+__global__ void __launch_bounds__(64) k_spectral_table(const double *w, const double *u,
+                                                       const double *iu3, int n, double z,
+                                                       double ds, float *tab)
+{
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= kSpecN) return;
+    const double tau = kSpecTau0 * expm1(k * ds);
+    double fi = 0.0, fh = 0.0;
+    for (int j = 0; j < n; ++j) {
+        const double v = w[j] * iu3[j] * exp(-tau * iu3[j]);
+        fi += v;
+        fh += v * (u[j] - 1.0);
+    }
+    tab[k] = (float)log(fmax(fi / z, 1e-300));
+    tab[kSpecN + k] = (float)log(fmax(fh / z, 1e-300));
+}
+
+// Tabulates a spectrum of nodes (u, w) with normalisation z at tab (device).
+static int tabulate(start_ctx *c, const std::vector<double> &u, const std::vector<double> &w,
+                    double z, float *tab)
+{
+    const size_t n = u.size();
+    std::vector<double> nodes(3 * n);
+    for (size_t j = 0; j < n; ++j) {
+        nodes[j] = w[j];
+        nodes[n + j] = u[j];
+        nodes[2 * n + j] = 1.0 / (u[j] * u[j] * u[j]);
+    }
+    DBuf buf;
+    if (ensure(buf, nodes.size() * sizeof(double)))
+        return set_err(c, START_ENOMEM, "out of device memory (spectral tables)");
+    cudaError_t e = cudaMemcpyAsync(buf.p, nodes.data(), nodes.size() * sizeof(double),
+                                    cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess) {
+        const double *d = buf.as<double>();
+        const double ds = log1p(kSpecTauMax / kSpecTau0) / (kSpecN - 1);
+        k_spectral_table<<<grid_for(kSpecN, 64), 64, 0, c->stream>>>(d, d + n, d + 2 * n, (int)n,
+                                                                      z, ds, tab);
+        ++c->launches;
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);   // nodes are on the host
+    }
+    release(buf);   // stream-ordered
+    return cuda_check(c, e, "k_spectral_table");
+}
+
 int spectral_table(start_ctx *c)
 {
     const double T = c->p.T_eff, Tr = c->p.T_rec;
     if (c->spec_T == T && c->spec_Trec == Tr && c->spec_tab.p) return START_OK;
-    std::vector<float> tab(4 * kSpecN, 0.f);
+    c->spec_T = c->spec_Trec = -1.0;
+    ST_TRY(ensure(c->spec_tab, 4 * kSpecN * sizeof(float)));
+    float *tab = c->spec_tab.as<float>();
+    ST_CUDA(c, cudaMemsetAsync(tab, 0, 4 * kSpecN * sizeof(float), c->stream));
     if (T > 0.0) {
         const double a = kHnuL / (kBoltz * T);
         std::vector<double> u, w;
@@ -86,18 +119,14 @@ int spectral_table(start_ctx *c)
             w[j] *= u[j] * u[j] / expm1(a * u[j]);
             z += w[j];
         }
-        tabulate(w, u, z, tab.data());
+        ST_TRY(tabulate(c, u, w, z, tab));
     }
     if (Tr > 0.0) {
         const double D = kBoltz * Tr / kHnuL;
         std::vector<double> u, w;
         gl_nodes(1.0, 1.0 + D, 16, u, w);
-        tabulate(w, u, D, tab.data() + 2 * kSpecN);
+        ST_TRY(tabulate(c, u, w, D, tab + 2 * kSpecN));
     }
-    ST_TRY(ensure(c->spec_tab, tab.size() * sizeof(float)));
-    ST_CUDA(c, cudaMemcpyAsync(c->spec_tab.p, tab.data(), tab.size() * sizeof(float),
-                               cudaMemcpyHostToDevice, c->stream));
-    ST_CUDA(c, cudaStreamSynchronize(c->stream));
     c->spec_T = T;
     c->spec_Trec = Tr;
     return START_OK;
