@@ -17,6 +17,11 @@
 namespace st {
 
 constexpr u32 kNone = 0xffffffffu;
+// Candidates of a neighbour list that a lane requests ahead of scoring.  The
+// later hops of a 128^3 diffuse step wait on these reads: 55 ms with one at a
+// time, 45 with four; two and six give 0.4-0.6 of that gain (six take
+// registers that cost a resident block).
+constexpr int kHopAhead = 4;
 
 struct MarchArgs {
     const u32 *pent, *ptgt;
@@ -141,18 +146,15 @@ __device__ __forceinline__ float link_dt(const MarchArgs &a, float4 pj, float4 s
     return a.sig * 0.5f * (pj.w + pu.w) * dl;
 }
 
-// Candidate s of the neighbour list of particle j (record pj) for a source
-// at b = r_s - r_j (|b| = bn): the closer-than test and the score with their
-// certified error bounds; keeps the best and second-best scores and the best
-// candidate, and flags a test inside its bound.
-__device__ __forceinline__ void hop_candidate(const MarchArgs &a, u32 s, float4 pj, float bx,
-                                              float by, float bz, float bn, float &bc, float &sc,
-                                              u32 &bk, bool &unsure)
+// Candidate k (record pk) of the neighbour list of particle j (record pj) for a
+// source at b = r_s - r_j (|b| = bn): the closer-than test and the score with
+// their certified error bounds; keeps the best and second-best scores and the
+// best candidate, and flags a test inside its bound.
+__device__ __forceinline__ void hop_candidate(u32 k, float4 pk, float4 pj, float bx, float by,
+                                              float bz, float bn, float &bc, float &sc, u32 &bk,
+                                              bool &unsure)
 {
     const float eps_q = 16.f * kU32;
-    u32 k = a.nb_idx[s];
-    if (k >= a.np) return;   // cannot happen: lists hold particle indices
-    float4 pk = a.pq[k];
     float ax = pk.x - pj.x, ay = pk.y - pj.y, az = pk.z - pj.z;
     float a2 = ax * ax + ay * ay + az * az;
     if (a2 == 0.f) {
@@ -204,19 +206,34 @@ __device__ __forceinline__ u32 hop(const MarchArgs &a, u32 j, float4 pj, float4 
     unsigned long long msk = 0ull;   // list offsets to test, or 0: every neighbour
     if (G <= 4 && a.rbn && s1 - s0 <= 64u && bn > a.ramax[j])
         msk = a.rbm[(unsigned long long)j * (6 * a.rbn * a.rbn) + dir_bin(bx, by, bz, a.rbn)];
-    if (msk) {
-        unsigned long long m = msk;
+    // kHopAhead candidates' indices, then their records, are requested before the
+    // first is scored: one after the other, each waits for two dependent reads
+    unsigned long long m = msk;
+    if (msk)
         for (int t = 0; t < gl; ++t) m &= m - 1ull;   // this lane's first bit
-        while (m) {
-            hop_candidate(a, s0 + (u32)(__ffsll((long long)m) - 1), pj, bx, by, bz, bn, bc, sc,
-                          bk, unsure);
+    u32 s = s0 + gl;
+    while (msk ? m != 0ull : s < s1) {
+        u32 k[kHopAhead];
+        float4 pk[kHopAhead];
 #pragma unroll
-            for (int t = 0; t < G; ++t) m &= m - 1ull;
+        for (int c = 0; c < kHopAhead; ++c) {
+            u32 at = s;
+            bool has = s < s1;
+            if (msk) {
+                has = m != 0ull;
+                at = s0 + (has ? (u32)(__ffsll((long long)m) - 1) : 0u);
+#pragma unroll
+                for (int t = 0; t < G; ++t) m &= m - 1ull;
+            }
+            s += G;
+            k[c] = has ? a.nb_idx[at] : kNone;
         }
-    } else {
-#pragma unroll 4
-        for (u32 s = s0 + gl; s < s1; s += G)
-            hop_candidate(a, s, pj, bx, by, bz, bn, bc, sc, bk, unsure);
+#pragma unroll
+        for (int c = 0; c < kHopAhead; ++c)   // lists hold particle indices
+            pk[c] = k[c] < a.np ? a.pq[k[c]] : pj;
+#pragma unroll
+        for (int c = 0; c < kHopAhead; ++c)
+            if (k[c] < a.np) hop_candidate(k[c], pk[c], pj, bx, by, bz, bn, bc, sc, bk, unsure);
     }
     float mc = bc;
     u32 mk = bk;
