@@ -545,23 +545,44 @@ __device__ __forceinline__ void score_staged4(const float4 *nba, uchar4 q, float
     bc = fmaxf(bc, h);
 }
 
-// Appends the flagged lanes' (slot, upstream) to the first level's list of
-// links left to k_memo_link; every lane of the warp calls it.
-__device__ __forceinline__ void append_miss(const MemoArgs &a, bool flag, u32 slot, u32 upv)
-{
-    const int lane = threadIdx.x & 31;
-    const unsigned m = __ballot_sync(0xffffffffu, flag);
-    if (!m) return;
-    const int leader = __ffs(m) - 1;
-    unsigned long long b = 0;
-    if (lane == leader) b = atomicAdd(a.nmiss, (unsigned long long)__popc(m));
-    b = __shfl_sync(0xffffffffu, b, leader);
-    if (flag) {
-        const unsigned long long q = b + __popc(m & ((1u << lane) - 1u));
-        a.miss[q] = slot;
-        a.ups[q] = upv;
+// The first level's list of links left to k_memo_link takes a warp's entries
+// 32 at a time: every iteration of a row adds a few, and one counter update
+// per iteration made the warps of the whole device wait for one address (first hops of
+// a 128^3 diffuse step 157 -> 151 ms).
+struct MissBuffer {
+    uint2 *e;   // 64 entries (slot, upstream) of this warp
+    int n;      // held, warp-uniform, below 32 between calls
+
+    // Writes the first m held entries to the list; the whole warp calls it.
+    __device__ __forceinline__ void flush(const MemoArgs &a, int m)
+    {
+        const int lane = threadIdx.x & 31;
+        unsigned long long b = 0;
+        if (lane == 0) b = atomicAdd(a.nmiss, (unsigned long long)m);
+        b = __shfl_sync(0xffffffffu, b, 0);
+        if (lane < m) {
+            a.miss[b + lane] = e[lane].x;
+            a.ups[b + lane] = e[lane].y;
+        }
     }
-}
+    __device__ __forceinline__ void add(const MemoArgs &a, bool flag, u32 slot, u32 upv)
+    {
+        const int lane = threadIdx.x & 31;
+        const unsigned m = __ballot_sync(0xffffffffu, flag);
+        if (!m) return;
+        if (flag) e[n + __popc(m & ((1u << lane) - 1u))] = make_uint2(slot, upv);
+        n += __popc(m);
+        __syncwarp();
+        if (n >= 32) {
+            flush(a, 32);
+            n -= 32;
+            const uint2 rest = e[32 + lane];
+            __syncwarp();
+            if (lane < n) e[lane] = rest;
+            __syncwarp();
+        }
+    }
+};
 
 // W target rows per block (the tile shape; 8 KB of stage per row): 32 warps
 // per SM either way.  With direction bins (a.m.rbn = N > 0) a pair whose
@@ -577,6 +598,7 @@ __global__ void __launch_bounds__(32 * W, 32 / W) k_memo_hop_rows(MemoArgs a)
     __shared__ uint4 nbr[W][kRowNB];    // (k, row start, row end, -), slot indices
     // the candidates a warp iteration scans, padded to fours
     __shared__ uchar4 qsel4[W][kRowNB / 4 + 1];
+    __shared__ uint2 missed[W][64];
     const float two_eps = 32.f * kU32;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned me = 1u << lane;
@@ -603,6 +625,7 @@ __global__ void __launch_bounds__(32 * W, 32 / W) k_memo_hop_rows(MemoArgs a)
     const int nbins = 6 * a.m.rbn * a.m.rbn;
     const bool count = (i & 63) == 0;   // candidate statistics on every 64th row
     unsigned cand = 0;
+    MissBuffer miss{missed[w], 0};
     const unsigned long long *masks = a.m.rbm + (u64)i * nbins;
     for (u32 k0 = 0; k0 < len; k0 += 32) {   // warp-uniform: the list appends below
         const u32 p = r0 + k0 + lane;
@@ -675,8 +698,9 @@ __global__ void __launch_bounds__(32 * W, 32 / W) k_memo_hop_rows(MemoArgs a)
         warp_append(hard, p, (u32)i, a.hard, a.nhard);
         // links found in up's row are done; the others are listed for
         // k_memo_link's table, marked as searched
-        append_miss(a, valid && !hard && up != kNone && nx == kNone, p, up | kRowMiss);
+        miss.add(a, valid && !hard && up != kNone && nx == kNone, p, up | kRowMiss);
     }
+    if (miss.n) miss.flush(a, miss.n);
     if (count) {   // warp-uniform
         for (int o = 16; o; o >>= 1) cand += __shfl_xor_sync(0xffffffffu, cand, o);
         if (lane == 0) {
