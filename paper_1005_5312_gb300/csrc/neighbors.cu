@@ -2,24 +2,29 @@
 // RSPH upstream search of Section 2.2.1 chooses from), found through the
 // particle octree that Section 2.2.2 reuses from the gravity solver.
 //
-// A warp takes 32 targets in Morton order, spatial neighbours, and walks the
-// particle tree once for all of them: 32 consecutive cells of the pre-order at
+// A warp takes 32 / P targets in Morton order, spatial neighbours, P lanes each
+// (one where the targets fill the device), and walks the particle tree once for all
+// of them: 32 consecutive cells of the pre-order at
 // a time, one per lane, are tested against the box around the targets'
 // spheres, and the skip pointers of those outside tell which of the 32 the walk
 // reaches and where it goes on.  The members of the leaves it reaches are read
-// one per lane, those inside the box are staged, and every lane
-// tests its own target against each staged member (a broadcast read), first
+// one per lane, those inside the box are staged, and the lanes of a
+// target test it against their parts of the staged members (broadcast reads), first
 // without branches into a bit mask, then its few candidates by the FP32-filtered
 // exact test with an FP64 fallback.  The walk keeps the first kNbCap neighbours
 // per target; after the scan of the counts the rows are copied into the CSR,
 // and only targets with more neighbours than that walk again, a thread each, to
 // fill their rows.  (One walk per thread for every target, a chain of dependent
 // cell and member reads: 1570 us at 2^20 particles, 157 us at 2 k, where it
-// left most of the chip idle, against 1150 and 54 us.  Tighter boxes, of the
+// left most of the chip idle, against 1150 and 22 us.  Reading the members of the few
+// ranges of the sorted keys that cover the box, with no walk: 1310 and 58 us with a
+// lane per target, where the walk takes 1150 and 54.  Tighter boxes, of the
 // targets' octets, stage fewer members but cost more than they save: 1266 us;
 // of their quads 1560; staging each octet's members apart 1617.  The test as |p|^2
 // + t.p in three FMAs takes more registers than it saves issue: 1417.)
 #include "common.cuh"
+
+#include <type_traits>
 
 namespace st {
 
@@ -64,34 +69,58 @@ __device__ __forceinline__ float nb_reach(float two_h, float cmag)
     return __fadd_rn(__fmul_rn(two_h, 1.f + 1e-5f), __fmul_rn(16.f * kU32, cmag));
 }
 
-// The staged members [0, 32) against the lane's target: its neighbours among
-// them, in order, to its list.  thr: a little above (2 h)^2.
+// The staged members [0, 32) against the group's targets, P lanes each (a lane
+// takes 32 / P of them): the neighbours among them, in order, to the target's
+// list.  thr: a little above (2 h)^2.
+template <int P>
 __device__ __forceinline__ void nb_take(const float4 *buf, float4 pi, float two_h, double two_h64,
-                                        float thr, u32 self, u32 (*list)[33], int lane, u32 &c,
-                                        unsigned &fb)
+                                        float thr, u32 self, u32 (*list)[32 / P + 1], int lane,
+                                        u32 &c, unsigned &fb)
 {
+    const float4 *part = buf + (32 / P) * (lane % P);
     u32 m = 0;
 #pragma unroll
-    for (int k = 0; k < 32; ++k) {
-        const float4 p = buf[k];
+    for (int k = 0; k < 32 / P; ++k) {
+        const float4 p = part[k];
         const float ax = p.x - pi.x, ay = p.y - pi.y, az = p.z - pi.z;
         if (ax * ax + ay * ay + az * az < thr) m |= 1u << k;
     }
-    while (m) {
-        const float4 p = buf[__ffs(m) - 1];
-        m &= m - 1u;
-        const u32 r = __float_as_uint(p.w);
-        if (r != self && member_in(p, pi, two_h, two_h64, fb)) {
-            if (c < kNbCap) list[c][lane] = r;
-            ++c;
+    if (P == 1) {
+        while (m) {
+            const float4 p = part[__ffs(m) - 1];
+            m &= m - 1u;
+            const u32 r = __float_as_uint(p.w);
+            if (r != self && member_in(p, pi, two_h, two_h64, fb)) {
+                if (c < kNbCap) list[c][lane] = r;
+                ++c;
+            }
         }
+        return;
     }
+    u32 in = 0;
+    for (u32 t = m; t; t &= t - 1u) {
+        const int k = __ffs(t) - 1;
+        const float4 p = part[k];
+        if (__float_as_uint(p.w) != self && member_in(p, pi, two_h, two_h64, fb)) in |= 1u << k;
+    }
+    // the target's lanes hold consecutive parts of the members
+    const u32 cnt = (u32)__popc(in);
+    u32 end = cnt;
+#pragma unroll
+    for (int o = 1; o < P; o <<= 1) {
+        const u32 y = __shfl_up_sync(0xffffffffu, end, o, P);
+        if (lane % P >= o) end += y;
+    }
+    for (u32 at = c + end - cnt; in; in &= in - 1u, ++at)
+        if (at < kNbCap) list[at][lane / P] = __float_as_uint(part[__ffs(in) - 1].w);
+    c += __shfl_sync(0xffffffffu, end, P - 1, P);
 }
 
 // Counts every target's neighbours into cnt[i] and keeps the first kNbCap in
 // scratch[i kNbCap ..], in Morton order; n_over counts the targets with more.
 // cells: the first cell of every key (the cells of problem b of a batch are
 // [cells[start b], cells[start b + 1])).
+template <int P>
 __global__ void __launch_bounds__(32 * kNbWarps)
 k_neighbours(const float4 *pq, const float *h, long long np, const float4 *box, const uint4 *meta,
              Segs segs, const u32 *cells, const FrameRec *frames, u32 *cnt,
@@ -99,12 +128,12 @@ k_neighbours(const float4 *pq, const float *h, long long np, const float4 *box, 
 {
     __shared__ float4 buf[kNbWarps][64];      // staged members: position, index
     __shared__ float4 sphere[kNbWarps][32];   // the targets' positions and squared reaches
-    __shared__ u32 list[kNbWarps][kNbCap][33];
+    __shared__ u32 list[kNbWarps][kNbCap][32 / P + 1];
     const float4 far = make_float4(1e30f, 1e30f, 1e30f, 0.f);   // no target's neighbour
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const long long i0 = ((long long)blockIdx.x * kNbWarps + w) * 32;
+    const long long i0 = ((long long)blockIdx.x * kNbWarps + w) * (32 / P);
     if (i0 >= np) return;   // warp-uniform
-    const long long i = i0 + lane;
+    const long long i = i0 + lane / P;
     const bool live = i < np;
     float4 pi = make_float4(0.f, 0.f, 0.f, 0.f);
     float two_h = 0.f;
@@ -163,7 +192,7 @@ k_neighbours(const float4 *pq, const float *h, long long np, const float4 *box, 
                       __fadd_rn(b.z, b.w) >= lo[2];
                 if (wide && hit) {
                     hit = false;
-                    for (int t = 0; t < 32 && !hit; ++t) {
+                    for (int t = 0; t < 32 && !hit; t += P) {
                         const float4 p = sphere[w][t];
                         hit = cell_d2(b, p.x, p.y, p.z) <= p.w;
                     }
@@ -211,7 +240,7 @@ k_neighbours(const float4 *pq, const float *h, long long np, const float4 *box, 
                 staged += __popc(nm);
                 __syncwarp();
                 if (staged >= 32) {
-                    nb_take(buf[w], pi, two_h, two_h64, thr, (u32)i, list[w], lane, c, fb);
+                    nb_take<P>(buf[w], pi, two_h, two_h64, thr, (u32)i, list[w], lane, c, fb);
                     __syncwarp();
                     staged -= 32;
                     if (lane < staged) buf[w][lane] = buf[w][32 + lane];
@@ -222,19 +251,19 @@ k_neighbours(const float4 *pq, const float *h, long long np, const float4 *box, 
         if (staged) {
             if (lane >= staged) buf[w][lane] = far;
             __syncwarp();
-            nb_take(buf[w], pi, two_h, two_h64, thr, (u32)i, list[w], lane, c, fb);
+            nb_take<P>(buf[w], pi, two_h, two_h64, thr, (u32)i, list[w], lane, c, fb);
             __syncwarp();
         }
     }
-    if (live) cnt[i] = c;
+    if (live && lane % P == 0) cnt[i] = c;
     __syncwarp();
     // the rows, one after the other, lanes along the row
-    const int rows = (int)min(32ll, np - i0);
+    const int rows = (int)min((long long)(32 / P), np - i0);
     for (int t = 0; t < rows; ++t) {
-        const u32 m = min(kNbCap, __shfl_sync(0xffffffffu, c, t));
+        const u32 m = min(kNbCap, __shfl_sync(0xffffffffu, c, t * P));
         for (u32 k = lane; k < m; k += 32) scratch[(size_t)(i0 + t) * kNbCap + k] = list[w][k][t];
     }
-    const unsigned over = __ballot_sync(0xffffffffu, live && c > kNbCap);
+    const unsigned over = __ballot_sync(0xffffffffu, live && lane % P == 0 && c > kNbCap);
     for (int o = 16; o; o >>= 1) fb += __shfl_xor_sync(0xffffffffu, fb, o);
     if (lane == 0) {
         if (over) atomicAdd(n_over, (unsigned long long)__popc(over));
@@ -334,9 +363,21 @@ int build_neighbours(start_ctx *c, const Segs &segs, const FrameRec *frames)
     unsigned long long *n_over = ctr + C_NB_OVER;
     ST_CUDA(c, cudaMemsetAsync(n_over, 0, sizeof(unsigned long long), c->stream));
     const Tree &t = c->pt;
-    k_neighbours<<<grid_for(np, 32 * kNbWarps), 32 * kNbWarps, 0, c->stream>>>(
-        c->pq.as<float4>(), c->ph.as<float>(), np, t.box.as<float4>(), t.meta.as<uint4>(), segs,
-        t.pos.as<u32>(), frames, c->lcount.as<u32>(), fb, scratch.as<u32>(), n_over);
+    auto search = [&](auto lanes) {
+        constexpr int P = decltype(lanes)::value;
+        k_neighbours<P><<<grid_for(np, 32 / P * kNbWarps), 32 * kNbWarps, 0, c->stream>>>(
+            c->pq.as<float4>(), c->ph.as<float>(), np, t.box.as<float4>(), t.meta.as<uint4>(),
+            segs, t.pos.as<u32>(), frames, c->lcount.as<u32>(), fb, scratch.as<u32>(), n_over);
+    };
+    // lanes per target: where a lane each leaves warps' slots empty, more and
+    // shorter walks.  us with 1 / 2 / 8 / 16 lanes: 53 / 38 / 26 / 22 at 2 k particles,
+    // 99 / 59 / 40 / 33 at 8 k, 107 / 87 / 61 / 66 at 16 k, 110 / 92 / 65 / 72 at 23 k,
+    // 114 / 90 / 86 / 106 at 43 k, 166 / 122 / 144 / - at 65 k, 254 / 252 / 326 / - at
+    // 160 k, 304 / 313 / 445 / - at 262 k
+    if (np <= 12288) search(std::integral_constant<int, 16>());
+    else if (np <= 40960) search(std::integral_constant<int, 8>());
+    else if (np <= 200000) search(std::integral_constant<int, 2>());
+    else search(std::integral_constant<int, 1>());
     ++c->launches;
     ST_CUDA(c, cudaGetLastError());
     // offsets in u64 first to detect overflow of the u32 CSR
