@@ -35,6 +35,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -892,40 +893,48 @@ __device__ __forceinline__ u32 link_or_claim(const MemoArgs &a, u32 vid, u32 up,
     return kNone;
 }
 
-// One thread follows one chain (hop<1>, then the link search and claim);
-// a chain per thread keeps many chains in flight, which matters more here
-// than a shorter neighbour scan per link (cooperative groups of eight lanes
-// per chain measured slower: 1.0 ms against 0.73 ms per step on the 64^3,
-// 1024-source workload).
+// G lanes follow one chain: the hop together, the link search and claim by
+// the first.  Many chains fill the device with a lane each, and more lanes then
+// slow them down; few are bound by the latency of a chain's hops, which
+// more lanes shorten.
+template <int G>
 __global__ void __launch_bounds__(128) k_memo_tail(MemoArgs a, long long max_iter)
 {
-    const long long it = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long it = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / G;
     if (it >= a.nf) return;
-    const unsigned me = 1u << (threadIdx.x & 31);
+    const int lane = threadIdx.x & 31, gl = lane % G;
+    const unsigned gmask = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << (lane - gl);
     unsigned long long fbs = 0;
     u32 s = a.fbase + (u32)it;
+    const u32 vid = a.svid[s], key = a.sord[s];
+    const float4 src = vsource(a, vid);
+    u32 j = a.sj[s];
     for (long long n = 0;; ++n) {
         if (n > max_iter) {
-            atomicAdd(&a.m.counters[C_TAIL_CAP], 1ull);
+            if (gl == 0) atomicAdd(&a.m.counters[C_TAIL_CAP], 1ull);
             break;
         }
-        const u32 vid = a.svid[s], j = a.sj[s];
-        const float4 src = vsource(a, vid);
         float dt, dl;
-        const u32 up = hop<1>(a.m, j, a.m.pq[j], src, 0, me, dt, fbs, &dl);
-        u32 nx = kNone, hpend = 0;
-        bool claimed = false;
-        if (up != kNone) nx = link_or_claim(a, vid, up, a.sord[s], claimed, hpend);
-        // a pending link's table index at the slot's position after fbase
-        // (k_memo_resolve then runs over the slots from fbase on)
-        if (nx == kPendMark) a.ups[s - a.fbase] = hpend;
-        a.state[s] = make_uint2(nx, __float_as_uint(dt));
-        if (a.dl) a.dl[s] = dl;
-        if (a.nx0) a.nx0[s] = nx;
-        if (!claimed) break;
-        s = nx;
+        const u32 up = hop<G>(a.m, j, a.m.pq[j], src, gl, gmask, dt, fbs, &dl);
+        u32 next = kNone;   // the slot claimed here, if any
+        if (gl == 0) {
+            u32 nx = kNone, hpend = 0;
+            bool claimed = false;
+            if (up != kNone) nx = link_or_claim(a, vid, up, key, claimed, hpend);
+            // a pending link's table index at the slot's position after fbase
+            // (k_memo_resolve then runs over the slots from fbase on)
+            if (nx == kPendMark) a.ups[s - a.fbase] = hpend;
+            a.state[s] = make_uint2(nx, __float_as_uint(dt));
+            if (a.dl) a.dl[s] = dl;
+            if (a.nx0) a.nx0[s] = nx;
+            if (claimed) next = nx;
+        }
+        if (G > 1) next = __shfl_sync(gmask, next, 0, G);
+        if (next == kNone) break;
+        s = next;
+        j = up;
     }
-    if (fbs) atomicAdd(&a.m.counters[C_MARCH_FB], fbs);
+    if (gl == 0 && fbs) atomicAdd(&a.m.counters[C_MARCH_FB], fbs);
 }
 
 // Chain links of the march: the slots allocated, which the host reads only
@@ -1658,7 +1667,17 @@ static int memo_attempt(start_ctx *c, const MarchArgs &m, float theta, size_t ca
             // the remaining levels in one launch, then the pending links
             a.dlv = nullptr;
             ev(0);
-            k_memo_tail<<<grid_for(a.nf, 128), 128, 0, s>>>(a, max_iter - iter);
+            auto tail = [&](auto lanes) {
+                constexpr int G = decltype(lanes)::value;
+                k_memo_tail<G><<<grid_for(a.nf * G, 128), 128, 0, s>>>(a, max_iter - iter);
+            };
+            // us with 1 / 2 / 8 / 16 lanes a chain: 70 / 52 / 34 / 29 for 1.3 k chains,
+            // 98 / 76 / 54 / 63 for 12 k, 129 / 98 / 90 / 107 for 22 k, 120 / 98 / 137 / 171
+            // for 72 k, 137 / 153 / 261 / 336 for 115 k, 292 / 314 / 615 / 839 for 233 k
+            if (a.nf <= 8192) tail(std::integral_constant<int, 16>());
+            else if (a.nf <= 24576) tail(std::integral_constant<int, 8>());
+            else if (a.nf <= 81920) tail(std::integral_constant<int, 2>());
+            else tail(std::integral_constant<int, 1>());
             ev(1);
             ++c->launches;
             ST_CUDA(c, cudaGetLastError());

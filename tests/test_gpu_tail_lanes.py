@@ -1,0 +1,38 @@
+"""The last levels of the chains with 16, 8, 2 and 1 lanes per chain (a request's
+frontier of about 0.6, 4.6, 18, 56 and 120 k chains): chain lengths and Gamma
+against the per-ray march, which shares neither the links nor their search."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("row_bins", [0, 4])
+@pytest.mark.parametrize("n_p,n_s", [(33, 1), (700, 20), (2048, 64), (12000, 64), (16384, 200),
+                                     (23000, 429)])
+def test_tail_matches_the_ray_march(n_p, n_s, row_bins):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1005_5312_gb300 as S
+    S.build()
+    rng = np.random.default_rng(n_p)
+    pos = rng.uniform(0.0, 1.0, (3, n_p)).astype(np.float32)
+    h = np.full(n_p, 0.985 * n_p ** (-1.0 / 3.0), np.float32)
+    src = rng.uniform(0.0, 1.0, (3, n_s)).astype(np.float32)
+    L = rng.lognormal(0.0, 1.0, n_s) * 1e48
+    n_HI = rng.uniform(0.0, 2.0, n_p).astype(np.float32)
+    out = []
+    for mode in (1, 0):
+        ctx = S.Context(march_mode=mode, link_counts=mode, row_bins=row_bins, tau_cut=1e30,
+                        sigma_cm2=1.0, len_unit_cm=1.0)
+        ctx.build_trees(pos, h, src, L)
+        g = np.zeros(n_p, np.float32)
+        ctx.rt_solve(0.7, n_HI=n_HI, gamma_out=g)
+        out.append((g.astype(np.float64), ctx.stats()))
+    (gm, sm), (gr, sr) = out
+    assert sm["rays"] == sr["rays"]
+    assert sm["hops"] == sr["hops"] and sm["max_hops"] == sr["max_hops"]
+    # compensated sums of the same links both ways: a few roundings of tau (below
+    # 4) and of each contribution
+    np.testing.assert_allclose(gm, gr, rtol=2e-5)
