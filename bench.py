@@ -291,12 +291,14 @@ def phase_models(st, n_p, n_s, diffuse, chunk_count):
     nb = st["nbr_total"]
     nodes = st["nodes_part"] + st["nodes_src"] + (st["nodes_emit"] if diffuse else 0)
     return {
-        # frame, keys, 8 radix passes (key + index in and out), octree records,
-        # neighbour search (its CSR written) and the records of the particles
-        "build": {"kernels": "k_bbox, k_morton, k_rs_*, k_level_census, octree levels, "
-                             "k_moments_*, k_neighbours, k_nb_compact",
-                  "bytes": n_p * (12 + 4 + 8 + 8 * 24 + 16 + 8) + nb * 4 + nodes * 64,
-                  "model": "per particle: position, h, key, 8 radix passes x 24 B, record, CSR "
+        # frame, keys, 4 radix passes over the leading bits (key + index in and
+        # out), octree records, neighbour search (its CSR written) and the
+        # records of the particles
+        "build": {"kernels": "k_bbox, k_morton, k_rs_*, k_sort_runs, k_rank_sort, "
+                             "k_tree_census, k_tree_emit, k_moments_*, k_neighbours<P>, "
+                             "k_nb_compact",
+                  "bytes": n_p * (12 + 4 + 8 + 4 * 24 + 16 + 8) + nb * 4 + nodes * 64,
+                  "model": "per particle: position, h, key, 4 radix passes x 24 B, record, CSR "
                            "offsets; 4 B per neighbour; 64 B per octree node"},
         "density": {"kernels": "k_mass_to_morton, k_sph_density",
                     "bytes": n_p * 36 + nb * 24,
@@ -311,7 +313,7 @@ def phase_models(st, n_p, n_s, diffuse, chunk_count):
                  "bytes": rays * 12 + n_p * 16 * chunk_count,
                  "model": "per pair 12 B (canonical id written, read, order key written); per "
                           "target and walk its 16 B record"},
-        "hops": {"kernels": "k_memo_hop_rows, k_memo_hop_hard, k_memo_hop<G>, k_memo_tail",
+        "hops": {"kernels": "k_memo_hop_rows, k_memo_hop_hard, k_memo_hop<G>, k_memo_tail<G>",
                  "bytes": links * 32 + off * ALGO_BYTES_PER_EVAL + n_p * chunk_count * 676,
                  "model": "per chain link 32 B (id, order key and its direction bin's candidate "
                           "mask read; state (next, d_tau), length and next written); per link "
@@ -321,14 +323,15 @@ def phase_models(st, n_p, n_s, diffuse, chunk_count):
                  "bytes": off * 56 + rays * 8,
                  "model": "per link outside the lists 56 B (upstream, id, key, table entry, "
                           "claimed slot, next written); per pair 8 B (row search)"},
-        "jump": {"kernels": "k_memo_jump8<3, 12>",
-                 "bytes": st["jump_bytes"],
-                 "model": "8 B own state (next, FP32 sum) per slot and round; 16 B per slot "
-                          "that advances (first successor read and the write); 8 B per further "
-                          "successor read; 8 B per closed chain copied once"},
-        "gamma": {"kernels": "k_memo_gamma",
-                  "bytes": rays * 12 + n_p * 8,
-                  "model": "per pair 12 B (8-byte chain state, id); per target 8 B"},
+        # one count for both: the Gamma sum follows the chains that the last
+        # round leaves open
+        "jump+gamma": {"kernels": "k_memo_jump8<3, 12>, k_memo_gamma",
+                       "bytes": st["jump_bytes"] + rays * 12 + n_p * 8,
+                       "model": "8 B own state (next, FP32 sum) per slot and round; 16 B per "
+                                "slot that advances (first successor read and the write); 8 B "
+                                "per further successor read and per state of an open chain "
+                                "read by the Gamma sum; 8 B per closed chain copied once; per "
+                                "pair 12 B (8-byte chain state, id); per target 8 B"},
         "ionize": {"kernels": "k_ionize",
                    "bytes": n_p * (36 if diffuse else 28),
                    "model": "per particle: y read and written (16), Gamma (4), n_H (4), n_HI "
@@ -339,9 +342,10 @@ def phase_models(st, n_p, n_s, diffuse, chunk_count):
 def kernel_table(phase_ms, models, step_ms, peak):
     rows = []
     for name, m in models.items():
-        ms = phase_ms.get(name)
-        if ms is None or ms < 0:
+        parts = [phase_ms.get(p) for p in name.split("+")]
+        if any(p is None or p < 0 for p in parts):
             continue
+        ms = sum(parts)
         gbs = m["bytes"] / (ms * 1e-3) / 1e9 if ms > 0 else 0.0
         rows.append({"phase": name, "kernels": m["kernels"], "ms_per_step": ms,
                      "share_of_step": ms / step_ms, "algorithmic_bytes_per_step": m["bytes"],

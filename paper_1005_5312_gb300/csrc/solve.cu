@@ -1228,7 +1228,7 @@ static int run_grouped(start_ctx *c, float theta, float *gout_dev, long long max
     if (h.empty()) ST_TRY(group_histogram(c, theta, h));
     const unsigned long long SN = (unsigned long long)c->stree.n;
     const unsigned long long NT = SN + (unsigned long long)(c->walk_emit ? c->et.n : 0);
-    // bins [b0, b1) of each group, about 0.8 max_pairs each by the sample
+    // bins [b0, b1) of each group, about 0.9 max_pairs each by the sample
     std::vector<std::pair<int, int>> groups;
     {
         const double target = 0.9 * (double)maxp;
