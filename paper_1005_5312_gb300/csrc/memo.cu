@@ -1028,6 +1028,14 @@ constexpr int kJumpR8 = 12;  // 8-byte form: slots per thread
 // 1.7 M x 500 (0.999) and 7.2 against 4.5 ms on 128^3 x 64 (0.9998; a third
 // round, 0.979 open after the second, 4.9 ms).
 constexpr double kJumpOpen = 0.995;
+// Chains lengthen with the particles along the box while the share left open by
+// the first round hardly moves, and the long ones hold up their warps' sums: above
+// kJumpMany particles a second round runs while more than kJumpOpenMany is open.
+// One round against two, every particle emitting: 125 against 140 ms on 128^3
+// (0.87 open), 296 / 307 on 160^3 (0.86), 594 / 575 on 192^3 (0.86), 181 / 172 on
+// 192^3 at theta = 1 (0.79), 2.46 / 1.83 s on 256^3 (0.84).
+constexpr long long kJumpMany = 6000000;
+constexpr double kJumpOpenMany = 0.6;
 constexpr int kGammaU = 3;   // pairs per lane in flight in the rows of a group
 
 // The march's states widened for the counting form: one link, no
@@ -1769,7 +1777,10 @@ static int memo_attempt(start_ctx *c, const MarchArgs &m, float theta, size_t ca
         jc[0] = v[C_JUMP_MOVED];
         jc[1] = v[C_JUMP_LEFT];
         nslots = (long long)v[C_SLOTS];
-        if (!wide) few = (unsigned long long)(kJumpOpen * (double)nslots);
+        if (!wide) {
+            const bool many = round == 0 && c->np > kJumpMany;
+            few = (unsigned long long)((many ? kJumpOpenMany : kJumpOpen) * (double)nslots);
+        }
         if (timing) {
             float ms = 0.f;
             if (cudaEventElapsedTime(&ms, c->hev[0], c->hev[1]) == cudaSuccess) jump_ms += ms;
