@@ -835,7 +835,7 @@ __global__ void __launch_bounds__(256) k_memo_link(MemoArgs a)
     }
 }
 
-// 2c. the last levels, once the frontier is small: each thread takes one
+// 2c. the last levels, once the frontier is small: each group of lanes takes one
 // frontier slot and follows its chain itself -- the hop, then the upstream
 // link in its row or the table; a link it claims becomes its next slot -- so
 // the remaining levels need no launch and no host round trip each.  Links
